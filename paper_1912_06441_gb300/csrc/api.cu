@@ -55,136 +55,117 @@ labfm_status cuda_fail(labfm_ctx *ctx, cudaError_t e, const char *where)
 }
 
 // ---------------------------------------------------------------------------------------------
-// Exclusive scan (Blelloch-style in shared memory, recursive over block sums).
+// Exclusive scan of int32 counts into int64 offsets, out[n] the total.  One launch up to SCAN_ITEMS elements; beyond,
+// the sums of the blocks' runs first, then every block adds up the sums before its own (up to SCAN_DIRECT blocks:
+// 8 bytes each from L2, less than the launches that scanning them would take; above, they are scanned by a
+// recursion) and scans its run.  Two launches for what took four; a small search is mostly launches.
 // ---------------------------------------------------------------------------------------------
 constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_ITEMS = 2 * SCAN_THREADS;
+constexpr int64_t SCAN_DIRECT = 4096;
+
+// Sum over the block, on every thread.
+__device__ __forceinline__ int64_t scan_block_sum(int64_t v, int64_t *sh)
+{
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = sh[threadIdx.x & 31];  // SCAN_THREADS / 32 = 32 warps
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();  // sh is free again
+    return v;
+}
 
 template <class Tin>
-__global__ void k_scan_block(const Tin *__restrict__ in, int64_t *__restrict__ out, int64_t n,
-                             int64_t *__restrict__ block_sums)
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_sums(const Tin *__restrict__ in, int64_t n, int64_t *__restrict__ sums)
 {
-    __shared__ int64_t s[SCAN_ITEMS];
-    int64_t base = (int64_t)blockIdx.x * SCAN_ITEMS;
-    int t = threadIdx.x;
-    for (int u = 0; u < 2; u++) {
-        int64_t g = base + t + u * SCAN_THREADS;
-        s[t + u * SCAN_THREADS] = g < n ? (int64_t)in[g] : 0;
-    }
-    __syncthreads();
-    // up-sweep
-    for (int d = 1; d < SCAN_ITEMS; d <<= 1) {
-        int idx = (t + 1) * 2 * d - 1;
-        if (idx < SCAN_ITEMS) s[idx] += s[idx - d];
-        __syncthreads();
-    }
-    if (t == 0) {
-        if (block_sums) block_sums[blockIdx.x] = s[SCAN_ITEMS - 1];
-        s[SCAN_ITEMS - 1] = 0;
-    }
-    __syncthreads();
-    // down-sweep
-    for (int d = SCAN_ITEMS >> 1; d >= 1; d >>= 1) {
-        int idx = (t + 1) * 2 * d - 1;
-        if (idx < SCAN_ITEMS) {
-            int64_t v = s[idx - d];
-            s[idx - d] = s[idx];
-            s[idx] += v;
-        }
-        __syncthreads();
-    }
-    for (int u = 0; u < 2; u++) {
-        int64_t g = base + t + u * SCAN_THREADS;
-        if (g < n) out[g] = s[t + u * SCAN_THREADS];
-    }
+    __shared__ int64_t sh[32];
+    const int64_t g = (int64_t)blockIdx.x * SCAN_ITEMS + threadIdx.x;
+    int64_t v = g < n ? (int64_t)in[g] : 0;
+    if (g + SCAN_THREADS < n) v += (int64_t)in[g + SCAN_THREADS];
+    v = scan_block_sum(v, sh);
+    if (threadIdx.x == 0) sums[blockIdx.x] = v;
 }
 
-__global__ void k_scan_add(int64_t *__restrict__ out, int64_t n, const int64_t *__restrict__ block_offsets)
+// sums: the sums of the blocks' runs, or with `scanned` their exclusive scan; null for a single block
+template <class Tin>
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const Tin *__restrict__ in, int64_t *__restrict__ out, int64_t n,
+                                                             const int64_t *__restrict__ sums, int scanned)
 {
-    int64_t g = (int64_t)blockIdx.x * SCAN_ITEMS + threadIdx.x;
-    int64_t add = block_offsets[blockIdx.x];
-    if (g < n) out[g] += add;
-    if (g + SCAN_THREADS < n) out[g + SCAN_THREADS] += add;
+    __shared__ int64_t sh[32];
+    int64_t before = 0;  // the sum of all earlier blocks' runs
+    if (sums && scanned) {
+        before = sums[blockIdx.x];
+    } else if (sums) {
+        for (int64_t b = threadIdx.x; b < blockIdx.x; b += SCAN_THREADS) before += sums[b];
+        before = scan_block_sum(before, sh);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t g = (int64_t)blockIdx.x * SCAN_ITEMS + 2 * threadIdx.x;
+    const int64_t a = g < n ? (int64_t)in[g] : 0, b = g + 1 < n ? (int64_t)in[g + 1] : 0;
+    int64_t v = a + b;  // inclusive scan of the threads' pairs
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t w = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += w;
+    }
+    if (lane == 31) sh[warp] = v;
+    __syncthreads();
+    int64_t ws = lane < warp ? sh[lane] : 0;
+    for (int o = 16; o > 0; o >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, o);
+    const int64_t at = before + ws + v - (a + b);
+    if (g < n) out[g] = at;
+    if (g + 1 < n) out[g + 1] = at + a;
+    if (g < n && g + 2 >= n) out[n] = at + a + b;  // the thread of the last element
 }
 
-__global__ void k_scan_total(const int64_t *__restrict__ out_excl, const int64_t *__restrict__ last_in_i64,
-                             const int32_t *__restrict__ last_in_i32, int64_t n, int64_t *__restrict__ total)
-{
-    if (n == 0) {
-        *total = 0;
-        return;
-    }
-    int64_t last = last_in_i64 ? last_in_i64[n - 1] : (int64_t)last_in_i32[n - 1];
-    *total = out_excl[n - 1] + last;
-}
+__global__ void k_scan_empty(int64_t *out) { out[0] = 0; }
 
 template <class Tin>
 static cudaError_t scan_rec(const Tin *in, int64_t *out, int64_t n, int64_t *tmp, cudaStream_t s)
 {
-    int64_t nb = (n + SCAN_ITEMS - 1) / SCAN_ITEMS;
-    if (nb <= 1) {
-        k_scan_block<Tin><<<1, SCAN_THREADS, 0, s>>>(in, out, n, nullptr);
-        return cudaGetLastError();
+    const int64_t nb = (n + SCAN_ITEMS - 1) / SCAN_ITEMS;
+    int64_t *sums = nullptr;
+    if (nb > 1) {
+        sums = tmp;
+        k_scan_sums<Tin><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, sums);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (nb > SCAN_DIRECT) {
+            int64_t *scanned = tmp + nb;  // nb + 1 elements
+            if ((e = scan_rec<int64_t>(sums, scanned, nb, tmp + 2 * nb + 1, s)) != cudaSuccess) return e;
+            sums = scanned;
+        }
     }
-    int64_t *sums = tmp;
-    int64_t *sums_scanned = tmp + nb;
-    k_scan_block<Tin><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, sums);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    e = scan_rec<int64_t>(sums, sums_scanned, nb, tmp + 2 * nb, s);
-    if (e != cudaSuccess) return e;
-    k_scan_add<<<(unsigned)nb, SCAN_THREADS, 0, s>>>(out, n, sums_scanned);
+    k_scan_apply<Tin><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, sums, nb > SCAN_DIRECT ? 1 : 0);
     return cudaGetLastError();
 }
 
-static size_t scan_tmp_elems(int64_t n)
+size_t scan_workspace_elems(int64_t n)
 {
     size_t tot = 0;
     while (true) {
         int64_t nb = (n + SCAN_ITEMS - 1) / SCAN_ITEMS;
         if (nb <= 1) break;
-        tot += 2 * nb;
+        tot += 2 * nb + 1;
         n = nb;
     }
     return tot + 16;
 }
 
-cudaError_t exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, DevBuf &tmp, cudaStream_t s)
+cudaError_t exclusive_scan_i32_to_i64_ws(const int32_t *in, int64_t *out, int64_t n, int64_t *tmp, size_t tmp_elems,
+                                         cudaStream_t s)
 {
-    cudaError_t e = tmp.reserve(scan_tmp_elems(n) * sizeof(int64_t));
-    if (e != cudaSuccess) return e;
-    if (n > 0) {
-        e = scan_rec<int64_t>(in, out, n, tmp.as<int64_t>(), s);
-        if (e != cudaSuccess) return e;
-    }
-    k_scan_total<<<1, 1, 0, s>>>(out, in, nullptr, n, out + n);
+    if (scan_workspace_elems(n) > tmp_elems) return cudaErrorInvalidValue;
+    if (n > 0) return scan_rec<int32_t>(in, out, n, tmp, s);
+    k_scan_empty<<<1, 1, 0, s>>>(out);
     return cudaGetLastError();
 }
 
 cudaError_t exclusive_scan_i32_to_i64(const int32_t *in, int64_t *out, int64_t n, DevBuf &tmp, cudaStream_t s)
 {
-    cudaError_t e = tmp.reserve(scan_tmp_elems(n) * sizeof(int64_t));
-    if (e != cudaSuccess) return e;
-    if (n > 0) {
-        e = scan_rec<int32_t>(in, out, n, tmp.as<int64_t>(), s);
-        if (e != cudaSuccess) return e;
-    }
-    k_scan_total<<<1, 1, 0, s>>>(out, nullptr, in, n, out + n);
-    return cudaGetLastError();
-}
-
-size_t scan_workspace_elems(int64_t n) { return scan_tmp_elems(n); }
-
-cudaError_t exclusive_scan_i32_to_i64_ws(const int32_t *in, int64_t *out, int64_t n, int64_t *tmp, size_t tmp_elems,
-                                         cudaStream_t s)
-{
-    if (scan_tmp_elems(n) > tmp_elems) return cudaErrorInvalidValue;
-    if (n > 0) {
-        cudaError_t e = scan_rec<int32_t>(in, out, n, tmp, s);
-        if (e != cudaSuccess) return e;
-    }
-    k_scan_total<<<1, 1, 0, s>>>(out, nullptr, in, n, out + n);
-    return cudaGetLastError();
+    const size_t elems = scan_workspace_elems(n);
+    cudaError_t e = tmp.reserve(elems * sizeof(int64_t));
+    return e == cudaSuccess ? exclusive_scan_i32_to_i64_ws(in, out, n, tmp.as<int64_t>(), elems, s) : e;
 }
 
 }  // namespace labfm

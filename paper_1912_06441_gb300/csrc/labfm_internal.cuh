@@ -111,8 +111,7 @@ namespace labfm {
 labfm_status fail(labfm_ctx *ctx, labfm_status st, const std::string &msg);
 labfm_status cuda_fail(labfm_ctx *ctx, cudaError_t e, const char *where);
 
-// Exclusive prefix sum of in[0..n) (int64) into out[0..n]; out[n] = total.  `tmp` is scratch.
-cudaError_t exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, DevBuf &tmp, cudaStream_t s);
+// Exclusive prefix sum of in[0..n) into out[0..n]; out[n] = total.  `tmp` is scratch.
 cudaError_t exclusive_scan_i32_to_i64(const int32_t *in, int64_t *out, int64_t n, DevBuf &tmp, cudaStream_t s);
 // The same scan on a caller-provided workspace of tmp_elems int64 (at least scan_workspace_elems(n)).
 size_t scan_workspace_elems(int64_t n);

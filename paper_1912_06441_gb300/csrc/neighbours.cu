@@ -2,9 +2,9 @@
 //
 // Cells have side >= 2 h_max, so every neighbour of a node lies in its own cell or one of
 // the 8 cells around it (with wrap-around in a periodic box).  Nodes are counting-sorted by
-// cell; one thread per node (in cell order, so a warp sweeps the same few cells) counts its
-// neighbours, a prefix sum gives the CSR row pointers, a second sweep writes the column
-// indices, and each row is sorted ascending.  The distance test is evaluated in IEEE double
+// cell; one warp per node (in cell order, so the warps of a block sweep the same few cells) counts its
+// neighbours, a prefix sum gives the CSR row pointers, and a second sweep collects each row in shared
+// memory, sorts it in registers and writes it whole.  The distance test is evaluated in IEEE double
 // with explicitly rounded operations (no fused multiply-add), so the result does not depend
 // on the compiler's contraction choices; a float pre-classification with a proven error bound
 // settles every candidate that is not within a thin shell at the radius (on GB300 the double
@@ -20,6 +20,7 @@ namespace labfm {
 namespace {
 
 constexpr int NB_THREADS = 256;
+constexpr int ROW_MAX = 128;  // entries of a row that a warp sorts in registers
 
 struct Grid {
     double lo[2], L[2], halfL[2], inv_cs[2];
@@ -36,9 +37,11 @@ struct Grid {
 
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
 
-// Validate nodes and find max h.  misc[0] = bits of max h, misc[1] = number of bad nodes.
+// Validate nodes and find max h.  misc[0] = bits of max h, misc[1] = number of bad nodes.  The context's copies of
+// the positions and h are written on the way (xy_out, h_out; null: no copies).
 __global__ void k_check(int64_t n, const double *__restrict__ xy, const double *__restrict__ h, double lo0, double lo1,
-                        double hi0, double hi1, unsigned long long *__restrict__ misc)
+                        double hi0, double hi1, unsigned long long *__restrict__ misc, double2 *__restrict__ xy_out,
+                        double *__restrict__ h_out)
 {
     __shared__ unsigned long long s_max[NB_THREADS / 32];
     __shared__ unsigned int s_bad[NB_THREADS / 32];
@@ -46,6 +49,10 @@ __global__ void k_check(int64_t n, const double *__restrict__ xy, const double *
     unsigned int bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         double x = xy[2 * i], y = xy[2 * i + 1], hv = h[i];
+        if (xy_out) {
+            xy_out[i] = make_double2(x, y);
+            h_out[i] = hv;
+        }
         bool ok = isfinite(x) && isfinite(y) && isfinite(hv) && hv > 0.0 && x >= lo0 && x <= hi0 && y >= lo1 &&
                   y <= hi1;
         if (!ok) bad++;
@@ -79,7 +86,7 @@ __device__ __forceinline__ int cell_coord(double x, double lo, double inv_cs, in
 }
 
 __global__ void k_cell_assign(int64_t n, const double *__restrict__ xy, Grid g, int32_t *__restrict__ cell_of,
-                              int32_t *__restrict__ cell_count)
+                              int32_t *__restrict__ cell_count, int32_t *__restrict__ rank)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -87,18 +94,18 @@ __global__ void k_cell_assign(int64_t n, const double *__restrict__ xy, Grid g, 
     int cy = cell_coord(xy[2 * i + 1], g.lo[1], g.inv_cs[1], g.nc[1]);
     int c = cy * g.nc[0] + cx;
     cell_of[i] = c;
-    atomicAdd(&cell_count[c], 1);
+    rank[i] = atomicAdd(&cell_count[c], 1);  // the node's place within its cell
 }
 
 __global__ void k_cell_scatter(int64_t n, const double *__restrict__ xy, const int32_t *__restrict__ cell_of,
-                               const int64_t *__restrict__ cell_start, int32_t *__restrict__ cursor,
+                               const int64_t *__restrict__ cell_start, const int32_t *__restrict__ rank,
                                int32_t *__restrict__ cell_nodes, double2 *__restrict__ cell_xy,
                                float2 *__restrict__ cell_xyf)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int c = cell_of[i];
-    int64_t pos = cell_start[c] + atomicAdd(&cursor[c], 1);
+    int64_t pos = cell_start[c] + rank[i];
     cell_nodes[pos] = (int32_t)i;
     const double x = xy[2 * i], y = xy[2 * i + 1];
     cell_xy[pos] = make_double2(x, y);
@@ -138,7 +145,69 @@ __device__ __forceinline__ bool within_exact(double qx, double qy, double xi, do
     return r2 < R2;
 }
 
-// One sweep over the candidate cells of node i.  WRITE = false: count; true: write col[].
+// Ascending sort of a warp's row of cnt <= 32 E entries from shared memory, element e 32 + lane in register e of
+// lane (a bitonic network; exchanges of partners 32 or more apart stay within a lane), then the row to out.
+template <int E>
+__device__ __forceinline__ void sort_row(const int32_t *buf, int cnt, int lane, int32_t *__restrict__ out)
+{
+    int v[E];
+#pragma unroll
+    for (int e = 0; e < E; e++) v[e] = 32 * e + lane < cnt ? buf[32 * e + lane] : 0x7fffffff;
+#pragma unroll
+    for (int k = 2; k <= 32 * E; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= 32) {
+#pragma unroll
+                for (int e = 0; e < E; e++) {
+                    const int f = e ^ (j / 32);
+                    if (f > e) {
+                        const bool up = ((32 * e) & k) == 0;  // k > 32 here, or all of them up at the last k
+                        const int a = min(v[e], v[f]), b = max(v[e], v[f]);
+                        v[e] = up ? a : b;
+                        v[f] = up ? b : a;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; e++) {
+                    const int o = __shfl_xor_sync(0xffffffffu, v[e], j);
+                    const bool up = ((32 * e + lane) & k) == 0;
+                    v[e] = (((lane & j) == 0) == up) ? min(v[e], o) : max(v[e], o);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < E; e++)
+        if (32 * e + lane < cnt) out[32 * e + lane] = v[e];
+}
+
+// Ascending sort of a longer row in place in global memory by one warp: the bitonic network whose exchanges all
+// put the smaller entry first, so that entries from cnt on may be taken as larger than any and left out.
+__device__ __noinline__ void sort_long_row(int32_t *row, int cnt, int lane)
+{
+    for (int64_t k = 2; (k >> 1) < cnt; k <<= 1) {
+        for (int64_t j = k >> 1; j > 0; j >>= 1) {
+            __syncwarp();
+            const int64_t flip = j == (k >> 1) ? k - 1 : j;
+            for (int64_t a = lane; a < cnt; a += 32) {
+                const int64_t b = a ^ flip;
+                if (b > a && b < cnt && row[a] > row[b]) {
+                    const int32_t t = row[a];
+                    row[a] = row[b];
+                    row[b] = t;
+                }
+            }
+        }
+    }
+}
+
+// One sweep over the candidate cells of a node, one warp per node.  WRITE = false: count; true: write col[].
+// The candidates of a row of cells lie one behind another in cell order, so a node's up to nine cells are three runs
+// of nodes (six where the row wraps around), which the warp takes 32 candidates at a time; a ballot gives the
+// hits' places.  With a thread per node instead, the rows were sorted by insertion in global memory, which took
+// most of the search.
 // With cell_xyf, each candidate is first classified in float: r2f, the squared distance from
 // the float coordinates, differs from the double r2 by at most D = 2E(|dx_f| + |dy_f|) + 2E^2 +
 // 2^-23 r2f (E bounds the error of dx_f and dy_f); a candidate with r2f below or above
@@ -146,37 +215,65 @@ __device__ __forceinline__ bool within_exact(double qx, double qy, double xi, do
 // radius) takes the double test.  The result is the double test's, bit for bit; on GB300 the
 // double test costs FP64-pipe time per candidate, the float one does not.
 template <bool WRITE>
-__global__ void k_sweep(int64_t n, const double *__restrict__ xy, const double *__restrict__ h, Grid g,
-                        const int32_t *__restrict__ cell_of, const int64_t *__restrict__ cell_start,
-                        const int32_t *__restrict__ cell_nodes, const double2 *__restrict__ cell_xy,
-                        const float2 *__restrict__ cell_xyf, int32_t *__restrict__ counts,
-                        const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col)
+__global__ void __launch_bounds__(NB_THREADS) k_sweep(int64_t n, const double *__restrict__ h, Grid g, const int32_t *__restrict__ cell_of,
+                        const int64_t *__restrict__ cell_start, const int32_t *__restrict__ cell_nodes,
+                        const double2 *__restrict__ cell_xy, const float2 *__restrict__ cell_xyf,
+                        int32_t *__restrict__ counts, const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col)
 {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    int i = cell_nodes[t];
-    double xi = xy[2 * (int64_t)i], yi = xy[2 * (int64_t)i + 1];
-    double R = 2.0 * h[i];
-    double R2 = __dmul_rn(R, R);
+    __shared__ int32_t s_row[WRITE ? NB_THREADS / 32 : 1][WRITE ? ROW_MAX : 1];
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (int64_t)blockIdx.x * (NB_THREADS / 32) + (threadIdx.x >> 5);
+    if (t >= n) return;  // whole warps
+    const int64_t i = cell_nodes[t];
+    const double2 at = cell_xy[t];
+    const double R = 2.0 * h[i];
+    const double R2 = __dmul_rn(R, R);
     // float classification only where the float wrap cannot flip a candidate near the radius
     const bool filt = cell_xyf != nullptr && (!g.periodic || R2 <= g.r2_wrap_max);
-    const float xif = (float)xi, yif = (float)yi, R2f = (float)R2;
+    const float xif = (float)at.x, yif = (float)at.y, R2f = (float)R2;
     const float E = g.E;
-    int c = cell_of[i];
-    int cx = c % g.nc[0], cy = c / g.nc[0];
-    int xs[3], ys[3];
-    int mx = axis_cells(cx, g.nc[0], g.periodic, xs);
-    int my = axis_cells(cy, g.nc[1], g.periodic, ys);
+    const int c = cell_of[i];
+    const int cx = c % g.nc[0], cy = c / g.nc[0];
+    // the x range of cells, [xa, xb], and behind it the wrapped one [xc, xc] if there is one (xc < 0: none)
+    int xa = cx - 1, xb = cx + 1, xc = -1;
+    if (g.periodic && g.nc[0] > 3) {
+        if (xa < 0) xc = g.nc[0] - 1;
+        if (xb >= g.nc[0]) xc = 0;
+    } else if (g.periodic) {
+        xa = 0;
+        xb = g.nc[0] - 1;
+    }
+    xa = max(xa, 0);
+    xb = min(xb, g.nc[0] - 1);
+    int ys[3];
+    const int my = axis_cells(cy, g.nc[1], g.periodic, ys);
+    int64_t base = 0;
+    int total = 0;  // of the row, where it is written
+    if (WRITE) {
+        base = row_ptr[i];
+        total = (int)(row_ptr[i + 1] - base);
+    }
+    int32_t *dst = nullptr;
+    if constexpr (WRITE) dst = total <= ROW_MAX ? s_row[threadIdx.x >> 5] : col + base;
     int cnt = 0;
-    int64_t base = WRITE ? row_ptr[i] : 0;
-    for (int a = 0; a < my; a++) {
-        for (int b = 0; b < mx; b++) {
-            int cc = ys[a] * g.nc[0] + xs[b];
-            int64_t s = cell_start[cc], e = cell_start[cc + 1];
-            for (int64_t p = s; p < e; p++) {
-                int j = cell_nodes[p];
-                if (j == i) continue;
-                bool in;
+    for (int part = 0; part < (xc < 0 ? 1 : 2); part++) {
+        const int x0 = part ? xc : xa, x1 = part ? xc : xb;
+        int s[3], len[3];
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            s[a] = len[a] = 0;
+            if (a < my) {
+                s[a] = (int)cell_start[(int64_t)ys[a] * g.nc[0] + x0];
+                len[a] = (int)cell_start[(int64_t)ys[a] * g.nc[0] + x1 + 1] - s[a];
+            }
+        }
+        const int e1 = len[0], e2 = e1 + len[1], e3 = e2 + len[2];
+        const int d1 = s[1] - e1, d2 = s[2] - e2;
+        for (int q0 = 0; q0 < e3; q0 += 32) {
+            const int q = q0 + lane;
+            const int p = q + (q < e1 ? s[0] : q < e2 ? d1 : d2);
+            bool in = false;
+            if (q < e3 && p != t) {
                 int decided = 0;  // 1: inside, 2: outside, 0: to the double test
                 if (filt) {
                     const float2 qf = cell_xyf[p];
@@ -195,32 +292,27 @@ __global__ void k_sweep(int64_t n, const double *__restrict__ xy, const double *
                 if (decided) {
                     in = decided == 1;
                 } else {
-                    const double2 q = cell_xy[p];
-                    in = within_exact(q.x, q.y, xi, yi, R2, g);
-                }
-                if (in) {
-                    if (WRITE) col[base + cnt] = j;
-                    cnt++;
+                    const double2 qd = cell_xy[p];
+                    in = within_exact(qd.x, qd.y, at.x, at.y, R2, g);
                 }
             }
+            const unsigned hits = __ballot_sync(0xffffffffu, in);
+            if (WRITE && in) dst[cnt + __popc(hits & ((1u << lane) - 1u))] = cell_nodes[p];
+            cnt += __popc(hits);
         }
     }
-    if (!WRITE) {
-        counts[i] = cnt;
+    if constexpr (!WRITE) {
+        if (lane == 0) counts[i] = cnt;
     } else {
-        // insertion sort of the row (stencils hold tens of entries)
-        int32_t *row = col + base;
-        for (int u = 1; u < cnt; u++) {
-            int32_t v = row[u];
-            int w = u - 1;
-            while (w >= 0 && row[w] > v) {
-                row[w + 1] = row[w];
-                w--;
-            }
-            row[w + 1] = v;
-        }
+        __syncwarp();
+        if (cnt <= 32) sort_row<1>(dst, cnt, lane, col + base);
+        else if (cnt <= 64) sort_row<2>(dst, cnt, lane, col + base);
+        else if (cnt <= ROW_MAX) sort_row<4>(dst, cnt, lane, col + base);
+        else sort_long_row(col + base, cnt, lane);
     }
 }
+
+unsigned sweep_blocks(int64_t n) { return (unsigned)((n + NB_THREADS / 32 - 1) / (NB_THREADS / 32)); }
 
 }  // namespace
 
@@ -253,7 +345,10 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     unsigned long long *misc = ctx->misc.as<unsigned long long>();
     LABFM_CUDA_TRY(ctx, cudaMemsetAsync(misc, 0, 2 * sizeof(unsigned long long), s));
     int nb = (int)std::min<int64_t>((n + NB_THREADS - 1) / NB_THREADS, (int64_t)ctx->num_sms * 8);
-    k_check<<<nb, NB_THREADS, 0, s>>>(n, xy, h, lo[0], lo[1], hi[0], hi[1], misc);
+    LABFM_CUDA_TRY(ctx, ctx->node_xy.reserve(sizeof(double2) * n));
+    LABFM_CUDA_TRY(ctx, ctx->node_h.reserve(sizeof(double) * n));
+    k_check<<<nb, NB_THREADS, 0, s>>>(n, xy, h, lo[0], lo[1], hi[0], hi[1], misc, ctx->node_xy.as<double2>(),
+                                      ctx->node_h.as<double>());
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     unsigned long long *hs = (unsigned long long *)ctx->host_small;
     LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(hs, misc, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
@@ -307,13 +402,12 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
 
     int nbn = (int)((n + NB_THREADS - 1) / NB_THREADS);
     LABFM_CUDA_TRY(ctx, cudaMemsetAsync(cell_count, 0, sizeof(int32_t) * ncells, s));
-    k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count);
+    k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count, counts);  // counts: the ranks until the sweep
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(cell_count, cell_start, ncells, ctx->scan_tmp, s));
-    LABFM_CUDA_TRY(ctx, cudaMemsetAsync(cell_count, 0, sizeof(int32_t) * ncells, s));
-    k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, cell_count, cell_nodes, cell_xy, cell_xyf);
+    k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, cell_xyf);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
-    k_sweep<false><<<nbn, NB_THREADS, 0, s>>>(n, xy, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts,
+    k_sweep<false><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts,
                                               nullptr, nullptr);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(counts, row_ptr, n, ctx->scan_tmp, s));
@@ -323,7 +417,7 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     int64_t nnz = *nnz_h;
     if (nnz >= ((int64_t)1 << 40)) return fail(ctx, LABFM_ERR_CAPACITY, "too many stencil entries");
     LABFM_CUDA_TRY(ctx, ctx->col.reserve(sizeof(int32_t) * (nnz > 0 ? nnz : 1)));
-    k_sweep<true><<<nbn, NB_THREADS, 0, s>>>(n, xy, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr,
+    k_sweep<true><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr,
                                              row_ptr, ctx->col.as<int32_t>());
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
@@ -334,10 +428,6 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
         ctx->lo[d] = lo[d];
         ctx->hi[d] = hi[d];
     }
-    LABFM_CUDA_TRY(ctx, ctx->node_xy.reserve(sizeof(double) * 2 * n));
-    LABFM_CUDA_TRY(ctx, ctx->node_h.reserve(sizeof(double) * n));
-    LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->node_xy.ptr, xy, sizeof(double) * 2 * n, cudaMemcpyDeviceToDevice, s));
-    LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->node_h.ptr, h, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     *nnz_out = nnz;
     return LABFM_OK;
 }
@@ -433,7 +523,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
     // node check and h_max (the counters start at zero on every call)
     NA_TRY(cudaMemsetAsync(misc, 0, 2 * sizeof(unsigned long long), s));
     int nb = (int)std::min<int64_t>((n + NB_THREADS - 1) / NB_THREADS, (int64_t)num_sms * 8);
-    k_check<<<nb, NB_THREADS, 0, s>>>(n, xy, h, box_lo[0], box_lo[1], box_hi[0], box_hi[1], misc);
+    k_check<<<nb, NB_THREADS, 0, s>>>(n, xy, h, box_lo[0], box_lo[1], box_hi[0], box_hi[1], misc, nullptr, nullptr);
     NA_TRY(cudaGetLastError());
     unsigned long long hs[2];
     NA_TRY(cudaMemcpyAsync(hs, misc, sizeof hs, cudaMemcpyDeviceToHost, s));
@@ -467,14 +557,13 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
 
     int nbn = (int)((n + NB_THREADS - 1) / NB_THREADS);
     NA_TRY(cudaMemsetAsync(cell_count, 0, sizeof(int32_t) * ncells, s));
-    k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count);
+    k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count, counts);  // counts: the ranks until the sweep
     NA_TRY(cudaGetLastError());
     NA_TRY(exclusive_scan_i32_to_i64_ws(cell_count, cell_start, ncells, scan_tmp, NA_SCAN_ELEMS, s));
-    NA_TRY(cudaMemsetAsync(cell_count, 0, sizeof(int32_t) * ncells, s));
     // (the float pre-filter needs an array the fixed scratch does not hold: the double test alone)
-    k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, cell_count, cell_nodes, cell_xy, nullptr);
+    k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, nullptr);
     NA_TRY(cudaGetLastError());
-    k_sweep<false><<<nbn, NB_THREADS, 0, s>>>(n, xy, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, counts,
+    k_sweep<false><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, counts,
                                               nullptr, nullptr);
     NA_TRY(cudaGetLastError());
     NA_TRY(exclusive_scan_i32_to_i64_ws(counts, row_ptr, n, scan_tmp, NA_SCAN_ELEMS, s));
@@ -484,7 +573,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
     *nnz_out = nnz;
     if (nnz > col_capacity) return LABFM_ERR_CAPACITY;
     if (nnz > 0) {
-        k_sweep<true><<<nbn, NB_THREADS, 0, s>>>(n, xy, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr,
+        k_sweep<true><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr,
                                                  nullptr, row_ptr, col);
         NA_TRY(cudaGetLastError());
     }
