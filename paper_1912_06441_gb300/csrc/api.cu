@@ -190,6 +190,7 @@ labfm_status labfm_create(labfm_ctx **out, int device, void *stream)
         delete ctx;
         return LABFM_ERR_NOMEM;
     }
+    memset(ctx->host_small, 0, 1024);
     *out = ctx;
     return LABFM_OK;
 }
@@ -203,8 +204,10 @@ void labfm_destroy(labfm_ctx *ctx)
                       &ctx->cell_nodes, &ctx->counts, &ctx->scan_tmp, &ctx->misc, &ctx->w,
                       &ctx->status_tmp, &ctx->wtilde, &ctx->mscratch, &ctx->mrecs, &ctx->mwstore, &ctx->mfallback, &ctx->wcomb, &ctx->rk_acc,
                       &ctx->rk_stage_a, &ctx->rk_stage_b, &ctx->wburg, &ctx->bu_acc, &ctx->bu_stage_a,
-                      &ctx->bu_stage_b, &ctx->sol_w, &ctx->sol_vec, &ctx->sol_part, &ctx->sol_gmap, &ctx->sol_wg};
+                      &ctx->bu_stage_b, &ctx->sol_w, &ctx->sol_vec, &ctx->sol_part, &ctx->sol_gmap, &ctx->sync_buf};
     for (DevBuf *b : bufs) b->release();
+    ctx->sell.release();
+    ctx->sell_ghost.release();
     ctx->graph.release();
     ctx->graph_burgers.release();
     if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
@@ -236,6 +239,7 @@ labfm_status labfm_build_neighbours(labfm_ctx *ctx, int64_t n, const double *xy,
     if (cudaSetDevice(ctx->device) != cudaSuccess) return fail(ctx, LABFM_ERR_CUDA, "cudaSetDevice failed");
     ctx->have_weights = false;
     ctx->wcomb_valid = false;
+    ctx->sell.valid = false;
     return run_neighbours(ctx, n, xy, h, periodic ? 1 : 0, box_lo, box_hi, nnz_out);
 }
 
@@ -325,6 +329,7 @@ labfm_status labfm_apply(labfm_ctx *ctx, uint32_t op_mask, const void *f, int fi
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
+    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
     if (!f || !out) return fail(ctx, LABFM_ERR_ARG, "null field or output");
     if (field_dtype != LABFM_F64 && field_dtype != LABFM_F32) return fail(ctx, LABFM_ERR_ARG, "bad field_dtype");
     if (op_mask == 0 || (op_mask >> ctx->n_ops) != 0) return fail(ctx, LABFM_ERR_ARG, "op_mask selects no or unknown operators");
@@ -339,6 +344,7 @@ labfm_status labfm_step(labfm_ctx *ctx, const double *beta, void *u, int field_d
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
+    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
     if (!beta || !u) return fail(ctx, LABFM_ERR_ARG, "null beta or u");
     if (field_dtype != LABFM_F64 && field_dtype != LABFM_F32) return fail(ctx, LABFM_ERR_ARG, "bad field_dtype");
     if (!std::isfinite(dt) || nsteps < 0) return fail(ctx, LABFM_ERR_ARG, "dt must be finite and nsteps >= 0");
@@ -354,6 +360,7 @@ labfm_status labfm_solve(labfm_ctx *ctx, int op, const double *f, double *phi, c
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
+    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
     if (op < 0 || op >= ctx->n_ops) return fail(ctx, LABFM_ERR_ARG, "op must index a built operator");
     if (!f || !phi) return fail(ctx, LABFM_ERR_ARG, "null f or phi");
     if ((const void *)f == (const void *)phi) return fail(ctx, LABFM_ERR_ARG, "f and phi must be distinct buffers");
@@ -368,6 +375,7 @@ labfm_status labfm_solve_neumann(labfm_ctx *ctx, int op, const double *f, double
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
+    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
     if (op < 0 || op >= ctx->n_ops) return fail(ctx, LABFM_ERR_ARG, "op must index a built operator");
     if (!f || !phi) return fail(ctx, LABFM_ERR_ARG, "null f or phi");
     if ((const void *)f == (const void *)phi) return fail(ctx, LABFM_ERR_ARG, "f and phi must be distinct buffers");
@@ -394,6 +402,7 @@ labfm_status labfm_step_burgers(labfm_ctx *ctx, const double *beta, void *u, voi
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
+    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
     if (!ctx->grad01) return fail(ctx, LABFM_ERR_ARG, "operators 0 and 1 of the weights must be d/dx and d/dy");
     if (!beta || !u || !v) return fail(ctx, LABFM_ERR_ARG, "null beta, u or v");
     if (u == v) return fail(ctx, LABFM_ERR_ARG, "u and v must be distinct buffers");

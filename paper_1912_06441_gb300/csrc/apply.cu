@@ -1,17 +1,21 @@
 // Operator application (Eq. general_do) and the RK4 driver (Sec. 5.1).
 //
-// Both are streaming gather-sums over the CSR stencils: per stencil entry e of node i, read
+// Both are streaming gather-sums over the stencils: per stencil entry e of node i, read
 // col[e] and the weights w[e][*] once (HBM), gather f[col[e]] (stays in L2: the field is
 // small next to the weight stream and nodes are numbered in spatial order), and accumulate
-// (f_j - f_i) w.  A group of G lanes shares one node: the lanes read consecutive entries, so
-// every weight and index load of a warp is a contiguous, fully used segment; UNR entries per
-// lane are in flight before the first use.  The partial sums of a group are combined with
-// shuffles: by a reduce-scatter over the operators in the apply (each lane ends with one
-// operator's sum), by a butterfly tree in the RK4 and Burgers stages.
+// (f_j - f_i) w.
 //
-// (G, UNR) is chosen per context by a small autotuner: the first apply (or RK4 run) for a
-// given operator count, data types and problem class times every shape once on the real
+// The apply and the stages on float fields read the CSR rows: a group of G lanes shares one node, the
+// lanes read consecutive entries, so every weight and index load of a warp is a contiguous, fully used
+// segment; UNR entries per lane are in flight before the first use.  The partial sums of a group are combined with
+// shuffles: by a reduce-scatter over the operators in the apply (each lane ends with one
+// operator's sum), by a butterfly tree in the stages.  (G, UNR) is chosen per context by a small autotuner: the first
+// apply (or run) for a given operator count, data types and problem class times every shape once on the real
 // stencils and keeps the fastest.
+//
+// The stages on double fields read combined weights in the sliced layout of sell.cu: the FP64 pipe bounds them, and
+// there the lanes that combine sums and update nodes are a few percent of its work.
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -124,10 +128,10 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_apply(int64_t n, const int64_
 }
 
 // Storage of the combined RK4 weight wc_ji = sum_d beta_d w_ji^d (a context-owned buffer):
-//   CW_F64  double                    FP64 weights, FP64 fields: accumulated in double (the
-//                                     stencil indices are read from the CSR)
-//   CW_F32  int2 (j, w)               FP32 weights: each entry's stencil index and weight as one
-//                                     8-byte word, accumulated in the field type
+//   CW_S64  double                    FP64 weights, FP64 fields: accumulated in double, sliced layout
+//   CW_S32  float                     FP32 weights, FP64 fields: accumulated in double, sliced layout
+//   CW_F32  int2 (j, w)               FP32 weights and fields: each entry's stencil index and weight as one
+//                                     8-byte word in CSR order, accumulated in float
 //   CW_DF   int2 (j, hi), float lo    FP64 weights, FP32 fields: the double rounded to a
 //                                     double-float pair once, here, so that the stage
 //                                     accumulates on the FP32 pipes (about 48 bits, far below the
@@ -135,24 +139,33 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_apply(int64_t n, const int64_
 //                                     in FP64 for every stencil entry; the low parts follow the
 //                                     nnz index/high-part words
 // Packing the index with the weight gives one wide load per entry for the same bytes.
-enum { CW_F64 = 0, CW_F32 = 1, CW_DF = 2 };
+enum { CW_S64 = 0, CW_F32 = 1, CW_DF = 2, CW_S32 = 3 };
 
-int cw_format(int fdt, int wdt) { return wdt == LABFM_F32 ? CW_F32 : (fdt == LABFM_F32 ? CW_DF : CW_F64); }
-size_t cw_bytes(int fmt) { return fmt == CW_DF ? 12 : 8; }
+int cw_format(int fdt, int wdt)
+{
+    if (fdt == LABFM_F64) return wdt == LABFM_F64 ? CW_S64 : CW_S32;
+    return wdt == LABFM_F32 ? CW_F32 : CW_DF;
+}
+bool cw_sliced(int fmt) { return fmt == CW_S64 || fmt == CW_S32; }
+size_t cw_bytes(const labfm_ctx *ctx, int fmt)
+{
+    if (cw_sliced(fmt)) return (fmt == CW_S64 ? 8 : 4) * (size_t)ctx->sell.places;
+    return (fmt == CW_DF ? 12 : 8) * (size_t)ctx->nnz;
+}
+
+struct Beta {
+    double v[MAX_OPS];
+};
 
 template <class WT>
 __global__ void k_combine(int64_t nnz, int n_ops, const WT *__restrict__ w, const int32_t *__restrict__ col,
-                          void *__restrict__ wc, int fmt, double b0, double b1, double b2, double b3, double b4,
-                          double b5, double b6, double b7)
+                          void *__restrict__ wc, int fmt, Beta b)
 {
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= nnz) return;
-    const double b[8] = {b0, b1, b2, b3, b4, b5, b6, b7};
     double s = 0.0;
-    for (int d = 0; d < n_ops; d++) s = fma(b[d], (double)w[e * n_ops + d], s);
-    if (fmt == CW_F64) {
-        ((double *)wc)[e] = s;
-    } else if (fmt == CW_F32) {
+    for (int d = 0; d < n_ops; d++) s = fma(b.v[d], (double)w[e * n_ops + d], s);
+    if (fmt == CW_F32) {
         ((int2 *)wc)[e] = make_int2(col[e], __float_as_int((float)s));
     } else {
         df v = df_from_double(s);
@@ -161,39 +174,53 @@ __global__ void k_combine(int64_t nnz, int n_ops, const WT *__restrict__ w, cons
     }
 }
 
+// wc in the sliced layout (a warp per slice): 0 where there is no entry
+template <class WT, class VT>
+__global__ void __launch_bounds__(APPLY_THREADS) k_combine_sliced(int64_t n, SellView S,
+                                                                 const int64_t *__restrict__ row_ptr, int n_ops,
+                                                                 const WT *__restrict__ w, VT *__restrict__ wc, Beta b)
+{
+    const SellLane l((int64_t)blockIdx.x * (APPLY_THREADS / 32) + (threadIdx.x >> 5), threadIdx.x & 31, n, S);
+    const int64_t rs = l.i >= 0 ? row_ptr[l.i] : 0, re = l.i >= 0 ? row_ptr[l.i + 1] : 0;
+    for (int k = 0; k < l.steps; k++) {
+        const int64_t e = rs + ((int64_t)k << S.lg_l) + l.h;
+        double s = 0.0;
+        if (e < re)
+            for (int d = 0; d < n_ops; d++) s = fma(b.v[d], (double)w[e * n_ops + d], s);
+        wc[l.at + 32 * (int64_t)k] = (VT)s;
+    }
+}
+
 // One RK4 stage.  F_i = sum_j (src_j - src_i) wc_ji (0 on frozen nodes), then
 //   stage 0: acc = u + dt/6 F,  nxt = u + dt/2 F
 //   stage 1: acc += dt/3 F,     nxt = u + dt/2 F
 //   stage 2: acc += dt/3 F,     nxt = u + dt F
 //   stage 3: u = acc + dt/6 F
-// The per-node update runs in the field type.
-template <class FT, int CW, int UNR>
-__global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage(int64_t n, const int64_t *__restrict__ row_ptr,
+// with ca the coefficient of acc (or u) and cn that of nxt, products formed on the host (in FP64 a product per thread
+// takes the pipe as long as a stencil entry of the warp).  The per-node update runs in the field type.
+template <int CW, int UNR>
+__global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage_csr(int64_t n, const int64_t *__restrict__ row_ptr,
                                                              const int32_t *__restrict__ col,
                                                              const void *__restrict__ wc_raw,
                                                              const float *__restrict__ wc_lo,
-                                                             const FT *__restrict__ src, FT *__restrict__ u,
-                                                             FT *__restrict__ acc_buf, FT *__restrict__ nxt,
-                                                             const uint8_t *__restrict__ frozen, int stage, FT dt,
-                                                             int lg_g)
+                                                             const float *src, float *__restrict__ u,
+                                                             float *__restrict__ acc_buf, float *__restrict__ nxt,
+                                                             const uint8_t *__restrict__ frozen, int stage, float ca,
+                                                             float cnx, int lg_g)
 {
-    // AT: type of the stencil sum (double-float for CW_DF); the per-node update runs in FT
-    using AT = typename std::conditional<std::is_same<FT, float>::value && CW != CW_F64, float, double>::type;
-    using WT = typename std::conditional<CW == CW_F64, double, float2>::type;  // (weight, low part)
-    const double *__restrict__ wcd = (const double *)wc_raw;
     const int2 *__restrict__ wcp = (const int2 *)wc_raw;
     const int G = 1 << lg_g;  // lanes per node, a power of two
     const int lane = threadIdx.x & (G - 1);
     const int64_t i = ((int64_t)blockIdx.x * APPLY_THREADS + threadIdx.x) >> lg_g;
     const bool live = i < n;
     int64_t rs = 0, re = 0;
-    FT si = 0;
+    bool fixed = false;
     if (live) {
         rs = row_ptr[i];
         re = row_ptr[i + 1];
-        si = src[i];
+        fixed = frozen && frozen[i];
     }
-    AT acc = 0;
+    float acc = 0.0f;
     df accd{0.0f, 0.0f};
     // FP32 weights: the stencil stream is software-pipelined (the next batch of UNR entries per
     // lane is loaded before the gathers of the current one, so its latency overlaps them: +8 % at
@@ -201,30 +228,26 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage(int64_t n, const in
     // gains (-11 %), so those load each batch just before its gathers
     constexpr bool PIPE = CW == CW_F32;
     int cn[UNR];
-    WT wn[UNR];
+    float2 wn[UNR];  // (weight, low part)
     auto load_batch = [&](int64_t base) {
 #pragma unroll
         for (int q = 0; q < UNR; q++) {
             const int64_t e = base + (int64_t)q * G + lane;
             if (e < re) {
-                if constexpr (CW == CW_F64) {
-                    cn[q] = __ldcs(col + e);
-                    wn[q] = __ldcs(wcd + e);
-                } else {
-                    const int2 pr = __ldcs(wcp + e);  // stencil index and (high part of the) weight
-                    cn[q] = pr.x;
-                    wn[q] = make_float2(__int_as_float(pr.y), CW == CW_DF ? __ldcs(wc_lo + e) : 0.0f);
-                }
+                const int2 pr = __ldcs(wcp + e);  // stencil index and (high part of the) weight
+                cn[q] = pr.x;
+                wn[q] = make_float2(__int_as_float(pr.y), CW == CW_DF ? __ldcs(wc_lo + e) : 0.0f);
             } else {
                 cn[q] = -1;
             }
         }
     };
-    if (PIPE && rs < re) load_batch(rs);
+    if (rs < re) load_batch(rs);
+    const float si = live ? src[i] : 0.0f;
     for (int64_t base = rs; base < re; base += (int64_t)G * UNR) {
-        if (!PIPE) load_batch(base);
+        if (!PIPE && base != rs) load_batch(base);
         int cj[UNR];
-        WT wv[UNR];
+        float2 wv[UNR];
 #pragma unroll
         for (int q = 0; q < UNR; q++) {
             cj[q] = cn[q];
@@ -236,12 +259,10 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage(int64_t n, const in
             if (cj[q] >= 0) {
                 if constexpr (CW == CW_DF) {
                     float dh, dl;  // src_j - src_i exactly, as a double-float
-                    two_sum((float)src[cj[q]], -(float)si, dh, dl);
+                    two_sum(src[cj[q]], -si, dh, dl);
                     accd = df_fma(df{dh, dl}, df{wv[q].x, wv[q].y}, accd);
-                } else if constexpr (CW == CW_F32) {
-                    acc = fma((AT)src[cj[q]] - (AT)si, (AT)wv[q].x, acc);
                 } else {
-                    acc = fma((AT)src[cj[q]] - (AT)si, (AT)wv[q], acc);
+                    acc = fma(src[cj[q]] - si, wv[q].x, acc);
                 }
             }
         }
@@ -251,29 +272,84 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage(int64_t n, const in
             df other{__shfl_xor_sync(0xffffffffu, accd.hi, o), __shfl_xor_sync(0xffffffffu, accd.lo, o)};
             accd = df_add(accd, other);
         }
-        acc = accd.hi + accd.lo;  // CW_DF comes with FP32 fields
+        acc = accd.hi + accd.lo;
     } else {
         for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     }
     if (!live || lane != 0) return;
-    const FT F = (frozen && frozen[i]) ? (FT)0 : (FT)acc;
-    const FT ui = u[i];
-    switch (stage) {
-    case 0:
-        acc_buf[i] = ui + dt * (FT)(1.0 / 6.0) * F;
-        nxt[i] = ui + dt * (FT)0.5 * F;
-        break;
-    case 1:
-        acc_buf[i] = acc_buf[i] + dt * (FT)(1.0 / 3.0) * F;
-        nxt[i] = ui + dt * (FT)0.5 * F;
-        break;
-    case 2:
-        acc_buf[i] = acc_buf[i] + dt * (FT)(1.0 / 3.0) * F;
-        nxt[i] = ui + dt * F;
-        break;
-    default:
-        u[i] = acc_buf[i] + dt * (FT)(1.0 / 6.0) * F;
-        break;
+    const float F = fixed ? 0.0f : acc;
+    if (stage == 3) {
+        u[i] = acc_buf[i] + ca * F;
+        return;
+    }
+    const float ui = u[i];
+    acc_buf[i] = (stage == 0 ? ui : acc_buf[i]) + ca * F;
+    nxt[i] = ui + cnx * F;
+}
+
+// Coefficients of a step's stages
+struct RkCoef {
+    double sixth, third, half, one;  // dt / 6, dt / 3, dt / 2, dt
+};
+RkCoef rk_coef(double dt) { return RkCoef{dt * (1.0 / 6.0), dt * (1.0 / 3.0), dt * 0.5, dt}; }
+
+// nsteps steps on double fields, sliced layout, one cooperative launch (see GridBarrier): a warp per slice, the next
+// RUN_U steps' indices and weights loaded before the gathers of the current ones, the first of a sweep before its
+// barrier.  A lane adds into two sums in turn, because a dependent FP64 add waits several times the pipe's time for one.
+constexpr int RUN_U = 8;
+template <class VT>
+__global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView S, const VT *__restrict__ wc, double *u,
+                                                           double *acc_buf, double *sa, double *sb,
+                                                           const uint8_t *__restrict__ frozen, int64_t nsteps, RkCoef rk,
+                                                           GridSync sync)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t s0, s1;
+    slice_share(S.n_slices, s0, s1);
+    GridBarrier bar{sync};
+    const SellLane first(s0 + warp < s1 ? s0 + warp : S.n_slices, lane, n, S);
+    SliceBatch<RUN_U, 1, VT> nx;
+    nx.load(first, lane, 0, S, wc);
+    for (int64_t it = 0; it < 4 * nsteps; it++) {
+        const int stage = (int)(it & 3);
+        const double *src = stage == 0 ? u : stage == 2 ? sb : sa;
+        for (int64_t slice = s0 + warp; slice < s1; slice += RUN_THREADS / 32) {
+            SellLane l = first;
+            if (slice != s0 + warp) {
+                l = SellLane(slice, lane, n, S);
+                nx.load(l, lane, 0, S, wc);
+            }
+            const int64_t i = l.i;
+            const double si = i >= 0 ? src[i] : 0.0;
+            const bool row = i >= 0 && l.h == 0;  // this lane updates the node; what it needs is read ahead
+            const bool fixed = row && frozen && frozen[i];
+            const double ui = row && stage != 3 ? u[i] : 0.0, ai = row && stage != 0 ? acc_buf[i] : 0.0;
+            double sum[2] = {0.0, 0.0};
+            for (int k0 = 0; k0 < l.steps; k0 += RUN_U) {
+                double x[RUN_U];
+                const SliceBatch<RUN_U, 1, VT> b = nx;
+#pragma unroll
+                for (int q = 0; q < RUN_U; q++)
+                    if (b.c[q] >= 0) x[q] = src[b.c[q]];
+                if (k0 + RUN_U < l.steps) nx.load(l, lane, k0 + RUN_U, S, wc);
+#pragma unroll
+                for (int q = 0; q < RUN_U; q++)
+                    if (b.c[q] >= 0) sum[q & 1] = fma(x[q] - si, (double)b.w[q][0], sum[q & 1]);
+            }
+            double acc = sum[0] + sum[1];
+            for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (!row) continue;
+            const double F = fixed ? 0.0 : acc;
+            if (stage == 3) {
+                u[i] = ai + rk.sixth * F;
+                continue;
+            }
+            acc_buf[i] = stage == 0 ? ui + rk.sixth * F : ai + rk.third * F;
+            (stage == 1 ? sb : sa)[i] = ui + (stage == 2 ? rk.one : rk.half) * F;
+        }
+        if (it + 1 == 4 * nsteps) break;
+        nx.load(first, lane, 0, S, wc);
+        if (!bar.wait()) return;
     }
 }
 
@@ -295,6 +371,11 @@ Shape default_shape(const labfm_ctx *ctx, int min_g)
 }
 
 unsigned blocks_for(int64_t n, int G) { return (unsigned)((n * G + APPLY_THREADS - 1) / APPLY_THREADS); }
+
+// Coefficients of stage 0 .. 3 (see k_rk4_stage_csr)
+float stage_ca(int stage, double dt) { return (float)dt * (float)(stage == 0 || stage == 3 ? 1.0 / 6.0 : 1.0 / 3.0); }
+float stage_cn(int stage, double dt) { return stage == 2 ? (float)dt : (float)dt * 0.5f; }
+
 int log2_of(int G)
 {
     int l = 0;
@@ -318,24 +399,27 @@ cudaError_t launch_apply_shape(labfm_ctx *ctx, Shape sh, uint32_t mask, const vo
     return cudaGetLastError();
 }
 
-template <class FT, int CW>
-cudaError_t launch_stage_shape(labfm_ctx *ctx, Shape sh, const FT *src, FT *u, FT *acc, FT *nxt, const uint8_t *frozen,
-                               int stage, double dt, cudaStream_t s)
+template <int CW>
+cudaError_t launch_stage_csr(labfm_ctx *ctx, Shape sh, const float *src, float *u, float *acc, float *nxt,
+                             const uint8_t *frozen, int stage, double dt, cudaStream_t s)
 {
     const unsigned blocks = blocks_for(ctx->n, sh.G);
     const void *wc = ctx->wcomb.ptr;
     const float *wc_lo = CW == CW_DF ? reinterpret_cast<const float *>(ctx->wcomb.as<int2>() + ctx->nnz) : nullptr;
     auto args = [&](auto kern) {
-        kern<<<blocks, APPLY_THREADS, 0, s>>>(ctx->n, ctx->row_ptr.as<int64_t>(), ctx->col.as<int32_t>(), wc, wc_lo,
-                                              src, u, acc, nxt, frozen, stage, (FT)dt, log2_of(sh.G));
+        kern<<<blocks, APPLY_THREADS, 0, s>>>(ctx->n, ctx->row_ptr.as<int64_t>(), ctx->col.as<int32_t>(), wc, wc_lo, src, u,
+                                              acc, nxt, frozen, stage, stage_ca(stage, dt), stage_cn(stage, dt),
+                                              log2_of(sh.G));
     };
     switch (sh.UNR) {
-    case 2: args(k_rk4_stage<FT, CW, 2>); break;
-    case 8: args(k_rk4_stage<FT, CW, 8>); break;
-    default: args(k_rk4_stage<FT, CW, 4>); break;
+    case 2: args(k_rk4_stage_csr<CW, 2>); break;
+    case 8: args(k_rk4_stage_csr<CW, 8>); break;
+    default: args(k_rk4_stage_csr<CW, 4>); break;
     }
     return cudaGetLastError();
 }
+
+unsigned slice_blocks(const labfm_ctx *ctx, int threads) { return (unsigned)((ctx->sell.n_slices * 32 + threads - 1) / threads); }
 
 // Time every shape with `run` (which enqueues one launch on ctx->stream) and keep the fastest.
 template <class RunFn>
@@ -425,38 +509,45 @@ cudaError_t launch_apply_n(labfm_ctx *ctx, uint32_t mask, const void *f, int fdt
                             : launch_apply_t<NOPS, float, float>(ctx, mask, f, fdt, out);
 }
 
-template <class FT, int CW>
-cudaError_t enqueue_steps(labfm_ctx *ctx, void *u, int fdt, double dt, int64_t nsteps, const uint8_t *frozen,
-                          cudaStream_t s)
+// Float fields: the launches of nsteps steps on stream s (nsteps = 0: only tunes the launch shape, on ctx->stream)
+template <int CW>
+cudaError_t enqueue_steps_csr(labfm_ctx *ctx, void *u, double dt, int64_t nsteps, const uint8_t *frozen, cudaStream_t s)
 {
-    FT *uu = (FT *)u, *acc = ctx->rk_acc.as<FT>(), *sa = ctx->rk_stage_a.as<FT>(), *sb = ctx->rk_stage_b.as<FT>();
+    float *uu = (float *)u, *acc = ctx->rk_acc.as<float>(), *sa = ctx->rk_stage_a.as<float>(), *sb = ctx->rk_stage_b.as<float>();
     // tune on stage 0, which reads u and writes only the work buffers
     Shape sh;
     cudaError_t e = autotune(
-        ctx, tune_key(ctx, 2, 1, fdt, ctx->wdtype), 1,
-        [&](Shape sp) { return launch_stage_shape<FT, CW>(ctx, sp, uu, uu, acc, sa, frozen, 0, dt, ctx->stream); },
-        sh);
+        ctx, tune_key(ctx, 2, 1, LABFM_F32, ctx->wdtype), 1,
+        [&](Shape sp) { return launch_stage_csr<CW>(ctx, sp, uu, uu, acc, sa, frozen, 0, dt, ctx->stream); }, sh);
     if (e != cudaSuccess) return e;
     for (int64_t st = 0; st < nsteps; st++) {
-        if ((e = launch_stage_shape<FT, CW>(ctx, sh, uu, uu, acc, sa, frozen, 0, dt, s)) != cudaSuccess) return e;
-        if ((e = launch_stage_shape<FT, CW>(ctx, sh, sa, uu, acc, sb, frozen, 1, dt, s)) != cudaSuccess) return e;
-        if ((e = launch_stage_shape<FT, CW>(ctx, sh, sb, uu, acc, sa, frozen, 2, dt, s)) != cudaSuccess) return e;
-        if ((e = launch_stage_shape<FT, CW>(ctx, sh, sa, uu, acc, (FT *)nullptr, frozen, 3, dt, s)) != cudaSuccess)
-            return e;
+        if ((e = launch_stage_csr<CW>(ctx, sh, uu, uu, acc, sa, frozen, 0, dt, s)) != cudaSuccess) return e;
+        if ((e = launch_stage_csr<CW>(ctx, sh, sa, uu, acc, sb, frozen, 1, dt, s)) != cudaSuccess) return e;
+        if ((e = launch_stage_csr<CW>(ctx, sh, sb, uu, acc, sa, frozen, 2, dt, s)) != cudaSuccess) return e;
+        if ((e = launch_stage_csr<CW>(ctx, sh, sa, uu, acc, nullptr, frozen, 3, dt, s)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-cudaError_t enqueue_steps_dt(labfm_ctx *ctx, int fdt, void *u, double dt, int64_t nsteps, const uint8_t *frozen,
+cudaError_t enqueue_steps_dt(labfm_ctx *ctx, int fmt, void *u, double dt, int64_t nsteps, const uint8_t *frozen,
                              cudaStream_t s)
 {
-    switch (cw_format(fdt, ctx->wdtype)) {
-    case CW_F64: return enqueue_steps<double, CW_F64>(ctx, u, fdt, dt, nsteps, frozen, s);
-    case CW_DF: return enqueue_steps<float, CW_DF>(ctx, u, fdt, dt, nsteps, frozen, s);
-    default:
-        return fdt == LABFM_F64 ? enqueue_steps<double, CW_F32>(ctx, u, fdt, dt, nsteps, frozen, s)
-                                : enqueue_steps<float, CW_F32>(ctx, u, fdt, dt, nsteps, frozen, s);
-    }
+    return fmt == CW_DF ? enqueue_steps_csr<CW_DF>(ctx, u, dt, nsteps, frozen, s)
+                        : enqueue_steps_csr<CW_F32>(ctx, u, dt, nsteps, frozen, s);
+}
+
+// Steps of a run in one cooperative launch: it holds its SMs until it ends, so that it is kept to tens of milliseconds
+// (about 5 ns per thousand entries and stage)
+int64_t steps_per_run(const labfm_ctx *ctx) { return std::max<int64_t>(1, (int64_t)1000000000 / (ctx->nnz + 100000)); }
+
+// Double fields: the run as cooperative launches on the context's stream; fn(steps) enqueues one
+template <class Fn>
+cudaError_t enqueue_runs(const labfm_ctx *ctx, int64_t nsteps, Fn fn)
+{
+    const int64_t per = steps_per_run(ctx);
+    cudaError_t e = cudaSuccess;
+    for (int64_t at = 0; at < nsteps && e == cudaSuccess; at += per) e = fn(std::min(per, nsteps - at));
+    return e;
 }
 
 }  // namespace
@@ -482,23 +573,38 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
     const int64_t n = ctx->n, nnz = ctx->nnz;
     size_t fsz = fdt == LABFM_F64 ? 8 : 4;
     const int fmt = cw_format(fdt, ctx->wdtype);
+    if (cw_sliced(fmt)) {
+        labfm_status st = ensure_sell(ctx);
+        if (st != LABFM_OK) return st;
+    }
     // combined weight, cached while beta, the weights and the storage format are unchanged
     bool same_beta = ctx->wcomb_valid && ctx->wcomb_dtype == fmt;
     for (int d = 0; d < ctx->n_ops && same_beta; d++) same_beta = (ctx->beta_cached[d] == beta[d]);
     if (!same_beta) {
-        LABFM_CUDA_TRY(ctx, ctx->wcomb.reserve(cw_bytes(fmt) * (nnz > 0 ? nnz : 1)));
-        double b[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int d = 0; d < ctx->n_ops; d++) b[d] = beta[d];
-        unsigned blocks = (unsigned)((nnz + 255) / 256);
+        const size_t bytes = cw_bytes(ctx, fmt);
+        LABFM_CUDA_TRY(ctx, ctx->wcomb.reserve(bytes > 0 ? bytes : 8));
+        Beta b{};
+        for (int d = 0; d < ctx->n_ops; d++) b.v[d] = beta[d];
+        const int64_t *rp = ctx->row_ptr.as<int64_t>();
+        const int32_t *cl = ctx->col.as<int32_t>();
+        const unsigned blocks = (unsigned)((nnz + 255) / 256), sb = slice_blocks(ctx, APPLY_THREADS);
         if (nnz > 0) {
-            if (ctx->wdtype == LABFM_F64)
-                k_combine<double><<<blocks, 256, 0, s>>>(nnz, ctx->n_ops, ctx->w.as<double>(), ctx->col.as<int32_t>(),
-                                                         ctx->wcomb.ptr, fmt,
-                                                         b[0], b[1], b[2], b[3], b[4], b[5], b[6], b[7]);
-            else
-                k_combine<float><<<blocks, 256, 0, s>>>(nnz, ctx->n_ops, ctx->w.as<float>(), ctx->col.as<int32_t>(),
-                                                        ctx->wcomb.ptr, fmt,
-                                                        b[0], b[1], b[2], b[3], b[4], b[5], b[6], b[7]);
+            switch (fmt) {
+            case CW_S64:
+                k_combine_sliced<double, double><<<sb, APPLY_THREADS, 0, s>>>(n, sell_view(ctx->sell), rp, ctx->n_ops,
+                                                                             ctx->w.as<double>(), ctx->wcomb.as<double>(), b);
+                break;
+            case CW_S32:
+                k_combine_sliced<float, float><<<sb, APPLY_THREADS, 0, s>>>(n, sell_view(ctx->sell), rp, ctx->n_ops,
+                                                                           ctx->w.as<float>(), ctx->wcomb.as<float>(), b);
+                break;
+            case CW_DF:
+                k_combine<double><<<blocks, 256, 0, s>>>(nnz, ctx->n_ops, ctx->w.as<double>(), cl, ctx->wcomb.ptr, fmt, b);
+                break;
+            default:
+                k_combine<float><<<blocks, 256, 0, s>>>(nnz, ctx->n_ops, ctx->w.as<float>(), cl, ctx->wcomb.ptr, fmt, b);
+                break;
+            }
             LABFM_CUDA_TRY(ctx, cudaGetLastError());
         }
         for (int d = 0; d < ctx->n_ops; d++) ctx->beta_cached[d] = beta[d];
@@ -508,6 +614,19 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
     LABFM_CUDA_TRY(ctx, ctx->rk_acc.reserve(fsz * n));
     LABFM_CUDA_TRY(ctx, ctx->rk_stage_a.reserve(fsz * n));
     LABFM_CUDA_TRY(ctx, ctx->rk_stage_b.reserve(fsz * n));
+
+    if (cw_sliced(fmt)) {
+        double *uu = (double *)u, *acc = ctx->rk_acc.as<double>(), *sa = ctx->rk_stage_a.as<double>(), *sb = ctx->rk_stage_b.as<double>();
+        const SellView S = sell_view(ctx->sell);
+        LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
+        cudaError_t e = enqueue_runs(ctx, nsteps, [&](int64_t steps) {
+            return fmt == CW_S64 ? launch_run(ctx, S.n_slices, k_rk4_run<double>, n, S, ctx->wcomb.as<double>(), uu, acc, sa, sb,
+                                              frozen, steps, rk_coef(dt), grid_sync(ctx))
+                                 : launch_run(ctx, S.n_slices, k_rk4_run<float>, n, S, ctx->wcomb.as<float>(), uu, acc, sa, sb,
+                                              frozen, steps, rk_coef(dt), grid_sync(ctx));
+        });
+        return e == cudaSuccess ? LABFM_OK : cuda_fail(ctx, e, "RK4 run");
+    }
 
     StepGraph &g = ctx->graph;
     const bool same = g.exec && g.u == u && g.frozen == frozen && g.dtype == fdt && g.dt == dt &&
@@ -524,13 +643,13 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
         cudaGraph_t graph = nullptr;
         // shapes are tuned (on the context stream) before the capture begins
         {
-            cudaError_t te = enqueue_steps_dt(ctx, fdt, u, dt, 0, frozen, s);
+            cudaError_t te = enqueue_steps_dt(ctx, fmt, u, dt, 0, frozen, s);
             if (te != cudaSuccess) return cuda_fail(ctx, te, "RK4 stage tuning");
             // the capture stream must not start before the tuning launches end
             LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
         }
         LABFM_CUDA_TRY(ctx, cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = enqueue_steps_dt(ctx, fdt, u, dt, nsteps, frozen, ctx->capture_stream);
+        cudaError_t e = enqueue_steps_dt(ctx, fmt, u, dt, nsteps, frozen, ctx->capture_stream);
         cudaError_t e2 = cudaStreamEndCapture(ctx->capture_stream, &graph);
         if (e != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
@@ -572,172 +691,242 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
 namespace labfm {
 namespace {
 
-// per entry: (w^0, w^1, sum_{d>=2} beta_d w^d), the last summed in double
+// Weights of the stages, the third summed in double: (w^0, w^1, sum_{d>=2} beta_d w^d) per entry in CSR order (float
+// fields), or in the sliced layout, three runs of 32 per step of a slice (double fields).
 template <class WT>
-__global__ void k_burg_combine(int64_t nnz, int n_ops, const WT *__restrict__ w, WT *__restrict__ wb, double b2,
-                               double b3, double b4, double b5, double b6, double b7)
+__global__ void k_burg_combine(int64_t nnz, int n_ops, const WT *__restrict__ w, WT *__restrict__ wb, Beta b)
 {
-    const double bb[6] = {b2, b3, b4, b5, b6, b7};
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz; e += (int64_t)gridDim.x * blockDim.x) {
         const WT *we = w + e * n_ops;
         double s = 0.0;
-        for (int d = 2; d < n_ops; d++) s += bb[d - 2] * (double)we[d];
+        for (int d = 2; d < n_ops; d++) s += b.v[d] * (double)we[d];
         wb[3 * e] = we[0];
         wb[3 * e + 1] = we[1];
         wb[3 * e + 2] = (WT)s;
     }
 }
 
-// One RK4 stage for the pair (u, v).  With the stage's source fields (su, sv):
-//   A_x(s)_i = sum_j (s_j - s_i) w^0,  A_y(s)_i = sum_j (s_j - s_i) w^1,  B(s)_i = sum_j (s_j - s_i) wl
-//   F_u = -(su_i A_x(su) + sv_i A_y(su)) + B(su),   F_v = -(su_i A_x(sv) + sv_i A_y(sv)) + B(sv)
-// (0 on frozen nodes), then the stage updates of k_rk4_stage for both fields; acc and nxt hold
-// u in [0, n) and v in [n, 2n).  Sums in double unless fields and weights are both float.
-template <class FT, class WT, int UNR>
-__global__ void __launch_bounds__(APPLY_THREADS) k_burgers_stage(int64_t n, const int64_t *__restrict__ row_ptr,
-                                                                 const int32_t *__restrict__ col,
-                                                                 const WT *__restrict__ wb, const FT *__restrict__ su,
-                                                                 const FT *__restrict__ sv, FT *__restrict__ u,
-                                                                 FT *__restrict__ v, FT *__restrict__ acc,
-                                                                 FT *__restrict__ nxt,
-                                                                 const uint8_t *__restrict__ frozen, int stage, FT dt,
-                                                                 int lg_g)
+template <class WT>
+__global__ void __launch_bounds__(APPLY_THREADS) k_burg_combine_sliced(int64_t n, SellView S,
+                                                                      const int64_t *__restrict__ row_ptr, int n_ops,
+                                                                      const WT *__restrict__ w, WT *__restrict__ wb, Beta b)
 {
-    using AT = typename std::conditional<std::is_same<FT, float>::value && std::is_same<WT, float>::value, float,
-                                         double>::type;
+    const int lane = threadIdx.x & 31;
+    const SellLane l((int64_t)blockIdx.x * (APPLY_THREADS / 32) + (threadIdx.x >> 5), lane, n, S);
+    const int64_t rs = l.i >= 0 ? row_ptr[l.i] : 0, re = l.i >= 0 ? row_ptr[l.i + 1] : 0;
+    WT *out = wb + 3 * (l.at - lane) + lane;
+    for (int k = 0; k < l.steps; k++, out += 96) {
+        const int64_t e = rs + ((int64_t)k << S.lg_l) + l.h;
+        const WT *we = w + e * n_ops;
+        double s = 0.0;
+        if (e < re)
+            for (int d = 2; d < n_ops; d++) s += b.v[d] * (double)we[d];
+        out[0] = e < re ? we[0] : (WT)0;
+        out[32] = e < re ? we[1] : (WT)0;
+        out[64] = (WT)s;
+    }
+}
+
+// One RK4 stage for the pair (u, v).  With the stage's source fields (su, sv), the advection weights of node i join
+// the linear one per entry, c_ji = wl_ji - su_i w^0_ji - sv_i w^1_ji, and
+//   F_u = sum_j (su_j - su_i) c_ji,   F_v = sum_j (sv_j - sv_i) c_ji
+// (0 on frozen nodes): six FP64 instructions per entry and two sums to combine, where the sums with w^0, w^1 and wl
+// apart take eight and six; the FP64 pipe bounds the stage on sets that fit the L2 cache.  Then the stage updates
+// of k_rk4_stage for both fields; acc and nxt hold u in [0, n) and v in [n, 2n).  Sums in double unless fields and
+// weights are both float.
+template <class WT, int UNR>
+__global__ void __launch_bounds__(APPLY_THREADS) k_burgers_stage_csr(int64_t n, const int64_t *__restrict__ row_ptr,
+                                                                 const int32_t *__restrict__ col,
+                                                                 const WT *__restrict__ wb, const float *su,
+                                                                 const float *sv, float *__restrict__ u,
+                                                                 float *__restrict__ v, float *__restrict__ acc,
+                                                                 float *__restrict__ nxt,
+                                                                 const uint8_t *__restrict__ frozen, int stage, float ca,
+                                                                 float cnx, int lg_g)
+{
+    using AT = WT;  // float weights: sums in float
     const int G = 1 << lg_g;
     const int lane = threadIdx.x & (G - 1);
     const int64_t i = ((int64_t)blockIdx.x * APPLY_THREADS + threadIdx.x) >> lg_g;
     const bool live = i < n;
     int64_t rs = 0, re = 0;
-    AT ui = 0, vi = 0;
+    bool fixed = false;
     if (live) {
         rs = row_ptr[i];
         re = row_ptr[i + 1];
-        ui = (AT)su[i];
-        vi = (AT)sv[i];
+        fixed = frozen && frozen[i];
     }
-    AT s[6] = {0, 0, 0, 0, 0, 0};  // A_x(u), A_y(u), B(u), A_x(v), A_y(v), B(v)
-    for (int64_t base = rs; base < re; base += (int64_t)G * UNR) {
-        int cj[UNR];
-        AT w0[UNR], w1[UNR], wl[UNR];
+    int cj[UNR];
+    WT w0[UNR], w1[UNR], wl[UNR];
+    auto load_batch = [&](int64_t base) {
 #pragma unroll
         for (int q = 0; q < UNR; q++) {
             const int64_t e = base + (int64_t)q * G + lane;
             if (e < re) {
                 cj[q] = __ldcs(col + e);
-                w0[q] = (AT)__ldcs(wb + 3 * e);
-                w1[q] = (AT)__ldcs(wb + 3 * e + 1);
-                wl[q] = (AT)__ldcs(wb + 3 * e + 2);
+                w0[q] = __ldcs(wb + 3 * e);
+                w1[q] = __ldcs(wb + 3 * e + 1);
+                wl[q] = __ldcs(wb + 3 * e + 2);
             } else {
                 cj[q] = -1;
             }
         }
+    };
+    if (rs < re) load_batch(rs);
+    const AT ui = live ? (AT)su[i] : (AT)0, vi = live ? (AT)sv[i] : (AT)0;
+    AT fu = 0, fv = 0;
+    for (int64_t base = rs; base < re; base += (int64_t)G * UNR) {
+        if (base != rs) load_batch(base);
 #pragma unroll
         for (int q = 0; q < UNR; q++) {
             if (cj[q] >= 0) {
-                const AT du = (AT)su[cj[q]] - ui, dv = (AT)sv[cj[q]] - vi;
-                s[0] = fma(du, w0[q], s[0]);
-                s[1] = fma(du, w1[q], s[1]);
-                s[2] = fma(du, wl[q], s[2]);
-                s[3] = fma(dv, w0[q], s[3]);
-                s[4] = fma(dv, w1[q], s[4]);
-                s[5] = fma(dv, wl[q], s[5]);
+                const AT c = fma(-vi, (AT)w1[q], fma(-ui, (AT)w0[q], (AT)wl[q]));
+                fu = fma((AT)su[cj[q]] - ui, c, fu);
+                fv = fma((AT)sv[cj[q]] - vi, c, fv);
             }
         }
     }
-    for (int o = G >> 1; o > 0; o >>= 1)
-#pragma unroll
-        for (int t = 0; t < 6; t++) s[t] += __shfl_xor_sync(0xffffffffu, s[t], o);
+    for (int o = G >> 1; o > 0; o >>= 1) {
+        fu += __shfl_xor_sync(0xffffffffu, fu, o);
+        fv += __shfl_xor_sync(0xffffffffu, fv, o);
+    }
     if (!live || lane != 0) return;
-    const bool fz = frozen && frozen[i];
-    const FT Fu = fz ? (FT)0 : (FT)(-(ui * s[0] + vi * s[1]) + s[2]);
-    const FT Fv = fz ? (FT)0 : (FT)(-(ui * s[3] + vi * s[4]) + s[5]);
-    const FT u0 = u[i], v0 = v[i];
-    switch (stage) {
-    case 0:
-        acc[i] = u0 + dt * (FT)(1.0 / 6.0) * Fu;
-        acc[n + i] = v0 + dt * (FT)(1.0 / 6.0) * Fv;
-        nxt[i] = u0 + dt * (FT)0.5 * Fu;
-        nxt[n + i] = v0 + dt * (FT)0.5 * Fv;
-        break;
-    case 1:
-        acc[i] = acc[i] + dt * (FT)(1.0 / 3.0) * Fu;
-        acc[n + i] = acc[n + i] + dt * (FT)(1.0 / 3.0) * Fv;
-        nxt[i] = u0 + dt * (FT)0.5 * Fu;
-        nxt[n + i] = v0 + dt * (FT)0.5 * Fv;
-        break;
-    case 2:
-        acc[i] = acc[i] + dt * (FT)(1.0 / 3.0) * Fu;
-        acc[n + i] = acc[n + i] + dt * (FT)(1.0 / 3.0) * Fv;
-        nxt[i] = u0 + dt * Fu;
-        nxt[n + i] = v0 + dt * Fv;
-        break;
-    default:
-        u[i] = acc[i] + dt * (FT)(1.0 / 6.0) * Fu;
-        v[i] = acc[n + i] + dt * (FT)(1.0 / 6.0) * Fv;
-        break;
+    const float Fu = fixed ? 0.0f : (float)fu;
+    const float Fv = fixed ? 0.0f : (float)fv;
+    if (stage == 3) {
+        u[i] = acc[i] + ca * Fu;
+        v[i] = acc[n + i] + ca * Fv;
+        return;
+    }
+    const float u0 = u[i], v0 = v[i];
+    acc[i] = (stage == 0 ? u0 : acc[i]) + ca * Fu;
+    acc[n + i] = (stage == 0 ? v0 : acc[n + i]) + ca * Fv;
+    nxt[i] = u0 + cnx * Fu;
+    nxt[n + i] = v0 + cnx * Fv;
+}
+
+// The same on double fields (see k_rk4_run)
+template <class VT>
+__global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellView S, const VT *__restrict__ wb, double *u,
+                                                               double *v, double *acc, double *sa, double *sb,
+                                                               const uint8_t *__restrict__ frozen, int64_t nsteps,
+                                                               RkCoef rk, GridSync sync)
+{
+    constexpr int U = RUN_U / 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t s0, s1;
+    slice_share(S.n_slices, s0, s1);
+    GridBarrier bar{sync};
+    const SellLane first(s0 + warp < s1 ? s0 + warp : S.n_slices, lane, n, S);
+    SliceBatch<U, 3, VT> nx;
+    nx.load(first, lane, 0, S, wb);
+    for (int64_t it = 0; it < 4 * nsteps; it++) {
+        const int stage = (int)(it & 3);
+        const double *su = stage == 0 ? u : stage == 2 ? sb : sa, *sv = stage == 0 ? v : su + n;
+        for (int64_t slice = s0 + warp; slice < s1; slice += RUN_THREADS / 32) {
+            SellLane l = first;
+            if (slice != s0 + warp) {
+                l = SellLane(slice, lane, n, S);
+                nx.load(l, lane, 0, S, wb);
+            }
+            const int64_t i = l.i;
+            const double ui = i >= 0 ? su[i] : 0.0, vi = i >= 0 ? sv[i] : 0.0;
+            const bool row = i >= 0 && l.h == 0;
+            const bool fixed = row && frozen && frozen[i];
+            double *const field[2] = {u, v};
+            double u0[2] = {0.0, 0.0}, a0[2] = {0.0, 0.0};
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                if (row && stage != 3) u0[c] = field[c][i];
+                if (row && stage != 0) a0[c] = acc[c * n + i];
+            }
+            double fu = 0.0, fv = 0.0;
+            for (int k0 = 0; k0 < l.steps; k0 += U) {
+                double x[U], y[U];
+                const SliceBatch<U, 3, VT> b = nx;
+#pragma unroll
+                for (int q = 0; q < U; q++)
+                    if (b.c[q] >= 0) {
+                        x[q] = su[b.c[q]];
+                        y[q] = sv[b.c[q]];
+                    }
+                if (k0 + U < l.steps) nx.load(l, lane, k0 + U, S, wb);
+#pragma unroll
+                for (int q = 0; q < U; q++)
+                    if (b.c[q] >= 0) {
+                        const double c = fma(-vi, (double)b.w[q][1], fma(-ui, (double)b.w[q][0], (double)b.w[q][2]));
+                        fu = fma(x[q] - ui, c, fu);
+                        fv = fma(y[q] - vi, c, fv);
+                    }
+            }
+            for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) {
+                fu += __shfl_xor_sync(0xffffffffu, fu, o);
+                fv += __shfl_xor_sync(0xffffffffu, fv, o);
+            }
+            if (!row) continue;
+            const double F[2] = {fixed ? 0.0 : fu, fixed ? 0.0 : fv};
+            double *const nxt = stage == 1 ? sb : sa;
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                if (stage == 3) {
+                    field[c][i] = a0[c] + rk.sixth * F[c];
+                    continue;
+                }
+                acc[c * n + i] = stage == 0 ? u0[c] + rk.sixth * F[c] : a0[c] + rk.third * F[c];
+                nxt[c * n + i] = u0[c] + (stage == 2 ? rk.one : rk.half) * F[c];
+            }
+        }
+        if (it + 1 == 4 * nsteps) break;
+        nx.load(first, lane, 0, S, wb);
+        if (!bar.wait()) return;
     }
 }
 
-template <class FT, class WT>
-cudaError_t launch_burg_stage_shape(labfm_ctx *ctx, Shape sh, const FT *su, const FT *sv, FT *u, FT *v, FT *acc,
-                                    FT *nxt, const uint8_t *frozen, int stage, double dt, cudaStream_t s)
+template <class WT>
+cudaError_t launch_burg_stage_csr(labfm_ctx *ctx, Shape sh, const float *su, const float *sv, float *u, float *v,
+                                  float *acc, float *nxt, const uint8_t *frozen, int stage, double dt, cudaStream_t s)
 {
     const unsigned blocks = blocks_for(ctx->n, sh.G);
     auto args = [&](auto kern) {
         kern<<<blocks, APPLY_THREADS, 0, s>>>(ctx->n, ctx->row_ptr.as<int64_t>(), ctx->col.as<int32_t>(),
-                                              ctx->wburg.as<WT>(), su, sv, u, v, acc, nxt, frozen, stage, (FT)dt,
-                                              log2_of(sh.G));
+                                              ctx->wburg.as<WT>(), su, sv, u, v, acc, nxt, frozen, stage,
+                                              stage_ca(stage, dt), stage_cn(stage, dt), log2_of(sh.G));
     };
     switch (sh.UNR) {
-    case 2: args(k_burgers_stage<FT, WT, 2>); break;
-    case 8: args(k_burgers_stage<FT, WT, 8>); break;
-    default: args(k_burgers_stage<FT, WT, 4>); break;
+    case 2: args(k_burgers_stage_csr<WT, 2>); break;
+    case 8: args(k_burgers_stage_csr<WT, 8>); break;
+    default: args(k_burgers_stage_csr<WT, 4>); break;
     }
     return cudaGetLastError();
 }
 
-template <class FT, class WT>
-cudaError_t enqueue_burgers(labfm_ctx *ctx, void *u_, void *v_, int fdt, double dt, int64_t nsteps,
-                            const uint8_t *frozen, cudaStream_t s)
+template <class WT>
+cudaError_t enqueue_burgers_csr(labfm_ctx *ctx, void *u_, void *v_, double dt, int64_t nsteps, const uint8_t *frozen,
+                                cudaStream_t s)
 {
     const int64_t n = ctx->n;
-    FT *u = (FT *)u_, *v = (FT *)v_;
-    FT *acc = ctx->bu_acc.as<FT>(), *sa = ctx->bu_stage_a.as<FT>(), *sb = ctx->bu_stage_b.as<FT>();
+    float *u = (float *)u_, *v = (float *)v_, *acc = ctx->bu_acc.as<float>();
+    float *sa = ctx->bu_stage_a.as<float>(), *sb = ctx->bu_stage_b.as<float>();
     // tune on stage 0, which reads u and v and writes only the work buffers
     Shape sh;
     cudaError_t e = autotune(
-        ctx, tune_key(ctx, 3, 2, fdt, ctx->wdtype), 1,
-        [&](Shape sp) {
-            return launch_burg_stage_shape<FT, WT>(ctx, sp, u, v, u, v, acc, sa, frozen, 0, dt, ctx->stream);
-        },
-        sh);
+        ctx, tune_key(ctx, 3, 2, LABFM_F32, ctx->wdtype), 1,
+        [&](Shape sp) { return launch_burg_stage_csr<WT>(ctx, sp, u, v, u, v, acc, sa, frozen, 0, dt, ctx->stream); }, sh);
     if (e != cudaSuccess) return e;
     for (int64_t st = 0; st < nsteps; st++) {
-        if ((e = launch_burg_stage_shape<FT, WT>(ctx, sh, u, v, u, v, acc, sa, frozen, 0, dt, s)) != cudaSuccess)
-            return e;
-        if ((e = launch_burg_stage_shape<FT, WT>(ctx, sh, sa, sa + n, u, v, acc, sb, frozen, 1, dt, s)) !=
-            cudaSuccess)
-            return e;
-        if ((e = launch_burg_stage_shape<FT, WT>(ctx, sh, sb, sb + n, u, v, acc, sa, frozen, 2, dt, s)) !=
-            cudaSuccess)
-            return e;
-        if ((e = launch_burg_stage_shape<FT, WT>(ctx, sh, sa, sa + n, u, v, acc, (FT *)nullptr, frozen, 3, dt, s)) !=
-            cudaSuccess)
-            return e;
+        if ((e = launch_burg_stage_csr<WT>(ctx, sh, u, v, u, v, acc, sa, frozen, 0, dt, s)) != cudaSuccess) return e;
+        if ((e = launch_burg_stage_csr<WT>(ctx, sh, sa, sa + n, u, v, acc, sb, frozen, 1, dt, s)) != cudaSuccess) return e;
+        if ((e = launch_burg_stage_csr<WT>(ctx, sh, sb, sb + n, u, v, acc, sa, frozen, 2, dt, s)) != cudaSuccess) return e;
+        if ((e = launch_burg_stage_csr<WT>(ctx, sh, sa, sa + n, u, v, acc, nullptr, frozen, 3, dt, s)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-cudaError_t enqueue_burgers_dt(labfm_ctx *ctx, int fdt, void *u, void *v, double dt, int64_t nsteps,
-                               const uint8_t *frozen, cudaStream_t s)
+cudaError_t enqueue_burgers_dt(labfm_ctx *ctx, void *u, void *v, double dt, int64_t nsteps, const uint8_t *frozen,
+                               cudaStream_t s)
 {
-    if (fdt == LABFM_F64)
-        return ctx->wdtype == LABFM_F64 ? enqueue_burgers<double, double>(ctx, u, v, fdt, dt, nsteps, frozen, s)
-                                        : enqueue_burgers<double, float>(ctx, u, v, fdt, dt, nsteps, frozen, s);
-    return ctx->wdtype == LABFM_F64 ? enqueue_burgers<float, double>(ctx, u, v, fdt, dt, nsteps, frozen, s)
-                                    : enqueue_burgers<float, float>(ctx, u, v, fdt, dt, nsteps, frozen, s);
+    return ctx->wdtype == LABFM_F64 ? enqueue_burgers_csr<double>(ctx, u, v, dt, nsteps, frozen, s)
+                                    : enqueue_burgers_csr<float>(ctx, u, v, dt, nsteps, frozen, s);
 }
 
 }  // namespace
@@ -748,30 +937,55 @@ labfm_status run_step_burgers(labfm_ctx *ctx, const double *beta, void *u, void 
     cudaStream_t s = ctx->stream;
     const int64_t n = ctx->n, nnz = ctx->nnz;
     const size_t fsz = fdt == LABFM_F64 ? 8 : 4, wsz = ctx->wdtype == LABFM_F64 ? 8 : 4;
-    bool same_beta = ctx->wburg_valid;
+    const bool sliced = fdt == LABFM_F64;
+    if (sliced) {
+        labfm_status st = ensure_sell(ctx);
+        if (st != LABFM_OK) return st;
+    }
+    bool same_beta = ctx->wburg_valid && ctx->wburg_sliced == sliced;
     for (int d = 2; d < ctx->n_ops && same_beta; d++) same_beta = (ctx->beta_burg[d] == beta[d]);
     if (!same_beta) {
-        LABFM_CUDA_TRY(ctx, ctx->wburg.reserve(3 * wsz * (nnz > 0 ? nnz : 1)));
-        double b[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int d = 2; d < ctx->n_ops; d++) b[d] = beta[d];
+        const int64_t entries = sliced ? ctx->sell.places : nnz;
+        LABFM_CUDA_TRY(ctx, ctx->wburg.reserve(3 * wsz * (size_t)(entries > 0 ? entries : 1)));
+        Beta b{};
+        for (int d = 2; d < ctx->n_ops; d++) b.v[d] = beta[d];
         if (nnz > 0) {
-            const unsigned blocks = (unsigned)std::min<int64_t>((nnz + 255) / 256, (int64_t)ctx->num_sms * 32);
-            if (ctx->wdtype == LABFM_F64)
-                k_burg_combine<double><<<blocks, 256, 0, s>>>(nnz, ctx->n_ops, ctx->w.as<double>(),
-                                                               ctx->wburg.as<double>(), b[2], b[3], b[4], b[5], b[6],
-                                                               b[7]);
-            else
-                k_burg_combine<float><<<blocks, 256, 0, s>>>(nnz, ctx->n_ops, ctx->w.as<float>(),
-                                                              ctx->wburg.as<float>(), b[2], b[3], b[4], b[5], b[6],
-                                                              b[7]);
+            auto combine = [&](auto wt) {
+                using WT = decltype(wt);
+                if (sliced)
+                    k_burg_combine_sliced<WT><<<slice_blocks(ctx, APPLY_THREADS), APPLY_THREADS, 0, s>>>(
+                        n, sell_view(ctx->sell), ctx->row_ptr.as<int64_t>(), ctx->n_ops, ctx->w.as<WT>(),
+                        ctx->wburg.as<WT>(), b);
+                else
+                    k_burg_combine<WT><<<(unsigned)std::min<int64_t>((nnz + 255) / 256, (int64_t)ctx->num_sms * 32), 256, 0,
+                                         s>>>(nnz, ctx->n_ops, ctx->w.as<WT>(), ctx->wburg.as<WT>(), b);
+            };
+            if (ctx->wdtype == LABFM_F64) combine(0.0);
+            else combine(0.0f);
             LABFM_CUDA_TRY(ctx, cudaGetLastError());
         }
+        ctx->wburg_sliced = sliced;
         for (int d = 2; d < ctx->n_ops; d++) ctx->beta_burg[d] = beta[d];
         ctx->wburg_valid = true;
     }
     LABFM_CUDA_TRY(ctx, ctx->bu_acc.reserve(2 * fsz * n));
     LABFM_CUDA_TRY(ctx, ctx->bu_stage_a.reserve(2 * fsz * n));
     LABFM_CUDA_TRY(ctx, ctx->bu_stage_b.reserve(2 * fsz * n));
+
+    if (sliced) {
+        double *uu = (double *)u, *vv = (double *)v, *acc = ctx->bu_acc.as<double>();
+        double *sa = ctx->bu_stage_a.as<double>(), *sb = ctx->bu_stage_b.as<double>();
+        const SellView S = sell_view(ctx->sell);
+        LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
+        cudaError_t e = enqueue_runs(ctx, nsteps, [&](int64_t steps) {
+            return ctx->wdtype == LABFM_F64
+                       ? launch_run(ctx, S.n_slices, k_burgers_run<double>, n, S, ctx->wburg.as<double>(), uu, vv, acc, sa, sb,
+                                    frozen, steps, rk_coef(dt), grid_sync(ctx))
+                       : launch_run(ctx, S.n_slices, k_burgers_run<float>, n, S, ctx->wburg.as<float>(), uu, vv, acc, sa, sb,
+                                    frozen, steps, rk_coef(dt), grid_sync(ctx));
+        });
+        return e == cudaSuccess ? LABFM_OK : cuda_fail(ctx, e, "Burgers run");
+    }
 
     StepGraph &g = ctx->graph_burgers;
     const bool same = g.exec && g.u == u && g.v == v && g.frozen == frozen && g.dtype == fdt && g.dt == dt &&
@@ -785,13 +999,13 @@ labfm_status run_step_burgers(labfm_ctx *ctx, const double *beta, void *u, void 
         }
         LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));  // the combined weights, before the capture stream reads them
         {
-            cudaError_t te = enqueue_burgers_dt(ctx, fdt, u, v, dt, 0, frozen, s);  // tuning only
+            cudaError_t te = enqueue_burgers_dt(ctx, u, v, dt, 0, frozen, s);  // tuning only
             if (te != cudaSuccess) return cuda_fail(ctx, te, "Burgers stage tuning");
             LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
         }
         cudaGraph_t graph = nullptr;
         LABFM_CUDA_TRY(ctx, cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = enqueue_burgers_dt(ctx, fdt, u, v, dt, nsteps, frozen, ctx->capture_stream);
+        cudaError_t e = enqueue_burgers_dt(ctx, u, v, dt, nsteps, frozen, ctx->capture_stream);
         cudaError_t e2 = cudaStreamEndCapture(ctx->capture_stream, &graph);
         if (e != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);

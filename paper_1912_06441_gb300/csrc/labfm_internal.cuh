@@ -29,6 +29,22 @@ struct DevBuf {
     template <class T> T *as() const { return static_cast<T *>(ptr); }
 };
 
+// The sliced layout of the stencils (see sell.cu), built once per stencil search by the first call that reads it.
+struct Sell {
+    bool valid = false;
+    int lg_l = 0;          // lanes per node, log2
+    int64_t n_slices = 0;
+    int64_t places = 0;    // entries with the empty places
+    DevBuf off, col, steps;
+    void release()
+    {
+        valid = false;
+        off.release();
+        col.release();
+        steps.release();
+    }
+};
+
 // Cached CUDA graph of an RK4 run, with everything its launches were recorded with: it is
 // replayed only while all of these are unchanged.
 struct StepGraph {
@@ -47,6 +63,8 @@ struct StepGraph {
 
 }  // namespace labfm
 
+constexpr int LABFM_GAVE_UP = 1000;  // byte of the context's host words
+
 struct labfm_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -60,6 +78,8 @@ struct labfm_ctx {
     double lo[2] = {0, 0}, hi[2] = {0, 0};
     labfm::DevBuf node_xy, node_h;  // context copies of the node positions and h
     labfm::DevBuf row_ptr, col;
+    labfm::Sell sell;  // of these stencils, for the FP64 products
+    labfm::DevBuf sync_buf;  // barrier counter of the cooperative runs
     // scratch of the neighbour search
     labfm::DevBuf cell_of, cell_count, cell_start, cell_nodes, counts, scan_tmp, misc;
 
@@ -92,17 +112,19 @@ struct labfm_ctx {
     bool grad01 = false;  // operators 0 and 1 of the built weights are d/dx and d/dy
     labfm::DevBuf wburg, bu_acc, bu_stage_a, bu_stage_b;
     double beta_burg[LABFM_MAX_OPS] = {0};
-    bool wburg_valid = false;
+    bool wburg_valid = false, wburg_sliced = false;
     labfm::StepGraph graph_burgers;
 
-    // implicit solves (BiCGStab): operator weights as one FP64 stream, nine vectors, partial sums
-    labfm::DevBuf sol_w, sol_vec, sol_part, sol_gmap, sol_wg;  // sol_gmap/sol_wg: Neumann ghost rows
+    // implicit solves (BiCGStab): operator weights in the sliced layout, ten vectors, partial sums, and for Neumann
+    // ghost rows their map and the layout with their parents' stencils
+    labfm::DevBuf sol_w, sol_vec, sol_part, sol_gmap;
+    labfm::Sell sell_ghost;
 
     // launch shapes chosen by the apply / RK4 autotuner:
     // key (kind, n_ops, dtypes, size class of n, mean stencil size) -> (G << 8) | UNR
     std::unordered_map<uint64_t, uint32_t> tuned;
 
-    // pinned host word for status read-back
+    // pinned host words for status read-back; at byte LABFM_GAVE_UP: a barrier of an earlier run gave up
     void *host_small = nullptr;
 };
 
@@ -152,6 +174,138 @@ struct MixedArgsPublic {
 cudaError_t launch_build_mixed(int k, const MixedArgsPublic &p, cudaStream_t s);
 size_t mixed_scratch_bytes_per_node(int k);
 size_t mixed_record_bytes();
+
+// The sliced layout as kernels read it
+struct SellView {
+    int64_t n_slices;
+    const int64_t *off;
+    const int32_t *col;
+    int lg_l;
+};
+#ifdef __CUDACC__
+// A lane's place in the sliced layout: node i (-1: none) and entry k L + h of its row at step k
+struct SellLane {
+    int64_t i = -1, at = 0;
+    int steps = 0, h;
+    __device__ SellLane(int64_t slice, int lane, int64_t n, const SellView &S)
+    {
+        h = lane & ((1 << S.lg_l) - 1);
+        if (slice >= S.n_slices) return;
+        const int64_t node = slice * (32 >> S.lg_l) + (lane >> S.lg_l);
+        if (node < n) i = node;
+        at = S.off[slice] * 32 + lane;
+        steps = (int)(S.off[slice + 1] - S.off[slice]);
+    }
+};
+
+// A slice's steps U at a time: indices and weights (NW of them per entry, 32 places apart) in registers, loaded ahead.
+template <int U, int NW, class VT>
+struct SliceBatch {
+    int c[U];
+    VT w[U][NW];
+    // steps k0 .. k0 + U - 1 of lane l's slice; c = -1 where there is no entry
+    __device__ __forceinline__ void load(const SellLane &l, int lane, int k0, const SellView &S, const VT *__restrict__ wc)
+    {
+        const int64_t at = l.at + 32 * (int64_t)k0;
+        const VT *wr = wc + NW * (at - lane) + lane;
+#pragma unroll
+        for (int q = 0; q < U; q++) {
+            c[q] = -1;
+            if (k0 + q < l.steps) {
+                c[q] = __ldcs(S.col + at + 32 * q);
+#pragma unroll
+                for (int t = 0; t < NW; t++) w[q][t] = __ldcs(wr + 32 * (NW * q + t));
+            }
+        }
+    }
+};
+
+// Runs of many dependent sweeps over a node set (RK4 steps, solver iterations) as one cooperative launch: a block per
+// SM with an equal share of the slices, a barrier over the grid between sweeps.  Launched one by one a sweep of a small
+// set costs its launch and its uneven last blocks again as much as its sums.  What a sweep writes for others to read
+// carries no __restrict__ in the kernel: it is not constant data of the launch.
+constexpr int RUN_THREADS = 512;
+struct GridSync {
+    unsigned *count;    // device: arrivals, then 1 if a wait gave up; both 0 at the launch
+    unsigned *gave_up;  // pinned host word, set where a wait gave up
+};
+constexpr unsigned SYNC_POLLS = 1u << 21;  // about a second
+
+struct GridBarrier {
+    GridSync g;
+    unsigned target = 0;
+    // Waits until every block has arrived; what they wrote before is visible after.  false: a block did not arrive
+    // within SYNC_POLLS reads (or another block has found so): the caller returns.
+    __device__ bool wait()
+    {
+        __shared__ int s_ok;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            target += gridDim.x;
+            // (releases the whole block's writes: the barrier above orders them before it)
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.count) : "memory");
+            int ok = 1;
+            unsigned now, polls = 0;
+            while (true) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(g.count) : "memory");
+                if ((int)(now - target) >= 0) break;
+                if (++polls >= SYNC_POLLS || ((polls & 255u) == 0 && *(volatile unsigned *)(g.count + 1))) {
+                    *(volatile unsigned *)(g.count + 1) = 1u;
+                    *(volatile unsigned *)g.gave_up = 1u;
+                    __threadfence_system();
+                    ok = 0;
+                    break;
+                }
+            }
+            s_ok = ok;
+        }
+        __syncthreads();
+        return s_ok != 0;
+    }
+};
+
+// This block's share of the slices: [first, last)
+__device__ __forceinline__ void slice_share(int64_t n_slices, int64_t &first, int64_t &last)
+{
+    first = n_slices * blockIdx.x / gridDim.x;
+    last = n_slices * (blockIdx.x + 1) / gridDim.x;
+}
+
+// Cooperative launch of such a run on the context's stream
+template <class... P, class... A>
+cudaError_t launch_run(labfm_ctx *ctx, int64_t n_slices, void (*kern)(P...), A... args)
+{
+    cudaError_t e = ctx->sync_buf.reserve(256);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->sync_buf.ptr, 0, 2 * sizeof(unsigned), ctx->stream);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(n_slices < ctx->num_sms ? n_slices : ctx->num_sms));
+    cfg.blockDim = dim3(RUN_THREADS);
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+// Whether a barrier of an earlier run gave up (its results are not valid); the word is cleared.
+inline bool run_gave_up(labfm_ctx *ctx)
+{
+    volatile unsigned *w = reinterpret_cast<unsigned *>(static_cast<char *>(ctx->host_small) + LABFM_GAVE_UP);
+    const bool gave_up = *w != 0;
+    *w = 0;
+    return gave_up;
+}
+inline GridSync grid_sync(const labfm_ctx *ctx)
+{
+    return GridSync{ctx->sync_buf.as<unsigned>(), reinterpret_cast<unsigned *>(static_cast<char *>(ctx->host_small) + LABFM_GAVE_UP)};
+}
+#endif
+inline SellView sell_view(const Sell &L) { return SellView{L.n_slices, L.off.as<int64_t>(), L.col.as<int32_t>(), L.lg_l}; }
+labfm_status ensure_sell(labfm_ctx *ctx);  // ctx->sell of the current stencils
+// The layout of the stencils with the rows in gmap (>= 0: a Neumann ghost row) replaced by their parents' (gmap null: none)
+labfm_status build_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int64_t *parent);
 
 // Kernel launchers (each returns the launch error).
 labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const double *h, int periodic,

@@ -10,15 +10,17 @@
 //   rho = (r^, r); beta = (rho / rho_old)(alpha / omega); p = r + beta (p - omega v); y = M^-1 p
 //   v = A y; alpha = rho / (r^, v); s = r - alpha v; z = M^-1 s; t = A z
 //   omega = (t, s) / (t, t); x += alpha y + omega z; r = s - omega t
-// Every scalar stays in device memory: each reducing launch writes per-block partial dot
-// products and its last block (an atomic ticket) sums them in a fixed order and forms the
-// scalars, so an iteration is five launches with no host round trip (16 iterations recorded once
-// per call into a CUDA graph and replayed).  A device flag ends the iteration
-// (converged, breakdown, iteration limit); later launches see it and return at once, so the host
-// reads the flag once per chunk.
+// The iterations of a solve are one cooperative launch (up to ITERS_MAX of them, see GridBarrier): every block keeps its
+// rows, a product is followed by a barrier, and a sum over the set rides on the barrier that its iteration needs in any
+// case: each block publishes its partial sum before it and adds up all blocks' after it, in a fixed order and so to
+// the same bits everywhere.  The host reads the state once per launch.  Launched as five kernels an iteration, a
+// set of 66,000 nodes spent more than half of its time on launches and on the tails of the reducing blocks.
+//
+// The product reads the weights in the sliced layout of sell.cu: FP64 instructions bound it, one per entry there with
+// one lane a node, where four lanes of a CSR row each spent as many again on combining their sums, on the diagonal and
+// on the dot products as on their entries.
 #include <algorithm>
 #include <cmath>
-#include <vector>
 
 #include "labfm_internal.cuh"
 
@@ -26,58 +28,30 @@ namespace labfm {
 namespace {
 
 constexpr int SOLVE_THREADS = 256;
-constexpr int SOLVE_G = 4;      // lanes per node in the setup
-constexpr int SOLVE_G_MAX = 16; // the product's lanes per node are tuned in {4, 8, 16} x entries in flight {2, 4, 8}
-constexpr int SOLVE_VEC_MAX_BLOCKS = 1024;
+constexpr int SOLVE_U = 8;           // steps of a slice in flight
+constexpr int ITERS_MAX = 256;       // iterations of one launch, fewer on large sets (it holds its SMs until it ends)
+constexpr int NSLOT = 8;             // partial sums: (rhat, v) | (s, s) | (t, s), (t, t) | (rhat, r), (r, r) | true residual, (b, b)
 
 // device-resident solver state
 struct SolveState {
     double rho, rho_old, alpha, omega, beta;
     double bnorm2, rnorm2, snorm2;
     double tol2;       // (tol ||b||)^2
+    double resid2;     // ||b - A x||^2 at the end
     int done;          // 0 running, 1 converged, 2 breakdown, 3 iteration limit
     int skip;          // ||s|| already within the tolerance: omega = 0, x += alpha y, r = s
     int iters;
     int max_iter;
-    unsigned int ticket;  // blocks of the current launch that have written their partial sums
 };
 
-// Two sums over the block at once, of values held by the threads whose index is a multiple of
-// STRIDE (the others' are ignored), in a fixed order (deterministic); the results are valid in
-// warp 0.  The values go through shared memory and warp 0 alone adds them: on GB300 every FP64
-// add is scarce, and a shuffle tree in every warp would cost each warp five adds per sum, about
-// as many FP64 instructions as a product's stencil entries.  sh: 2 x SOLVE_THREADS / STRIDE.
-template <int STRIDE>
-__device__ __forceinline__ void block_sum2(double a, double b, double *sh, double &sa, double &sb)
-{
-    constexpr int NV = SOLVE_THREADS / STRIDE;
-    __syncthreads();  // sh is free (an earlier sum may still be reading it)
-    if (threadIdx.x % STRIDE == 0) {
-        sh[threadIdx.x / STRIDE] = a;
-        sh[NV + threadIdx.x / STRIDE] = b;
-    }
-    __syncthreads();
-    sa = sb = 0.0;
-    if (threadIdx.x < 32) {
-        for (int k = threadIdx.x; k < NV; k += 32) {
-            sa += sh[k];
-            sb += sh[NV + k];
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            sa += __shfl_xor_sync(0xffffffffu, sa, o);
-            sb += __shfl_xor_sync(0xffffffffu, sb, o);
-        }
-    }
-}
-
-// The scalars of the step that follows a reduction (thread 0 of the reducing block):
+// The scalars of the step that follows a reduction (thread 0 of every block, on its own copy of the state):
 //   step 0 (after the setup):       rnorm2, bnorm2, rho = rnorm2, alpha = omega = rho_old = 1, beta = 0
 //   step 2 (after v = A y):         alpha = rho / (rhat, v)
 //   step 4 (after t = A z):         skip = (s, s) <= tol2; omega = (t, s) / (t, t)
 //   step 5 (after the x, r update): rho_old = rho, rho = (rhat, r), rnorm2, iters++, convergence,
 //                                   beta of the next iteration
-// s0..s2: the sums of the three partial slots; s3: the sum of part2 (the (s, s) of phase 2).
-__device__ void form_scalars(int step, double s0, double s1, double s2, double s3, SolveState *st)
+// step 4 takes s0 = (t, s), s1 = (t, t) and snorm2 as it stands.
+__device__ void form_scalars(int step, double s0, double s1, SolveState *st)
 {
     switch (step) {
     case 0:
@@ -95,9 +69,8 @@ __device__ void form_scalars(int step, double s0, double s1, double s2, double s
         if (s0 == 0.0 || !isfinite(st->alpha)) st->done = 2;
         break;
     case 4:
-        st->snorm2 = s3;
-        st->skip = s3 <= st->tol2 ? 1 : 0;
-        st->omega = st->skip ? 0.0 : (s2 > 0.0 ? s0 / s2 : 0.0);
+        st->skip = st->snorm2 <= st->tol2 ? 1 : 0;
+        st->omega = st->skip ? 0.0 : (s1 > 0.0 ? s0 / s1 : 0.0);
         if (!isfinite(st->omega)) st->done = 2;
         break;
     default:
@@ -114,66 +87,6 @@ __device__ void form_scalars(int step, double s0, double s1, double s2, double s
         }
         break;
     }
-}
-
-// Called by every block after thread 0 has written the block's partials: the last block to
-// arrive sums all partials in a fixed order (deterministic) and forms the scalars of `step`.
-// The partials are read through L2 (__ldcg) after the other blocks' fence-then-ticket.
-__device__ void last_block_scalars(int nblk, int step, const double *part, int nblk2, const double *part2,
-                                   SolveState *st, double *sh)
-{
-    __shared__ bool s_last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(&st->ticket, 1u) == (unsigned)(nblk - 1);
-    }
-    __syncthreads();
-    if (!s_last) return;  // uniform per block
-    __threadfence();
-    double a = 0.0, b = 0.0, c = 0.0, d = 0.0;
-    for (int k = threadIdx.x; k < nblk; k += SOLVE_THREADS) {
-        a += __ldcg(part + 3 * k);
-        b += __ldcg(part + 3 * k + 1);
-        c += __ldcg(part + 3 * k + 2);
-    }
-    if (part2)
-        for (int k = threadIdx.x; k < nblk2; k += SOLVE_THREADS) d += __ldcg(part2 + 3 * k);
-    double s0, s1, s2, s3;
-    block_sum2<1>(a, b, sh, s0, s1);
-    block_sum2<1>(c, d, sh, s2, s3);
-    if (threadIdx.x == 0) {
-        form_scalars(step, s0, s1, s2, s3, st);
-        st->ticket = 0u;  // the next reduction starts from zero (it is a later launch)
-    }
-}
-
-// weights of operator d as one contiguous FP64 stream, the Jacobi scaling 1 / A_ii, and the
-// Dirichlet values into the initial guess: their residuals, search directions and updates are
-// then exactly zero, so those entries keep f_i exactly.  SOLVE_G lanes per node.
-template <class WT>
-__global__ void __launch_bounds__(SOLVE_THREADS) k_solve_setup(int64_t n, const int64_t *__restrict__ row_ptr,
-                                                              const WT *__restrict__ w, int n_ops, int op,
-                                                              double *__restrict__ wd, double *__restrict__ dinv,
-                                                              double *__restrict__ adiag,
-                                                              const uint8_t *__restrict__ dirichlet,
-                                                              const double *__restrict__ f, double *__restrict__ x)
-{
-    const int lane = threadIdx.x & (SOLVE_G - 1);
-    const int64_t i = ((int64_t)blockIdx.x * SOLVE_THREADS + threadIdx.x) / SOLVE_G;
-    double sum = 0.0;
-    if (i < n)
-        for (int64_t e = row_ptr[i] + lane; e < row_ptr[i + 1]; e += SOLVE_G) {
-            const double v = (double)w[e * n_ops + op];
-            wd[e] = v;
-            sum += v;
-        }
-    for (int o = SOLVE_G >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (i >= n || lane != 0) return;
-    const bool fixed = dirichlet && dirichlet[i];
-    if (fixed) x[i] = f[i];
-    const double a = -sum;  // A_ii
-    adiag[i] = a;
-    dinv[i] = fixed ? 1.0 : (a != 0.0 && isfinite(1.0 / a) ? 1.0 / a : 1.0);
 }
 
 // Neumann ghost rows (Sec. 5.2): gmap[ghost[g]] = g (gmap starts at -1), with the checks the host
@@ -196,248 +109,292 @@ __global__ void k_ghost_map(int64_t n, int64_t n_ghost, const int64_t *__restric
     if (atomicCAS(&gmap[gi], -1, (int)g) != -1) atomicOr(flag, 2u);
 }
 
-// goff[g] = sum over g' < g of the stencil size of parent[g'] (where ghost g's weights start in
-// the ghost weight stream), goff[n_ghost] the total; one block, each thread a contiguous run of
-// ghosts, then a scan of the per-thread sums in shared memory.  A parent out of range counts 0
-// (k_ghost_map has flagged it and the solve stops before any use).
-constexpr int GHOST_SCAN_THREADS = 1024;
-__global__ void __launch_bounds__(GHOST_SCAN_THREADS) k_ghost_offsets(int64_t n, int64_t n_ghost,
-                                                                      const int64_t *__restrict__ parent,
-                                                                      const int64_t *__restrict__ row_ptr,
-                                                                      int64_t *__restrict__ goff)
-{
-    __shared__ int64_t sh[GHOST_SCAN_THREADS];
-    const int64_t per = (n_ghost + GHOST_SCAN_THREADS - 1) / GHOST_SCAN_THREADS;
-    const int64_t g0 = (int64_t)threadIdx.x * per, g1 = g0 + per < n_ghost ? g0 + per : n_ghost;
-    auto size_of = [&](int64_t g) -> int64_t {
-        const int64_t b = parent[g];
-        return (b >= 0 && b < n) ? row_ptr[b + 1] - row_ptr[b] : 0;
-    };
-    int64_t run = 0;
-    for (int64_t g = g0; g < g1; g++) run += size_of(g);
-    sh[threadIdx.x] = run;
-    __syncthreads();
-    for (int o = 1; o < GHOST_SCAN_THREADS; o <<= 1) {  // inclusive scan (Hillis-Steele)
-        const int64_t add = threadIdx.x >= o ? sh[threadIdx.x - o] : 0;
-        __syncthreads();
-        sh[threadIdx.x] += add;
-        __syncthreads();
-    }
-    int64_t at = sh[threadIdx.x] - run;  // exclusive prefix of this thread's run
-    for (int64_t g = g0; g < g1; g++) {
-        goff[g] = at;
-        at += size_of(g);
-    }
-    if (threadIdx.x == GHOST_SCAN_THREADS - 1) goff[n_ghost] = sh[threadIdx.x];
-}
-
-// The ghost rows' weights and diagonals: row ghost[g] is n_x L^(op_x) + n_y L^(op_y) at the
-// parent b (Sec. 5.2): entry e of b's stencil gets c_e = n_x w^(op_x)_e + n_y w^(op_y)_e
-// (into wdg from goff[g]), the column of b gets -sum_e c_e (adiag), and the Jacobi scaling uses
-// the row's true diagonal, the c_e of the ghost itself within b's stencil (1 if it is absent or
-// zero).  SOLVE_G lanes per ghost; runs after k_solve_setup, whose values for these rows it
-// replaces.
-template <class WT>
-__global__ void __launch_bounds__(SOLVE_THREADS) k_solve_setup_ghost(
-    int64_t n_ghost, const int64_t *__restrict__ ghost, const int64_t *__restrict__ parent,
-    const double *__restrict__ normal, const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-    const WT *__restrict__ w, int n_ops, int op_x, int op_y, const int64_t *__restrict__ goff,
-    double *__restrict__ wdg, double *__restrict__ adiag, double *__restrict__ dinv)
-{
-    const int lane = threadIdx.x & (SOLVE_G - 1);
-    const int64_t g = ((int64_t)blockIdx.x * SOLVE_THREADS + threadIdx.x) / SOLVE_G;
-    double sum = 0.0, diag = 0.0;
-    int64_t gi = 0;
-    if (g < n_ghost) {
-        gi = ghost[g];
-        const int64_t b = parent[g];
-        const double nx = normal[2 * g], ny = normal[2 * g + 1];
-        const int64_t rs = row_ptr[b], re = row_ptr[b + 1], o = goff[g] - rs;
-        for (int64_t e = rs + lane; e < re; e += SOLVE_G) {
-            const double v = nx * (double)w[e * n_ops + op_x] + ny * (double)w[e * n_ops + op_y];
-            wdg[o + e] = v;
-            sum += v;
-            if (col[e] == gi) diag += v;
-        }
-    }
-    for (int o = SOLVE_G >> 1; o > 0; o >>= 1) {
-        sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        diag += __shfl_xor_sync(0xffffffffu, diag, o);
-    }
-    if (g >= n_ghost || lane != 0) return;
-    adiag[gi] = -sum;
-    dinv[gi] = (diag != 0.0 && isfinite(1.0 / diag)) ? 1.0 / diag : 1.0;
-}
-
-// The ghost rows as the product kernel reads them (all null when there are none)
+// The Neumann ghost rows as the kernels read them (all null when there are none)
 struct GhostRows {
     const int32_t *gmap = nullptr;   // [n]: ghost ordinal of row i, or -1
     const int64_t *parent = nullptr; // [n_ghost]
-    const int64_t *goff = nullptr;   // [n_ghost + 1]
-    const double *wdg = nullptr;     // ghost weight stream
+    const double *normal = nullptr;  // [n_ghost][2]
+    int op_x = 0, op_y = 0;
 };
 
-// out = A x with the matrix in its global form (Sec. 5.2): out_i = A_ii x_i + sum_j w_ji x_j, one
-// FP64 multiply-add per stencil entry (Dirichlet rows: out_i = x_i; a Neumann ghost row: the
-// stencil of its parent b with the ghost weights, and the diagonal term on x_b); G lanes per node
-// with UNR entries in flight per lane; fused partial dot products (a1 . out), (out . out) into
-// part[3 block + 0, 2]
-template <int G, int UNR>
-__global__ void __launch_bounds__(SOLVE_THREADS) k_solve_spmv(int64_t n, const int64_t *__restrict__ row_ptr,
-                                                             const int32_t *__restrict__ col,
-                                                             const double *__restrict__ wd,
-                                                             const double *__restrict__ adiag,
-                                                             const uint8_t *__restrict__ dirichlet,
-                                                             const double *__restrict__ x, double *__restrict__ out,
-                                                             const double *__restrict__ a1, double *__restrict__ part,
-                                                             int step, int nblk2, const double *__restrict__ part2,
-                                                             SolveState *__restrict__ st, GhostRows gr)
+// The rows in the sliced layout (a warp per slice): the weights of operator `op`, the diagonal A_ii = -sum_j w_ji, the
+// Jacobi scaling 1 / A_ii, and the Dirichlet values into the initial guess: their residuals, search
+// directions and updates are then exactly zero, so those entries keep f_i exactly.
+// A Neumann ghost row is n_x L^(op_x) + n_y L^(op_y) at its parent b (Sec. 5.2): entry e of b's stencil gets c_e = n_x
+// w^(op_x)_e + n_y w^(op_y)_e, the column of b gets -sum_e c_e (adiag), and the Jacobi scaling uses the row's true
+// diagonal, the c_e of the ghost itself within b's stencil (1 if it is absent or zero).
+template <class WT>
+__global__ void __launch_bounds__(SOLVE_THREADS) k_solve_setup(int64_t n, SellView S, const int64_t *__restrict__ row_ptr,
+                                                              const int32_t *__restrict__ col,
+                                                              const WT *__restrict__ w, int n_ops, int op, GhostRows gr,
+                                                              double *__restrict__ wd, double *__restrict__ dinv,
+                                                              double *__restrict__ adiag,
+                                                              const uint8_t *__restrict__ dirichlet,
+                                                              const double *__restrict__ f, double *__restrict__ x)
 {
-    if (st && st->done) return;
-    __shared__ double sh[2 * SOLVE_THREADS];
-    const int lane = threadIdx.x & (G - 1);
-    const int64_t i = ((int64_t)blockIdx.x * SOLVE_THREADS + threadIdx.x) / G;
-    const bool live = i < n;
-    int64_t rs = 0, re = 0, woff = 0;
-    const double *wrow = wd;
-    double xi = 0.0;  // x at the row's diagonal column (i, or a ghost row's parent)
-    if (live) {
-        int64_t src = i;
-        int gidx = -1;
-        if (gr.gmap) gidx = gr.gmap[i];
-        if (gidx >= 0) src = gr.parent[gidx];
-        rs = row_ptr[src];
-        re = row_ptr[src + 1];
-        xi = x[src];
-        if (gidx >= 0) {
-            wrow = gr.wdg;
-            woff = gr.goff[gidx] - rs;
+    const SellLane l((int64_t)blockIdx.x * (SOLVE_THREADS / 32) + (threadIdx.x >> 5), threadIdx.x & 31, n, S);
+    const int64_t i = l.i;
+    int64_t rs = 0, re = 0;
+    int g = -1;
+    double nx = 0.0, ny = 0.0;
+    if (i >= 0) {
+        int64_t r = i;
+        if (gr.gmap) g = gr.gmap[i];
+        if (g >= 0) {
+            r = gr.parent[g];
+            nx = gr.normal[2 * g];
+            ny = gr.normal[2 * g + 1];
         }
+        rs = row_ptr[r];
+        re = row_ptr[r + 1];
     }
-    double acc = 0.0;
-    for (int64_t base = rs; base < re; base += G * UNR) {
-        int cj[UNR];
-        double wv[UNR];
+    double sum = 0.0, diag = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < l.steps; k++) {
+        const int64_t e = rs + ((int64_t)k << S.lg_l) + l.h;
+        double v = 0.0;
+        if (e < re) {
+            if (g < 0) {
+                v = (double)w[e * n_ops + op];
+            } else {
+                v = nx * (double)w[e * n_ops + gr.op_x] + ny * (double)w[e * n_ops + gr.op_y];
+                if (col[e] == i) diag += v;
+            }
+        }
+        wd[l.at + 32 * (int64_t)k] = v;
+        sum += v;
+    }
+    for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        diag += __shfl_xor_sync(0xffffffffu, diag, o);
+    }
+    if (i < 0 || l.h != 0) return;
+    const bool fixed = dirichlet && dirichlet[i];
+    if (fixed) x[i] = f[i];
+    adiag[i] = -sum;  // A_ii (a ghost row: A_gb)
+    const double a = g >= 0 ? diag : -sum;
+    dinv[i] = fixed ? 1.0 : (a != 0.0 && isfinite(1.0 / a) ? 1.0 / a : 1.0);
+}
+
+struct SolveArgs {
+    int64_t n;
+    SellView S;
+    const double *wd, *adiag, *dinv, *b;
+    const uint8_t *dirichlet;
+    GhostRows gr;
+    double *x, *r, *rhat, *p, *v, *y, *s, *z, *t;
+    double *part;  // [NSLOT][blocks]
+    SolveState *st;
+    GridSync sync;
+};
+
+// One block's side of a run
+struct SolveBlock {
+    const SolveArgs &A;
+    GridBarrier bar;
+    int64_t s0, s1;  // slices
+    int64_t n0, n1;  // rows
+    int lane, warp;
+    SellLane first;
+    SliceBatch<SOLVE_U, 1, double> nx;
+
+    __device__ SolveBlock(const SolveArgs &args, int64_t s0_, int64_t s1_)
+        : A(args), bar{args.sync}, s0(s0_), s1(s1_), lane(threadIdx.x & 31), warp(threadIdx.x >> 5),
+          first(s0_ + (threadIdx.x >> 5) < s1_ ? s0_ + (threadIdx.x >> 5) : args.S.n_slices, threadIdx.x & 31, args.n, args.S)
+    {
+        n0 = s0 * (32 >> A.S.lg_l);
+        n1 = min(A.n, s1 * (32 >> A.S.lg_l));
+        nx.load(first, lane, 0, A.S, A.wd);
+    }
+
+    // A x over the block's rows with the matrix in its global form (Sec. 5.2), A_ii x_i + sum_j w_ji x_j, one FP64
+    // multiply-add per stencil entry (Dirichlet rows: x_i; a Neumann ghost row: the stencil of its parent b with the
+    // ghost weights, and the diagonal term on x_b): fn(i, (A x)_i, own_i) on one lane per row, own_i read ahead.  The first
+    // steps of the next product are on their way when it returns.
+    template <class Fn>
+    __device__ __forceinline__ void product(const double *x, const double *own, Fn fn)
+    {
+        for (int64_t slice = s0 + warp; slice < s1; slice += RUN_THREADS / 32) {
+            SellLane l = first;
+            if (slice != s0 + warp) {
+                l = SellLane(slice, lane, A.n, A.S);
+                nx.load(l, lane, 0, A.S, A.wd);
+            }
+            const int64_t i = l.i;
+            const bool row = i >= 0 && l.h == 0;
+            double xi = 0.0, ai = 0.0, oi = 0.0;
+            bool fixed = false;
+            if (row) {
+                oi = own[i];
+                int64_t src = i;
+                if (A.gr.gmap && A.gr.gmap[i] >= 0) src = A.gr.parent[A.gr.gmap[i]];
+                xi = x[src];
+                ai = A.adiag[i];
+                fixed = A.dirichlet && A.dirichlet[i];
+            }
+            double sum[2] = {0.0, 0.0};
+            for (int k0 = 0; k0 < l.steps; k0 += SOLVE_U) {
+                double xv[SOLVE_U];
+                const SliceBatch<SOLVE_U, 1, double> b = nx;
 #pragma unroll
-        for (int q = 0; q < UNR; q++) {
-            const int64_t e = base + q * G + lane;
-            cj[q] = e < re ? __ldcs(col + e) : -1;
-            wv[q] = e < re ? __ldcs(wrow + (e + woff)) : 0.0;
-        }
+                for (int q = 0; q < SOLVE_U; q++)
+                    if (b.c[q] >= 0) xv[q] = x[b.c[q]];
+                if (k0 + SOLVE_U < l.steps) nx.load(l, lane, k0 + SOLVE_U, A.S, A.wd);
 #pragma unroll
-        for (int q = 0; q < UNR; q++)
-            if (cj[q] >= 0) acc = fma(x[cj[q]], wv[q], acc);
+                for (int q = 0; q < SOLVE_U; q++)
+                    if (b.c[q] >= 0) sum[q & 1] = fma(xv[q], b.w[q][0], sum[q & 1]);
+            }
+            double acc = sum[0] + sum[1];
+            for (int o = (1 << A.S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (row) fn(i, fixed ? xi : fma(ai, xi, acc), oi);
+        }
+        nx.load(first, lane, 0, A.S, A.wd);
     }
-    for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    double d1 = 0.0, d3 = 0.0;
-    if (live && lane == 0) {
-        const double yi = (dirichlet && dirichlet[i]) ? xi : fma(adiag[i], xi, acc);
-        out[i] = yi;
-        if (a1) d1 = a1[i] * yi;
-        d3 = yi * yi;
-    }
-    if (!part) return;
-    double s1, s3;
-    block_sum2<G>(d1, d3, sh, s1, s3);
-    if (threadIdx.x == 0) {
-        part[3 * blockIdx.x] = s1;
-        part[3 * blockIdx.x + 1] = 0.0;
-        part[3 * blockIdx.x + 2] = s3;
-    }
-    if (step >= 0) last_block_scalars(gridDim.x, step, part, nblk2, part2, st, sh);
-}
 
-// the element-wise updates of one iteration, by phase
-//   0: r = b - r (r holds A x on entry), rhat = r, p = v = 0; partials (r, r), (b, b)
-//   1: p = r + beta (p - omega v); y = dinv p
-//   2: s = r - alpha v; z = dinv s; partial (s, s) into part2
-//   3: x += alpha y + omega z; r = s - omega t; partials (rhat, r), (r, r)
-__global__ void __launch_bounds__(SOLVE_THREADS) k_solve_vec(int64_t n, int phase, const double *__restrict__ b,
-                                                            double *__restrict__ x, double *__restrict__ r,
-                                                            double *__restrict__ rhat, double *__restrict__ p,
-                                                            double *__restrict__ v, double *__restrict__ y,
-                                                            double *__restrict__ s, double *__restrict__ z,
-                                                            const double *__restrict__ t,
-                                                            const double *__restrict__ dinv,
-                                                            double *__restrict__ part, SolveState *__restrict__ st)
-{
-    if (phase != 0 && st->done) return;
-    __shared__ double sh[2 * SOLVE_THREADS];
-    const double alpha = st ? st->alpha : 0.0, omega = st ? st->omega : 0.0, beta = st ? st->beta : 0.0;
-    double d1 = 0.0, d2 = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        switch (phase) {
-        case 0: {
-            const double ri = b[i] - r[i];
-            r[i] = ri;
-            rhat[i] = ri;
-            p[i] = 0.0;
-            v[i] = 0.0;
-            d1 = fma(ri, ri, d1);
-            d2 = fma(b[i], b[i], d2);
-            break;
+    // The sums of a and b over all blocks (NQ = 1: of a) through partial sums in slots q0 and q0 + 1, around a barrier; on
+    // thread 0 in out.  false: the barrier gave up.  Four warps add up a block's values, one from each of the SM's
+    // quarters: a shuffle tree in all sixteen would take the FP64 pipe longer.
+    template <int NQ>
+    __device__ bool reduce(int q0, double a, double b, double (&out)[2])
+    {
+        __shared__ double sh[NQ][RUN_THREADS], quarter[NQ][4], total[NQ];
+        __syncthreads();
+        sh[0][threadIdx.x] = a;
+        if (NQ > 1) sh[NQ - 1][threadIdx.x] = b;
+        __syncthreads();
+        if (warp < 4 * NQ) {
+            const double *v = sh[warp >> 2] + 128 * (warp & 3) + lane;
+            double w = (v[0] + v[32]) + (v[64] + v[96]);
+            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            if (lane == 0) quarter[warp >> 2][warp & 3] = w;
         }
-        case 1: {
-            const double pi = fma(beta, fma(-omega, v[i], p[i]), r[i]);
-            p[i] = pi;
-            y[i] = dinv[i] * pi;
-            break;
+        __syncthreads();
+        if (threadIdx.x < NQ) {
+            const double *q = quarter[threadIdx.x];
+            A.part[(q0 + threadIdx.x) * gridDim.x + blockIdx.x] = (q[0] + q[1]) + (q[2] + q[3]);
         }
-        case 2: {
-            const double si = fma(-alpha, v[i], r[i]);
-            s[i] = si;
-            z[i] = dinv[i] * si;
-            d1 = fma(si, si, d1);
-            break;
+        if (!bar.wait()) return false;
+        if (warp < NQ) {
+            const double *p = A.part + (q0 + warp) * gridDim.x;
+            double w0 = 0.0, w1 = 0.0;
+            for (unsigned k = lane; k < gridDim.x; k += 64) {
+                w0 += __ldcg(p + k);
+                if (k + 32 < gridDim.x) w1 += __ldcg(p + k + 32);
+            }
+            double w = w0 + w1;
+            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            if (lane == 0) total[warp] = w;
         }
-        default: {
-            x[i] = fma(omega, z[i], fma(alpha, y[i], x[i]));
-            const double ri = fma(-omega, t[i], s[i]);
-            r[i] = ri;
-            d1 = fma(rhat[i], ri, d1);
-            d2 = fma(ri, ri, d2);
-            break;
-        }
-        }
+        __syncthreads();
+        out[0] = total[0];
+        out[1] = total[NQ - 1];
+        return true;
     }
-    if (phase == 1) return;
-    double s1, s2;
-    block_sum2<1>(d1, d2, sh, s1, s2);
-    if (threadIdx.x == 0) {
-        part[3 * blockIdx.x] = s1;
-        part[3 * blockIdx.x + 1] = s2;
-        part[3 * blockIdx.x + 2] = 0.0;
+};
+
+// Up to `most` iterations; with `start` first the residual and the starting scalars of the iterate in x.  Once the
+// iteration has ended, the true residual of x too.
+__global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int start, int most)
+{
+    __shared__ SolveState st;
+    int64_t s0, s1;
+    slice_share(A.S.n_slices, s0, s1);
+    SolveBlock B(A, s0, s1);
+    if (threadIdx.x == 0) st = *A.st;
+    __syncthreads();
+    double sum[2] = {0.0, 0.0};
+    auto scalars = [&](int step) {
+        if (threadIdx.x == 0) form_scalars(step, sum[0], sum[1], &st);
+        __syncthreads();
+    };
+    if (start) {
+        double rr = 0.0, bb = 0.0;
+        B.product(A.x, A.b, [&](int64_t i, double ax, double bi) {
+            const double ri = bi - ax;
+            A.r[i] = ri;
+            A.rhat[i] = ri;
+            A.p[i] = 0.0;
+            A.v[i] = 0.0;
+            rr = fma(ri, ri, rr);
+            bb = fma(bi, bi, bb);
+        });
+        if (!B.reduce<2>(4, rr, bb, sum)) return;
+        scalars(0);
     }
-    // phase 0 forms the starting scalars, phase 3 those of the next iteration; the (s, s) of
-    // phase 2 is read with omega after t = A z
-    if (st && (phase == 0 || phase == 3)) last_block_scalars(gridDim.x, phase == 0 ? 0 : 5, part, 0, nullptr, st, sh);
-}
-
-template <int G, int UNR>
-cudaError_t launch_spmv_t(int64_t n, const int64_t *rp, const int32_t *cl, const double *wd, const double *adiag,
-                          const uint8_t *dirichlet, const double *x, double *out, const double *a1, double *part,
-                          int step, int nblk2, const double *part2, SolveState *st, const GhostRows &gr,
-                          cudaStream_t q)
-{
-    const unsigned blocks = (unsigned)((n * G + SOLVE_THREADS - 1) / SOLVE_THREADS);
-    k_solve_spmv<G, UNR><<<blocks, SOLVE_THREADS, 0, q>>>(n, rp, cl, wd, adiag, dirichlet, x, out, a1, part, step,
-                                                          nblk2, part2, st, gr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_spmv(int G, int UNR, int64_t n, const int64_t *rp, const int32_t *cl, const double *wd,
-                        const double *adiag, const uint8_t *dirichlet, const double *x, double *out, const double *a1,
-                        double *part, int step, int nblk2, const double *part2, SolveState *st, const GhostRows &gr,
-                        cudaStream_t q)
-{
-#define LABFM_SPMV_CASE(g, u)                                                                                   \
-    if (G == g && UNR == u) return launch_spmv_t<g, u>(n, rp, cl, wd, adiag, dirichlet, x, out, a1, part, step, \
-                                                       nblk2, part2, st, gr, q);
-    LABFM_SPMV_CASE(4, 2) LABFM_SPMV_CASE(4, 4) LABFM_SPMV_CASE(4, 8)
-    LABFM_SPMV_CASE(8, 2) LABFM_SPMV_CASE(8, 4) LABFM_SPMV_CASE(8, 8)
-    LABFM_SPMV_CASE(16, 2) LABFM_SPMV_CASE(16, 4) LABFM_SPMV_CASE(16, 8)
-#undef LABFM_SPMV_CASE
-    return cudaErrorInvalidValue;
+    for (int it = 0; it < most && !st.done; it++) {
+        // p = r + beta (p - omega v); y = dinv p
+        {
+            const double beta = st.beta, omega = st.omega;
+            for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
+                const double pi = fma(beta, fma(-omega, A.v[i], A.p[i]), A.r[i]);
+                A.p[i] = pi;
+                A.y[i] = A.dinv[i] * pi;
+            }
+        }
+        if (!B.bar.wait()) return;
+        // v = A y, (rhat, v) -> alpha
+        double d0 = 0.0, d1 = 0.0;
+        B.product(A.y, A.rhat, [&](int64_t i, double vi, double hi) {
+            A.v[i] = vi;
+            d0 = fma(hi, vi, d0);
+        });
+        if (!B.reduce<1>(0, d0, 0.0, sum)) return;
+        scalars(2);
+        if (st.done) break;
+        // s = r - alpha v; z = dinv s; (s, s)
+        d0 = 0.0;
+        {
+            const double alpha = st.alpha;
+            for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
+                const double si = fma(-alpha, A.v[i], A.r[i]);
+                A.s[i] = si;
+                A.z[i] = A.dinv[i] * si;
+                d0 = fma(si, si, d0);
+            }
+        }
+        if (!B.reduce<1>(1, d0, 0.0, sum)) return;
+        if (threadIdx.x == 0) st.snorm2 = sum[0];
+        // t = A z, (t, s), (t, t) -> omega
+        d0 = 0.0;
+        B.product(A.z, A.s, [&](int64_t i, double ti, double si) {
+            A.t[i] = ti;
+            d0 = fma(si, ti, d0);
+            d1 = fma(ti, ti, d1);
+        });
+        if (!B.reduce<2>(2, d0, d1, sum)) return;
+        scalars(4);
+        if (st.done) break;
+        // x += alpha y + omega z; r = s - omega t; (rhat, r), (r, r) -> rho, beta, convergence
+        d0 = d1 = 0.0;
+        {
+            const double alpha = st.alpha, omega = st.omega;
+            for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
+                A.x[i] = fma(omega, A.z[i], fma(alpha, A.y[i], A.x[i]));
+                const double ri = fma(-omega, A.t[i], A.s[i]);
+                A.r[i] = ri;
+                d0 = fma(A.rhat[i], ri, d0);
+                d1 = fma(ri, ri, d1);
+            }
+        }
+        if (!B.reduce<2>(4, d0, d1, sum)) return;
+        scalars(5);
+    }
+    if (st.done) {
+        double rr = 0.0, bb = 0.0;
+        B.product(A.x, A.b, [&](int64_t, double ax, double bi) {
+            const double ri = bi - ax;
+            rr = fma(ri, ri, rr);
+            bb = fma(bi, bi, bb);
+        });
+        if (!B.reduce<2>(6, rr, bb, sum)) return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (st.done) {
+            st.resid2 = sum[0];
+            st.bnorm2 = sum[1];
+        }
+        *A.st = st;
+    }
 }
 
 }  // namespace
@@ -447,160 +404,67 @@ labfm_status run_solve(labfm_ctx *ctx, int op, const double *f, double *phi, con
 {
     cudaStream_t s = ctx->stream;
     const int64_t n = ctx->n, nnz = ctx->nnz;
-    const int nblk_setup = (int)((n * SOLVE_G + SOLVE_THREADS - 1) / SOLVE_THREADS);
-    const int nblk_vec = (int)std::min<int64_t>((n + SOLVE_THREADS - 1) / SOLVE_THREADS, SOLVE_VEC_MAX_BLOCKS);
-    const size_t npart = 3 * (size_t)std::max<int64_t>((n * SOLVE_G_MAX + SOLVE_THREADS - 1) / SOLVE_THREADS, nblk_vec);
-    LABFM_CUDA_TRY(ctx, ctx->sol_w.reserve(sizeof(double) * (nnz > 0 ? nnz : 1)));
-    LABFM_CUDA_TRY(ctx, ctx->sol_vec.reserve(sizeof(double) * 10 * n));
-    LABFM_CUDA_TRY(ctx, ctx->sol_part.reserve(sizeof(double) * (npart + 3 * (size_t)nblk_vec) + sizeof(SolveState)));
-    double *V = ctx->sol_vec.as<double>();
-    double *dinv = V, *r = V + n, *rhat = V + 2 * n, *p = V + 3 * n, *v = V + 4 * n, *y = V + 5 * n, *sv = V + 6 * n,
-           *z = V + 7 * n, *t = V + 8 * n, *adiag = V + 9 * n;
-    double *part = ctx->sol_part.as<double>();
-    double *part2 = part + npart;  // (s, s) of phase 2, read with omega
-    SolveState *st = reinterpret_cast<SolveState *>(part2 + 3 * (size_t)nblk_vec);
-    const int64_t *rp = ctx->row_ptr.as<int64_t>();
-    const int32_t *cl = ctx->col.as<int32_t>();
-    const double *wd = ctx->sol_w.as<double>();
-    if (ctx->wdtype == LABFM_F64)
-        k_solve_setup<double><<<nblk_setup, SOLVE_THREADS, 0, s>>>(n, rp, ctx->w.as<double>(), ctx->n_ops, op,
-                                                               ctx->sol_w.as<double>(), dinv, adiag, dirichlet, f, phi);
-    else
-        k_solve_setup<float><<<nblk_setup, SOLVE_THREADS, 0, s>>>(n, rp, ctx->w.as<float>(), ctx->n_ops, op,
-                                                              ctx->sol_w.as<double>(), dinv, adiag, dirichlet, f, phi);
-    LABFM_CUDA_TRY(ctx, cudaGetLastError());
-    // Neumann ghost rows: map, checks and weight offsets, read back with one synchronisation;
-    // then their weights and diagonals replace what the setup wrote for those rows
+    // Neumann ghost rows: map and checks, read back with one synchronisation
     GhostRows gr;
     if (nm.n_ghost > 0) {
         const int64_t ng = nm.n_ghost;
         const size_t map_bytes = ((sizeof(int32_t) * (size_t)n + 15) / 16) * 16;
-        LABFM_CUDA_TRY(ctx, ctx->sol_gmap.reserve(map_bytes + sizeof(int64_t) * (size_t)(ng + 1) + 16));
+        LABFM_CUDA_TRY(ctx, ctx->sol_gmap.reserve(map_bytes + 16));
         int32_t *gmap = ctx->sol_gmap.as<int32_t>();
-        int64_t *goff = reinterpret_cast<int64_t *>(reinterpret_cast<char *>(gmap) + map_bytes);
-        unsigned int *gflag = reinterpret_cast<unsigned int *>(goff + ng + 1);
+        unsigned int *gflag = reinterpret_cast<unsigned int *>(reinterpret_cast<char *>(gmap) + map_bytes);
         LABFM_CUDA_TRY(ctx, cudaMemsetAsync(gmap, 0xff, sizeof(int32_t) * (size_t)n, s));  // -1
         LABFM_CUDA_TRY(ctx, cudaMemsetAsync(gflag, 0, sizeof(unsigned int), s));
         k_ghost_map<<<(unsigned)((ng + 255) / 256), 256, 0, s>>>(n, ng, nm.ghost, nm.parent, nm.normal, dirichlet,
                                                                  gmap, gflag);
-        k_ghost_offsets<<<1, GHOST_SCAN_THREADS, 0, s>>>(n, ng, nm.parent, rp, goff);
         LABFM_CUDA_TRY(ctx, cudaGetLastError());
-        unsigned long long *hs = (unsigned long long *)ctx->host_small;
-        LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(&hs[0], goff + ng, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(&hs[1], gflag, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
+        unsigned int *hs = (unsigned int *)ctx->host_small;
+        LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(hs, gflag, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
         LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-        const unsigned flag = (unsigned)(hs[1] & 0xffffffffull);
+        const unsigned flag = *hs;
         if (flag & 1u) return fail(ctx, LABFM_ERR_ARG, "a ghost or parent index is out of range, or a ghost is its own parent");
         if (flag & 2u) return fail(ctx, LABFM_ERR_ARG, "a ghost row is listed twice");
         if (flag & 4u) return fail(ctx, LABFM_ERR_ARG, "a ghost row is also a Dirichlet row");
         if (flag & 8u) return fail(ctx, LABFM_ERR_ARG, "a ghost normal is not finite");
-        const int64_t total = (int64_t)hs[0];
-        LABFM_CUDA_TRY(ctx, ctx->sol_wg.reserve(sizeof(double) * (size_t)(total > 0 ? total : 1)));
-        double *wdg = ctx->sol_wg.as<double>();
-        const unsigned gblk = (unsigned)((ng * SOLVE_G + SOLVE_THREADS - 1) / SOLVE_THREADS);
-        if (ctx->wdtype == LABFM_F64)
-            k_solve_setup_ghost<double><<<gblk, SOLVE_THREADS, 0, s>>>(ng, nm.ghost, nm.parent, nm.normal, rp, cl,
-                                                                     ctx->w.as<double>(), ctx->n_ops, nm.op_x,
-                                                                     nm.op_y, goff, wdg, adiag, dinv);
-        else
-            k_solve_setup_ghost<float><<<gblk, SOLVE_THREADS, 0, s>>>(ng, nm.ghost, nm.parent, nm.normal, rp, cl,
-                                                                    ctx->w.as<float>(), ctx->n_ops, nm.op_x,
-                                                                    nm.op_y, goff, wdg, adiag, dinv);
-        LABFM_CUDA_TRY(ctx, cudaGetLastError());
         gr.gmap = gmap;
         gr.parent = nm.parent;
-        gr.goff = goff;
-        gr.wdg = wdg;
+        gr.normal = nm.normal;
+        gr.op_x = nm.op_x;
+        gr.op_y = nm.op_y;
+    }
+    // the layout: the stencils' own, or with ghost rows one of this call
+    Sell &L = gr.gmap ? ctx->sell_ghost : ctx->sell;
+    const labfm_status ls = gr.gmap ? build_sell(ctx, L, gr.gmap, gr.parent) : ensure_sell(ctx);
+    if (ls != LABFM_OK) return ls;
+    const SellView S = sell_view(L);
+    LABFM_CUDA_TRY(ctx, ctx->sol_w.reserve(sizeof(double) * (L.places > 0 ? L.places : 1)));
+    LABFM_CUDA_TRY(ctx, ctx->sol_vec.reserve(sizeof(double) * 10 * n));
+    LABFM_CUDA_TRY(ctx, ctx->sol_part.reserve(sizeof(double) * NSLOT * (size_t)ctx->num_sms + sizeof(SolveState)));
+    LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
+    double *V = ctx->sol_vec.as<double>();
+    double *dinv = V, *r = V + n, *rhat = V + 2 * n, *p = V + 3 * n, *v = V + 4 * n, *y = V + 5 * n, *sv = V + 6 * n,
+           *z = V + 7 * n, *t = V + 8 * n, *adiag = V + 9 * n;
+    double *part = ctx->sol_part.as<double>();
+    SolveState *st = reinterpret_cast<SolveState *>(part + NSLOT * (size_t)ctx->num_sms);
+    const double *wd = ctx->sol_w.as<double>();
+    {
+        const unsigned blocks = (unsigned)((S.n_slices + SOLVE_THREADS / 32 - 1) / (SOLVE_THREADS / 32));
+        const int64_t *rp = ctx->row_ptr.as<int64_t>();
+        const int32_t *cl = ctx->col.as<int32_t>();
+        if (ctx->wdtype == LABFM_F64)
+            k_solve_setup<double><<<blocks, SOLVE_THREADS, 0, s>>>(n, S, rp, cl, ctx->w.as<double>(), ctx->n_ops, op, gr,
+                                                                  ctx->sol_w.as<double>(), dinv, adiag, dirichlet, f, phi);
+        else
+            k_solve_setup<float><<<blocks, SOLVE_THREADS, 0, s>>>(n, S, rp, cl, ctx->w.as<float>(), ctx->n_ops, op, gr,
+                                                                 ctx->sol_w.as<double>(), dinv, adiag, dirichlet, f, phi);
+        LABFM_CUDA_TRY(ctx, cudaGetLastError());
     }
     SolveState init{};
     init.tol2 = tol * tol;
     init.max_iter = max_iter;
     LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(st, &init, sizeof(SolveState), cudaMemcpyHostToDevice, s));
-    // the product's launch shape: tuned once per problem class on this context (not while the
-    // caller's stream is being captured, nor below 4096 nodes), kept in the context's table
-    int G = 4, UNR = 4;
-    {
-        const int64_t deg = n > 0 ? (nnz + n / 2) / n : 0;
-        int64_t lg = 0;
-        while (lg < 62 && ((int64_t)1 << (lg + 1)) <= n) lg++;
-        const uint64_t key = ((uint64_t)(deg > 0xffff ? 0xffff : deg) << 40) | ((uint64_t)lg << 32) | (4ull << 24);
-        auto it = ctx->tuned.find(key);
-        if (it != ctx->tuned.end()) {
-            G = (int)(it->second >> 8);
-            UNR = (int)(it->second & 0xff);
-        } else {
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            LABFM_CUDA_TRY(ctx, cudaStreamIsCapturing(s, &cap));
-            if (cap == cudaStreamCaptureStatusNone && n >= 4096) {
-                cudaEvent_t e0, e1;
-                LABFM_CUDA_TRY(ctx, cudaEventCreate(&e0));
-                LABFM_CUDA_TRY(ctx, cudaEventCreate(&e1));
-                float best = 1e30f;
-                const int gs[3] = {4, 8, 16}, us[3] = {2, 4, 8};
-                cudaError_t te = cudaSuccess;
-                for (int gi = 0; gi < 3 && te == cudaSuccess; gi++)
-                    for (int ui = 0; ui < 3 && te == cudaSuccess; ui++) {
-                        for (int rep = 0; rep < 2 && te == cudaSuccess; rep++) {  // warm-up, then timed
-                            if (rep) cudaEventRecord(e0, s);
-                            te = launch_spmv(gs[gi], us[ui], n, rp, cl, wd, adiag, dirichlet, f, t, nullptr, part, -1,
-                                             0, nullptr, nullptr, gr, s);
-                            if (rep) cudaEventRecord(e1, s);
-                        }
-                        float ms = 0.0f;
-                        if (te == cudaSuccess) te = cudaEventSynchronize(e1);
-                        if (te == cudaSuccess) te = cudaEventElapsedTime(&ms, e0, e1);
-                        if (te == cudaSuccess && ms < best) {
-                            best = ms;
-                            G = gs[gi];
-                            UNR = us[ui];
-                        }
-                    }
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
-                if (te != cudaSuccess) return cuda_fail(ctx, te, "solver launch-shape tuning");
-                ctx->tuned[key] = ((uint32_t)G << 8) | (uint32_t)UNR;
-            }
-        }
-    }
-    // step: the scalars the last block forms (-1: none, and no gating on the state)
-    auto spmv = [&](cudaStream_t q, const double *x, double *out, const double *a1, int step) {
-        launch_spmv(G, UNR, n, rp, cl, wd, adiag, dirichlet, x, out, a1, part, step, step == 4 ? nblk_vec : 0,
-                    step == 4 ? part2 : nullptr, step >= 0 ? st : nullptr, gr, q);
-    };
-    auto vec = [&](cudaStream_t q, int phase) {
-        k_solve_vec<<<nblk_vec, SOLVE_THREADS, 0, q>>>(n, phase, f, phi, r, rhat, p, v, y, sv, z, t, dinv,
-                                                       phase == 2 ? part2 : part, st);
-    };
-    // r = b - A x, r^ = r
-    spmv(s, phi, r, nullptr, -1);
-    vec(s, 0);                                // + the starting scalars
-    LABFM_CUDA_TRY(ctx, cudaGetLastError());
-    // one chunk of iterations, recorded once per call into a CUDA graph and replayed
-    constexpr int CHUNK = 16;
-    auto enqueue_chunk = [&](cudaStream_t q) {
-        for (int it = 0; it < CHUNK; it++) {
-            vec(q, 1);                        // p, y
-            spmv(q, y, v, rhat, 2);           // v = A y, (rhat, v) -> alpha
-            vec(q, 2);                        // s, z, (s, s)
-            spmv(q, z, t, sv, 4);             // t = A z, (s, t), (t, t) -> omega
-            vec(q, 3);                        // x, r, (rhat, r), (r, r) -> rho, beta, convergence
-        }
-    };
-    if (!ctx->capture_stream)
-        LABFM_CUDA_TRY(ctx, cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking));
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    LABFM_CUDA_TRY(ctx, cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
-    enqueue_chunk(ctx->capture_stream);
-    {
-        cudaError_t e = cudaGetLastError();
-        cudaError_t e2 = cudaStreamEndCapture(ctx->capture_stream, &graph);
-        if (e == cudaSuccess) e = e2;
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-        if (graph) cudaGraphDestroy(graph);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "BiCGStab chunk capture");
-    }
-    // Chunks of iterations until the device flag ends them; then the true residual.  BiCGStab
+    const SolveArgs args{n, S, wd, adiag, dinv, f, dirichlet, gr, phi, r, rhat, p, v, y, sv, z, t, part, st, grid_sync(ctx)};
+    const int most = (int)std::max<int64_t>(8, std::min<int64_t>(ITERS_MAX, (int64_t)1000000000 / (nnz + 100000)));
+    // Launches until the state says that the iteration ended, with the true residual.  BiCGStab
     // restarts from the current iterate (r = F - A Phi, r^ = r), at most MAX_RESTARTS times
     // within max_iter in total, in two cases: the recurrence residual, which drifts from the
     // true one in finite precision, says converged while the true residual is above tol; or the
@@ -613,48 +477,29 @@ labfm_status run_solve(labfm_ctx *ctx, int op, const double *f, double *phi, con
     SolveState h{};
     int total = 0, restarts = 0;
     double resid = 0.0;
-    std::vector<double> hp(3 * (size_t)nblk_vec);
     cudaError_t le = cudaSuccess;
+    int start = 1;
     while (true) {
-        for (int it = 0; it < max_iter - total && le == cudaSuccess; it += CHUNK) {
-            le = cudaGraphLaunch(exec, s);  // the iteration limit stops the last chunk early (done = 3)
+        do {
+            le = launch_run(ctx, S.n_slices, k_solve_run, args, start, most);
+            start = 0;
             if (le == cudaSuccess) le = cudaMemcpyAsync(&h, st, sizeof(SolveState), cudaMemcpyDeviceToHost, s);
             if (le == cudaSuccess) le = cudaStreamSynchronize(s);
-            if (h.done) break;
-        }
-        if (le != cudaSuccess) break;
+            if (le != cudaSuccess) return cuda_fail(ctx, le, "BiCGStab iterations");
+            if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the solver's blocks gave up");
+        } while (!h.done);
         total += h.iters;
-        // the true residual ||b - A x|| / ||b||: t = A x, then phase 0 on scratch copies
-        spmv(s, phi, t, nullptr, -1);
-        k_solve_vec<<<nblk_vec, SOLVE_THREADS, 0, s>>>(n, 0, f, nullptr, t, sv, z, y, nullptr, nullptr, nullptr,
-                                                       nullptr, nullptr, part, nullptr);
-        le = cudaGetLastError();
-        if (le == cudaSuccess)
-            le = cudaMemcpyAsync(hp.data(), part, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, s);
-        if (le == cudaSuccess) le = cudaStreamSynchronize(s);
-        if (le != cudaSuccess) break;
-        double rr = 0.0, bb = 0.0;
-        for (int k = 0; k < nblk_vec; k++) {
-            rr += hp[3 * k];
-            bb += hp[3 * k + 1];
-        }
-        resid = std::sqrt(rr) / (bb > 0.0 ? std::sqrt(bb) : 1.0);
+        resid = std::sqrt(h.resid2) / (h.bnorm2 > 0.0 ? std::sqrt(h.bnorm2) : 1.0);
         const bool drifted = h.done == 1 && resid > tol, broke_down = h.done == 2;
         if ((drifted || broke_down) && std::isfinite(resid) && restarts < MAX_RESTARTS && total < max_iter) {
             restarts++;
             init.max_iter = max_iter - total;
-            le = cudaMemcpyAsync(st, &init, sizeof(SolveState), cudaMemcpyHostToDevice, s);
-            if (le != cudaSuccess) break;
-            spmv(s, phi, r, nullptr, -1);
-            vec(s, 0);
-            le = cudaGetLastError();
-            if (le != cudaSuccess) break;
+            LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(st, &init, sizeof(SolveState), cudaMemcpyHostToDevice, s));
+            start = 1;
             continue;
         }
         break;
     }
-    cudaGraphExecDestroy(exec);
-    if (le != cudaSuccess) return cuda_fail(ctx, le, "BiCGStab iterations");
     if (iters_out) *iters_out = total;
     if (resid_out) *resid_out = resid;
     if (h.done == 1 && std::isfinite(resid) && resid <= tol) return LABFM_OK;
