@@ -293,10 +293,8 @@ struct RkCoef {
 };
 RkCoef rk_coef(double dt) { return RkCoef{dt * (1.0 / 6.0), dt * (1.0 / 3.0), dt * 0.5, dt}; }
 
-// nsteps steps on double fields, sliced layout, one cooperative launch (see GridBarrier): a warp per slice, the next
-// RUN_U steps' indices and weights loaded before the gathers of the current ones, the first of a sweep before its
-// barrier.  A lane adds into two sums in turn, because a dependent FP64 add waits several times the pipe's time for one.
-constexpr int RUN_U = 8;
+// nsteps steps on double fields, sliced layout, one cooperative launch (see GridBarrier): a warp per slice (see SlicePipe),
+// the first steps of a sweep loaded before its barrier.  A lane adds into two sums in turn, because a dependent FP64 add waits several times the pipe's time for one.
 template <class VT>
 __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView S, const VT *__restrict__ wc, double *u,
                                                            double *acc_buf, double *sa, double *sb,
@@ -308,8 +306,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView 
     slice_share(S.n_slices, s0, s1);
     GridBarrier bar{sync};
     const SellLane first(s0 + warp < s1 ? s0 + warp : S.n_slices, lane, n, S);
-    SliceBatch<RUN_U, 1, VT> nx;
-    nx.load(first, lane, 0, S, wc);
+    SlicePipe<4, 1, 1, VT> pipe;
+    pipe.preload(first, lane, S, wc);
     for (int64_t it = 0; it < 4 * nsteps; it++) {
         const int stage = (int)(it & 3);
         const double *src = stage == 0 ? u : stage == 2 ? sb : sa;
@@ -317,7 +315,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView 
             SellLane l = first;
             if (slice != s0 + warp) {
                 l = SellLane(slice, lane, n, S);
-                nx.load(l, lane, 0, S, wc);
+                pipe.preload(l, lane, S, wc);
             }
             const int64_t i = l.i;
             const double si = i >= 0 ? src[i] : 0.0;
@@ -325,17 +323,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView 
             const bool fixed = row && frozen && frozen[i];
             const double ui = row && stage != 3 ? u[i] : 0.0, ai = row && stage != 0 ? acc_buf[i] : 0.0;
             double sum[2] = {0.0, 0.0};
-            for (int k0 = 0; k0 < l.steps; k0 += RUN_U) {
-                double x[RUN_U];
-                const SliceBatch<RUN_U, 1, VT> b = nx;
-#pragma unroll
-                for (int q = 0; q < RUN_U; q++)
-                    if (b.c[q] >= 0) x[q] = src[b.c[q]];
-                if (k0 + RUN_U < l.steps) nx.load(l, lane, k0 + RUN_U, S, wc);
-#pragma unroll
-                for (int q = 0; q < RUN_U; q++)
-                    if (b.c[q] >= 0) sum[q & 1] = fma(x[q] - si, (double)b.w[q][0], sum[q & 1]);
-            }
+            pipe.run(l, lane, S, wc, [&](int j, double(&x)[1]) { x[0] = src[j]; },
+                     [&](int q, const double(&x)[1], const VT(&w)[1]) { sum[q & 1] = fma(x[0] - si, (double)w[0], sum[q & 1]); });
             double acc = sum[0] + sum[1];
             for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (!row) continue;
@@ -348,7 +337,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView 
             (stage == 1 ? sb : sa)[i] = ui + (stage == 2 ? rk.one : rk.half) * F;
         }
         if (it + 1 == 4 * nsteps) break;
-        nx.load(first, lane, 0, S, wc);
+        pipe.preload(first, lane, S, wc);
         if (!bar.wait()) return;
     }
 }
@@ -812,14 +801,13 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellV
                                                                const uint8_t *__restrict__ frozen, int64_t nsteps,
                                                                RkCoef rk, GridSync sync)
 {
-    constexpr int U = RUN_U / 2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t s0, s1;
     slice_share(S.n_slices, s0, s1);
     GridBarrier bar{sync};
     const SellLane first(s0 + warp < s1 ? s0 + warp : S.n_slices, lane, n, S);
-    SliceBatch<U, 3, VT> nx;
-    nx.load(first, lane, 0, S, wb);
+    SlicePipe<2, 3, 2, VT> pipe;
+    pipe.preload(first, lane, S, wb);
     for (int64_t it = 0; it < 4 * nsteps; it++) {
         const int stage = (int)(it & 3);
         const double *su = stage == 0 ? u : stage == 2 ? sb : sa, *sv = stage == 0 ? v : su + n;
@@ -827,7 +815,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellV
             SellLane l = first;
             if (slice != s0 + warp) {
                 l = SellLane(slice, lane, n, S);
-                nx.load(l, lane, 0, S, wb);
+                pipe.preload(l, lane, S, wb);
             }
             const int64_t i = l.i;
             const double ui = i >= 0 ? su[i] : 0.0, vi = i >= 0 ? sv[i] : 0.0;
@@ -841,24 +829,16 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellV
                 if (row && stage != 0) a0[c] = acc[c * n + i];
             }
             double fu = 0.0, fv = 0.0;
-            for (int k0 = 0; k0 < l.steps; k0 += U) {
-                double x[U], y[U];
-                const SliceBatch<U, 3, VT> b = nx;
-#pragma unroll
-                for (int q = 0; q < U; q++)
-                    if (b.c[q] >= 0) {
-                        x[q] = su[b.c[q]];
-                        y[q] = sv[b.c[q]];
-                    }
-                if (k0 + U < l.steps) nx.load(l, lane, k0 + U, S, wb);
-#pragma unroll
-                for (int q = 0; q < U; q++)
-                    if (b.c[q] >= 0) {
-                        const double c = fma(-vi, (double)b.w[q][1], fma(-ui, (double)b.w[q][0], (double)b.w[q][2]));
-                        fu = fma(x[q] - ui, c, fu);
-                        fv = fma(y[q] - vi, c, fv);
-                    }
-            }
+            pipe.run(l, lane, S, wb,
+                     [&](int j, double(&x)[2]) {
+                         x[0] = su[j];
+                         x[1] = sv[j];
+                     },
+                     [&](int, const double(&x)[2], const VT(&w)[3]) {
+                         const double c = fma(-vi, (double)w[1], fma(-ui, (double)w[0], (double)w[2]));
+                         fu = fma(x[0] - ui, c, fu);
+                         fv = fma(x[1] - vi, c, fv);
+                     });
             for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) {
                 fu += __shfl_xor_sync(0xffffffffu, fu, o);
                 fv += __shfl_xor_sync(0xffffffffu, fv, o);
@@ -877,7 +857,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellV
             }
         }
         if (it + 1 == 4 * nsteps) break;
-        nx.load(first, lane, 0, S, wb);
+        pipe.preload(first, lane, S, wb);
         if (!bar.wait()) return;
     }
 }

@@ -220,6 +220,45 @@ struct SliceBatch {
     }
 };
 
+// A slice's sums by one lane: indices and weights are loaded two batches of U steps ahead and the values they name
+// (NX of them per entry) gathered one batch ahead.  The warps of a block go in step through the FP64 pipe, so that
+// without that they all wait for each batch's gathers at the same time (0.35 us a batch).
+template <int U, int NW, int NX, class VT>
+struct SlicePipe {
+    SliceBatch<U, NW, VT> cur, nxt;
+    __device__ __forceinline__ void preload(const SellLane &l, int lane, const SellView &S, const VT *__restrict__ wc)
+    {
+        cur.load(l, lane, 0, S, wc);
+        nxt.load(l, lane, U, S, wc);
+    }
+    // gather(j, x) and add(q, x, w) for every entry of the lane; preload comes first
+    template <class Gather, class Add>
+    __device__ __forceinline__ void run(const SellLane &l, int lane, const SellView &S, const VT *__restrict__ wc, Gather gather,
+                                        Add add)
+    {
+        double x[U][NX], xn[U][NX];
+#pragma unroll
+        for (int q = 0; q < U; q++)
+            if (cur.c[q] >= 0) gather(cur.c[q], x[q]);
+        for (int k0 = 0; k0 < l.steps; k0 += U) {
+#pragma unroll
+            for (int q = 0; q < U; q++)
+                if (nxt.c[q] >= 0) gather(nxt.c[q], xn[q]);
+            SliceBatch<U, NW, VT> far;
+            far.load(l, lane, k0 + 2 * U, S, wc);
+#pragma unroll
+            for (int q = 0; q < U; q++)
+                if (cur.c[q] >= 0) add(q, x[q], cur.w[q]);
+            cur = nxt;
+            nxt = far;
+#pragma unroll
+            for (int q = 0; q < U; q++)
+#pragma unroll
+                for (int t = 0; t < NX; t++) x[q][t] = xn[q][t];
+        }
+    }
+};
+
 // Runs of many dependent sweeps over a node set (RK4 steps, solver iterations) as one cooperative launch: a block per
 // SM with an equal share of the slices, a barrier over the grid between sweeps.  Launched one by one a sweep of a small
 // set costs its launch and its uneven last blocks again as much as its sums.  What a sweep writes for others to read

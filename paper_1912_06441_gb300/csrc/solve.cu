@@ -28,7 +28,6 @@ namespace labfm {
 namespace {
 
 constexpr int SOLVE_THREADS = 256;
-constexpr int SOLVE_U = 8;           // steps of a slice in flight
 constexpr int ITERS_MAX = 256;       // iterations of one launch, fewer on large sets (it holds its SMs until it ends)
 constexpr int NSLOT = 8;             // partial sums: (rhat, v) | (s, s) | (t, s), (t, t) | (rhat, r), (r, r) | true residual, (b, b)
 
@@ -196,7 +195,7 @@ struct SolveBlock {
     int64_t n0, n1;  // rows
     int lane, warp;
     SellLane first;
-    SliceBatch<SOLVE_U, 1, double> nx;
+    SlicePipe<4, 1, 1, double> pipe;
 
     __device__ SolveBlock(const SolveArgs &args, int64_t s0_, int64_t s1_)
         : A(args), bar{args.sync}, s0(s0_), s1(s1_), lane(threadIdx.x & 31), warp(threadIdx.x >> 5),
@@ -204,7 +203,7 @@ struct SolveBlock {
     {
         n0 = s0 * (32 >> A.S.lg_l);
         n1 = min(A.n, s1 * (32 >> A.S.lg_l));
-        nx.load(first, lane, 0, A.S, A.wd);
+        pipe.preload(first, lane, A.S, A.wd);
     }
 
     // A x over the block's rows with the matrix in its global form (Sec. 5.2), A_ii x_i + sum_j w_ji x_j, one FP64
@@ -218,7 +217,7 @@ struct SolveBlock {
             SellLane l = first;
             if (slice != s0 + warp) {
                 l = SellLane(slice, lane, A.n, A.S);
-                nx.load(l, lane, 0, A.S, A.wd);
+                pipe.preload(l, lane, A.S, A.wd);
             }
             const int64_t i = l.i;
             const bool row = i >= 0 && l.h == 0;
@@ -233,22 +232,13 @@ struct SolveBlock {
                 fixed = A.dirichlet && A.dirichlet[i];
             }
             double sum[2] = {0.0, 0.0};
-            for (int k0 = 0; k0 < l.steps; k0 += SOLVE_U) {
-                double xv[SOLVE_U];
-                const SliceBatch<SOLVE_U, 1, double> b = nx;
-#pragma unroll
-                for (int q = 0; q < SOLVE_U; q++)
-                    if (b.c[q] >= 0) xv[q] = x[b.c[q]];
-                if (k0 + SOLVE_U < l.steps) nx.load(l, lane, k0 + SOLVE_U, A.S, A.wd);
-#pragma unroll
-                for (int q = 0; q < SOLVE_U; q++)
-                    if (b.c[q] >= 0) sum[q & 1] = fma(xv[q], b.w[q][0], sum[q & 1]);
-            }
+            pipe.run(l, lane, A.S, A.wd, [&](int j, double(&xv)[1]) { xv[0] = x[j]; },
+                     [&](int q, const double(&xv)[1], const double(&w)[1]) { sum[q & 1] = fma(xv[0], w[0], sum[q & 1]); });
             double acc = sum[0] + sum[1];
             for (int o = (1 << A.S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             if (row) fn(i, fixed ? xi : fma(ai, xi, acc), oi);
         }
-        nx.load(first, lane, 0, A.S, A.wd);
+        pipe.preload(first, lane, A.S, A.wd);
     }
 
     // The sums of a and b over all blocks (NQ = 1: of a) through partial sums in slots q0 and q0 + 1, around a barrier; on
