@@ -2,9 +2,9 @@
 //
 // Cells have side >= 2 h_max, so every neighbour of a node lies in its own cell or one of
 // the 8 cells around it (with wrap-around in a periodic box).  Nodes are counting-sorted by
-// cell; one warp per node (in cell order, so the warps of a block sweep the same few cells) counts its
-// neighbours, a prefix sum gives the CSR row pointers, and a second sweep collects each row in shared
-// memory, sorts it in registers and writes it whole.  The distance test is evaluated in IEEE double
+// cell; a warp counts the neighbours of a few nodes in cell order, which share their candidates, a prefix sum gives
+// the CSR row pointers, and a second sweep collects each row in shared memory, sorts it in registers and writes it
+// whole.  The distance test is evaluated in IEEE double
 // with explicitly rounded operations (no fused multiply-add), so the result does not depend
 // on the compiler's contraction choices; a float pre-classification with a proven error bound
 // settles every candidate that is not within a thin shell at the radius (on GB300 the double
@@ -112,24 +112,6 @@ __global__ void k_cell_scatter(int64_t n, const double *__restrict__ xy, const i
     if (cell_xyf) cell_xyf[pos] = make_float2((float)x, (float)y);
 }
 
-// The up-to-3 distinct cell coordinates around c along one axis.
-__device__ __forceinline__ int axis_cells(int c, int nc, int periodic, int out[3])
-{
-    int m = 0;
-    for (int d = -1; d <= 1; d++) {
-        int v = c + d;
-        if (periodic) {
-            v = v < 0 ? v + nc : (v >= nc ? v - nc : v);
-        } else if (v < 0 || v >= nc) {
-            continue;
-        }
-        bool dup = false;
-        for (int t = 0; t < m; t++) dup |= (out[t] == v);
-        if (!dup) out[m++] = v;
-    }
-    return m;
-}
-
 // The exact distance test of Sec. 2 in IEEE double, explicitly rounded (no contraction).
 __device__ __forceinline__ bool within_exact(double qx, double qy, double xi, double yi, double R2, const Grid &g)
 {
@@ -203,116 +185,241 @@ __device__ __noinline__ void sort_long_row(int32_t *row, int cnt, int lane)
     }
 }
 
-// One sweep over the candidate cells of a node, one warp per node.  WRITE = false: count; true: write col[].
-// The candidates of a row of cells lie one behind another in cell order, so a node's up to nine cells are three runs
-// of nodes (six where the row wraps around), which the warp takes 32 candidates at a time; a ballot gives the
-// hits' places.  With a thread per node instead, the rows were sorted by insertion in global memory, which took
-// most of the search.
-// With cell_xyf, each candidate is first classified in float: r2f, the squared distance from
-// the float coordinates, differs from the double r2 by at most D = 2E(|dx_f| + |dy_f|) + 2E^2 +
-// 2^-23 r2f (E bounds the error of dx_f and dy_f); a candidate with r2f below or above
-// (2h)^2 by more than 2D + 2^-23 (2h)^2 is decided there, and only the rest (a thin shell at the
-// radius) takes the double test.  The result is the double test's, bit for bit; on GB300 the
-// double test costs FP64-pipe time per candidate, the float one does not.
+// The float pre-filter of the distance test.  r2f, the squared distance from the float coordinates, differs from the double
+// r2 by at most D = 2E s + 2E^2 + 2^-23 r2f, s = |dx_f| + |dy_f| (E bounds the error of dx_f and dy_f); a candidate with
+// r2f below or above (2h)^2 by more than 2D + 2^-22 (2h)^2 is decided (the second half of it and the last term are
+// more than the roundings of this test itself), and only the rest (a thin shell at the radius) takes the double test.
+// The result is the double test's, bit for bit; on GB300 the double test costs FP64-pipe time per candidate, the
+// float one does not.
+struct Prefilter {
+    float xi, yi, below, above;  // (2h)^2 less and plus the terms that no candidate changes
+    __device__ __forceinline__ Prefilter(float x, float y, float R2f, const Grid &g) : xi(x), yi(y)
+    {
+        const float m = 2.3841858e-7f * R2f + 4.0f * g.E * g.E;
+        below = R2f - m;
+        above = R2f + m;
+    }
+    __device__ __forceinline__ void test(float2 q, bool wrap, const Grid &g, bool &in, bool &out) const
+    {
+        float dx = q.x - xi, dy = q.y - yi;
+        if (wrap) {
+            if (dx > g.halfLf[0]) dx -= g.Lf[0];
+            else if (dx < -g.halfLf[0]) dx += g.Lf[0];
+            if (dy > g.halfLf[1]) dy -= g.Lf[1];
+            else if (dy < -g.halfLf[1]) dy += g.Lf[1];
+        }
+        const float r2 = fmaf(dx, dx, dy * dy);
+        const float t = (4.0f * g.E) * (fabsf(dx) + fabsf(dy));
+        in = fmaf(r2, 1.0f + 2.3841858e-7f, t) < below;
+        out = fmaf(r2, 1.0f - 2.3841858e-7f, -t) > above;
+    }
+};
+
+// The candidates of a cell: the up to nine cells around it.  The cells of a row lie one behind another in cell order, so
+// they are three runs of nodes, and three more where the row wraps around; q = 0 .. total - 1 numbers them.
+struct Candidates {
+    int s[6], e[6];  // run k: candidates up to e[k] are node s[k] + q in cell order
+    int total;
+    bool wrap;       // an offset may have to be wrapped (a periodic box, the cell at its edge or fewer than five cells a side)
+    __device__ __forceinline__ Candidates(int c, const Grid &g, const int64_t *__restrict__ cell_start)
+    {
+        const int nx = g.nc[0], cx = c % nx, cy = c / nx;
+        // the x range of cells, [xa, xb], and behind it the wrapped one [xc, xc] if there is one (xc < 0: none)
+        int xa = cx - 1, xb = cx + 1, xc = -1;
+        if (g.periodic && nx > 3) {
+            if (xa < 0) xc = nx - 1;
+            if (xb >= nx) xc = 0;
+        } else if (g.periodic) {
+            xa = 0;
+            xb = nx - 1;
+        }
+        xa = max(xa, 0);
+        xb = min(xb, nx - 1);
+        // the distinct cell rows around cy
+        const int ny = g.nc[1];
+        int y0 = cy - 1, y1 = cy, y2 = cy + 1, my = 3;
+        if (g.periodic) {
+            if (y0 < 0) y0 += ny;
+            if (y2 >= ny) y2 -= ny;
+            my = ny < 3 ? ny : 3;
+            if (ny < 3) {
+                y0 = 0;
+                y1 = 1;
+            }
+        } else {
+            if (y2 >= ny) my = 2;
+            if (y0 < 0) {
+                y0 = y1;
+                y1 = y2;
+                my--;
+            }
+        }
+        wrap = g.periodic && (nx < 5 || g.nc[1] < 5 || xc >= 0 || cy == 0 || cy == g.nc[1] - 1);
+        total = 0;
+#pragma unroll
+        for (int k = 0; k < 6; k++) {
+            const int a = k % 3;
+            int from = 0, len = 0;
+            if (a < my && (k < 3 || xc >= 0)) {
+                const int64_t row = (int64_t)(a == 0 ? y0 : a == 1 ? y1 : y2) * nx;
+                from = (int)cell_start[row + (k < 3 ? xa : xc)];
+                len = (int)cell_start[row + (k < 3 ? xb : xc) + 1] - from;
+            }
+            s[k] = from - total;
+            total += len;
+            e[k] = total;
+        }
+    }
+    __device__ __forceinline__ int place(int q) const  // in cell order
+    {
+        int p = s[0];
+        p = q >= e[0] ? s[1] : p;
+        p = q >= e[1] ? s[2] : p;
+        if (e[5] > e[2]) {
+            p = q >= e[2] ? s[3] : p;
+            p = q >= e[3] ? s[4] : p;
+            p = q >= e[4] ? s[5] : p;
+        }
+        return p + q;
+    }
+};
+
+// One sweep over the candidates of every node; WRITE = false: count; true: write col[].  A warp takes SWEEP_NODES
+// consecutive nodes in cell order.  The nodes of a cell share their candidates, which the warp keeps in registers (up to
+// SWEEP_REGS per lane; more are read again for every node): per node there is the test of each candidate, a ballot
+// that gives the hits' places in the row, and the sort.  (A warp per node spent most of its time finding the
+// node's cells: 180 us a count and 254 us a write at 512^2, order 8.)
+constexpr int SWEEP_NODES = 8;
+constexpr int SWEEP_REGS = 8;
 template <bool WRITE>
-__global__ void __launch_bounds__(NB_THREADS) k_sweep(int64_t n, const double *__restrict__ h, Grid g, const int32_t *__restrict__ cell_of,
-                        const int64_t *__restrict__ cell_start, const int32_t *__restrict__ cell_nodes,
-                        const double2 *__restrict__ cell_xy, const float2 *__restrict__ cell_xyf,
-                        int32_t *__restrict__ counts, const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col)
+__global__ void __launch_bounds__(NB_THREADS) k_sweep(int64_t n, const double *__restrict__ h, Grid g,
+                                                      const int32_t *__restrict__ cell_of,
+                                                      const int64_t *__restrict__ cell_start,
+                                                      const int32_t *__restrict__ cell_nodes,
+                                                      const double2 *__restrict__ cell_xy,
+                                                      const float2 *__restrict__ cell_xyf, int32_t *__restrict__ counts,
+                                                      const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col)
 {
     __shared__ int32_t s_row[WRITE ? NB_THREADS / 32 : 1][WRITE ? ROW_MAX : 1];
+    const unsigned all = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int64_t t = (int64_t)blockIdx.x * (NB_THREADS / 32) + (threadIdx.x >> 5);
-    if (t >= n) return;  // whole warps
-    const int64_t i = cell_nodes[t];
-    const double2 at = cell_xy[t];
-    const double R = 2.0 * h[i];
-    const double R2 = __dmul_rn(R, R);
+    const int64_t t0 = ((int64_t)blockIdx.x * (NB_THREADS / 32) + (threadIdx.x >> 5)) * SWEEP_NODES;
+    if (t0 >= n) return;  // whole warps
+    const int nodes = (int)min((int64_t)SWEEP_NODES, n - t0);
+    // lane k: node k of the warp
+    int my_i = 0, my_cell = -1, my_total = 0, my_cnt = 0;
+    int64_t my_base = 0;
+    double2 my_at = make_double2(0.0, 0.0);
+    double my_R2 = 0.0;
+    if (lane < nodes) {
+        my_i = cell_nodes[t0 + lane];
+        my_at = cell_xy[t0 + lane];
+        const double R = 2.0 * h[my_i];
+        my_R2 = __dmul_rn(R, R);
+        my_cell = cell_of[my_i];
+        if (WRITE) {
+            my_base = row_ptr[my_i];
+            my_total = (int)(row_ptr[my_i + 1] - my_base);
+        }
+    }
+    const float my_xf = (float)my_at.x, my_yf = (float)my_at.y, my_R2f = (float)my_R2;
     // float classification only where the float wrap cannot flip a candidate near the radius
-    const bool filt = cell_xyf != nullptr && (!g.periodic || R2 <= g.r2_wrap_max);
-    const float xif = (float)at.x, yif = (float)at.y, R2f = (float)R2;
-    const float E = g.E;
-    const int c = cell_of[i];
-    const int cx = c % g.nc[0], cy = c / g.nc[0];
-    // the x range of cells, [xa, xb], and behind it the wrapped one [xc, xc] if there is one (xc < 0: none)
-    int xa = cx - 1, xb = cx + 1, xc = -1;
-    if (g.periodic && g.nc[0] > 3) {
-        if (xa < 0) xc = g.nc[0] - 1;
-        if (xb >= g.nc[0]) xc = 0;
-    } else if (g.periodic) {
-        xa = 0;
-        xb = g.nc[0] - 1;
-    }
-    xa = max(xa, 0);
-    xb = min(xb, g.nc[0] - 1);
-    int ys[3];
-    const int my = axis_cells(cy, g.nc[1], g.periodic, ys);
-    int64_t base = 0;
-    int total = 0;  // of the row, where it is written
-    if (WRITE) {
-        base = row_ptr[i];
-        total = (int)(row_ptr[i + 1] - base);
-    }
-    int32_t *dst = nullptr;
-    if constexpr (WRITE) dst = total <= ROW_MAX ? s_row[threadIdx.x >> 5] : col + base;
-    int cnt = 0;
-    for (int part = 0; part < (xc < 0 ? 1 : 2); part++) {
-        const int x0 = part ? xc : xa, x1 = part ? xc : xb;
-        int s[3], len[3];
+    const int my_filt = cell_xyf != nullptr && (!g.periodic || my_R2 <= g.r2_wrap_max);
+    for (int k0 = 0; k0 < nodes;) {
+        const int c = __shfl_sync(all, my_cell, k0);
+        const Candidates cand(c, g, cell_start);
+        float2 cq[SWEEP_REGS];
+        int cj[SWEEP_REGS];
+        unsigned valid = 0;
+        auto load = [&](int c0) {
+            valid = 0;
 #pragma unroll
-        for (int a = 0; a < 3; a++) {
-            s[a] = len[a] = 0;
-            if (a < my) {
-                s[a] = (int)cell_start[(int64_t)ys[a] * g.nc[0] + x0];
-                len[a] = (int)cell_start[(int64_t)ys[a] * g.nc[0] + x1 + 1] - s[a];
+            for (int r = 0; r < SWEEP_REGS; r++) {
+                const int q = c0 + 32 * r + lane;
+                cq[r] = make_float2(0.0f, 0.0f);
+                cj[r] = 0;
+                if (q < cand.total) {
+                    const int p = cand.place(q);
+                    cj[r] = cell_nodes[p];
+                    if (cell_xyf) cq[r] = cell_xyf[p];
+                    valid |= 1u << r;
+                }
             }
-        }
-        const int e1 = len[0], e2 = e1 + len[1], e3 = e2 + len[2];
-        const int d1 = s[1] - e1, d2 = s[2] - e2;
-        for (int q0 = 0; q0 < e3; q0 += 32) {
-            const int q = q0 + lane;
-            const int p = q + (q < e1 ? s[0] : q < e2 ? d1 : d2);
-            bool in = false;
-            if (q < e3 && p != t) {
-                int decided = 0;  // 1: inside, 2: outside, 0: to the double test
-                if (filt) {
-                    const float2 qf = cell_xyf[p];
-                    float dxf = qf.x - xif, dyf = qf.y - yif;
-                    if (g.periodic) {
-                        if (dxf > g.halfLf[0]) dxf -= g.Lf[0];
-                        else if (dxf < -g.halfLf[0]) dxf += g.Lf[0];
-                        if (dyf > g.halfLf[1]) dyf -= g.Lf[1];
-                        else if (dyf < -g.halfLf[1]) dyf += g.Lf[1];
+        };
+        const bool kept = cand.total <= 32 * SWEEP_REGS;
+        if (kept) load(0);
+        // this cell's nodes among the warp's
+        const unsigned same = __ballot_sync(all, lane >= k0 && my_cell == c);
+        const int k1 = 32 - __clz(same);  // cell order: consecutive
+        for (int k = k0; k < k1; k++) {
+            const int i = __shfl_sync(all, my_i, k);
+            const Prefilter pre(__shfl_sync(all, my_xf, k), __shfl_sync(all, my_yf, k), __shfl_sync(all, my_R2f, k), g);
+            const bool filt = __shfl_sync(all, my_filt, k) != 0;
+            const int64_t base = WRITE ? __shfl_sync(all, my_base, k) : 0;
+            int32_t *dst = nullptr;
+            if constexpr (WRITE) dst = __shfl_sync(all, my_total, k) <= ROW_MAX ? s_row[threadIdx.x >> 5] : col + base;
+            int cnt = 0;
+            for (int c0 = 0; c0 < cand.total; c0 += 32 * SWEEP_REGS) {
+                if (!kept) load(c0);
+                unsigned hit = 0, open = 0;  // bit r: candidate 32 r + lane is inside, is to take the double test
+#pragma unroll
+                for (int r = 0; r < SWEEP_REGS; r++)
+                    if (c0 + 32 * r < cand.total) {
+                        bool in, out;
+                        pre.test(cq[r], cand.wrap, g, in, out);
+                        if (cj[r] != i) {
+                            if (in) hit |= 1u << r;
+                            else if (!out) open |= 1u << r;
+                        }
+                        if (!filt && cj[r] != i) open |= 1u << r;
                     }
-                    const float r2f = fmaf(dxf, dxf, dyf * dyf);
-                    const float D = 2.0f * E * (fabsf(dxf) + fabsf(dyf)) + 2.0f * E * E + 1.1920929e-7f * r2f;
-                    const float M = 2.0f * D + 1.1920929e-7f * R2f;
-                    decided = r2f < R2f - M ? 1 : (r2f > R2f + M ? 2 : 0);
+                hit = filt ? hit & valid : 0u;
+                open &= valid;
+                if (__any_sync(all, open != 0)) {
+                    const double xd = __shfl_sync(all, my_at.x, k), yd = __shfl_sync(all, my_at.y, k);
+                    const double R2 = __shfl_sync(all, my_R2, k);
+                    while (open) {
+                        const int r = __ffs(open) - 1;
+                        open &= open - 1;
+                        const double2 qd = cell_xy[cand.place(c0 + 32 * r + lane)];
+                        if (within_exact(qd.x, qd.y, xd, yd, R2, g)) hit |= 1u << r;
+                    }
                 }
-                if (decided) {
-                    in = decided == 1;
+                if constexpr (WRITE) {
+                    __syncwarp();
+#pragma unroll
+                    for (int r = 0; r < SWEEP_REGS; r++)
+                        if (c0 + 32 * r < cand.total) {
+                            const bool in = (hit >> r) & 1u;
+                            const unsigned hits = __ballot_sync(all, in);
+                            if (in) dst[cnt + __popc(hits & ((1u << lane) - 1u))] = cj[r];
+                            cnt += __popc(hits);
+                        }
                 } else {
-                    const double2 qd = cell_xy[p];
-                    in = within_exact(qd.x, qd.y, at.x, at.y, R2, g);
+                    cnt += (int)__reduce_add_sync(all, (unsigned)__popc(hit));
                 }
             }
-            const unsigned hits = __ballot_sync(0xffffffffu, in);
-            if (WRITE && in) dst[cnt + __popc(hits & ((1u << lane) - 1u))] = cell_nodes[p];
-            cnt += __popc(hits);
+            if constexpr (!WRITE) {
+                if (lane == k) my_cnt = cnt;
+            } else {
+                __syncwarp();
+                if (cnt <= 32) sort_row<1>(dst, cnt, lane, col + base);
+                else if (cnt <= 64) sort_row<2>(dst, cnt, lane, col + base);
+                else if (cnt <= ROW_MAX) sort_row<4>(dst, cnt, lane, col + base);
+                else sort_long_row(col + base, cnt, lane);
+                __syncwarp();  // the row is read before the next one is collected
+            }
         }
+        k0 = k1;
     }
-    if constexpr (!WRITE) {
-        if (lane == 0) counts[i] = cnt;
-    } else {
-        __syncwarp();
-        if (cnt <= 32) sort_row<1>(dst, cnt, lane, col + base);
-        else if (cnt <= 64) sort_row<2>(dst, cnt, lane, col + base);
-        else if (cnt <= ROW_MAX) sort_row<4>(dst, cnt, lane, col + base);
-        else sort_long_row(col + base, cnt, lane);
-    }
+    if (!WRITE && lane < nodes) counts[my_i] = my_cnt;
 }
 
-unsigned sweep_blocks(int64_t n) { return (unsigned)((n + NB_THREADS / 32 - 1) / (NB_THREADS / 32)); }
+unsigned sweep_blocks(int64_t n)
+{
+    const int64_t per = NB_THREADS / 32 * SWEEP_NODES;
+    return (unsigned)((n + per - 1) / per);
+}
 
 }  // namespace
 
