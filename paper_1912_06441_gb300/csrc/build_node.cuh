@@ -8,7 +8,7 @@
 // barrier), where the p x p system is small and a whole CTA would spend its time in barrier
 // latency with most threads idle.  G per order is chosen by timing (build autotuner).
 //
-// Orders 1-3 form M from X and W themselves.  Orders 4-8 use two facts about the ABFs of Sec. 3.2:
+// Orders 1-3, and 4 with the full chain rule, form M from X and W themselves.  Orders 4-8 use two facts about the ABFs of Sec. 3.2:
 //
 // (1) The weights depend only on the space that the ABFs span: w_j = W_j . Psi with sum_j X_j w_j = C is
 //     the same for every basis of that space.  The elements of degree n whose ABF is dW0/dr d^alpha|r|
@@ -77,7 +77,11 @@ struct OrderItems {
 };
 
 constexpr int BUILD_THREADS = 256;
-constexpr int MOMENT_MIN_ORDER = 4;  // orders built from moments
+constexpr int MOMENT_MIN_ORDER = 4;  // orders whose kernels differ by the form of the ABFs
+
+// Orders built from moments: from 5 up, and order 4 where every ABF is dW0/dr d^alpha|r| (256^2 nodes: 1.55 ms against
+// 2.08 from X and W; with the full chain rule, where half of the 14 elements are further functions, 2.29 against 2.13).
+__host__ __device__ constexpr bool by_moments(int K, bool chain) { return K >= (chain ? 5 : 4); }
 
 // group sizes a given order may run with
 __host__ __device__ constexpr bool group_ok(int K, int G)
@@ -89,7 +93,7 @@ namespace {
 
 // Small arrays of the node being built, in the group's share of the CTA's dynamic shared memory.
 template <int P> struct NodeShared {
-    double psi[P * MAX_OPS];     // Psi^d (Phi^d from MOMENT_MIN_ORDER up)
+    double psi[P * MAX_OPS];     // Psi^d (Phi^d where built from moments)
     double low[7 * MAX_OPS];     // the coefficients of the chain-rule elements of degrees 2 and 3
     double invpiv[P];            // 1 / pivot of each column, reused by the back substitution
     double hpow[KMAX + 1];       // h^-n
@@ -107,20 +111,37 @@ constexpr size_t SMEM_CTA = 56 * 1024;
 // A2 (x^2 - y^2), A2 x y and B2 with A2 = (W'' - W'/r) / r^2 and B2 = W'' + W'/r (the Laplacian of W0); degree 3
 // spans A3 (x^3 - 3 x y^2), A3 (3 x^2 y - y^3), B3 x and B3 y with A3 = (W''' - 3 W''/r + 3 W'/r^2) / r^3 and
 // B3 = (W''' + W''/r - W'/r^2) / r.  Their moments with the rows X run over the degrees F + 1 .. F + K of the
-// monomials for family F = 0 (B2), 1 (B3), 2 (A2), 3 (A3).
+// monomials for family F = 0 (B2), 1 (B3), 2 (A2), 3 (A3).  Only A2 (from degree 2 on) and A3 are summed over the
+// neighbours: B2 = r^2 A2 + g_1 and B3 = r^2 A3 + 2 A2 (r in units of 2h), so the moments of the other two follow from
+// those and T_1.
 constexpr int NLOWFAM = 4;
 
 // Sizes of the moment path at order K.
 template <int K, bool CH> struct Mom {
     static constexpr int P = p_of_k(K);
     // items: one monomial x^s y^t of degree d = s + t per thread, degrees 2K down to K + 1 (T_K and the
-    // highest degree of T_(d-K)), with the chain rule on down to degree 1 (the further families)
+    // highest degree of T_(d-K)); with the chain rule the further families' sums join them, see ChainItems
     static constexpr int NBASE = 3 * K * (K + 1) / 2;
-    static constexpr int NIT = CH ? K * (2 * K + 3) : NBASE;
+    static constexpr int NSLOT = 2;  // sums of a chain-rule item
+    // sums over the monomials of degree d, T's and the families'
+    static __host__ __device__ constexpr int nsum(int d)
+    {
+        int c = (d > K) + (d > K && d < 2 * K);
+        for (int f = 2; f < NLOWFAM; f++) c += d >= f + (f == 3) && d <= f + K;
+        return c;
+    }
+    static __host__ __device__ constexpr int nitem()
+    {
+        if (!CH) return NBASE;
+        int c = 0;
+        for (int d = 1; d <= 2 * K; d++) c += (d + 1) * ((nsum(d) + NSLOT - 1) / NSLOT);
+        return c;
+    }
+    static constexpr int NIT = nitem();
     static constexpr int SPAN = (NIT + 31) / 32 * 32;
-    // staged row of a neighbour: x^0 .. x^2K, y^0 .. y^2K, g_1 .. g_K, the further families
+    // staged row of a neighbour: x^0 .. x^2K, y^0 .. y^2K, g_1 .. g_K, A2, A3
     static constexpr int XO = 0, YO = 2 * K + 1, GO = 2 * YO, FO = GO + K;
-    static constexpr int LD = (FO + (CH ? NLOWFAM : 0)) | 1;  // odd: consecutive neighbours on distinct banks
+    static constexpr int LD = (FO + (CH ? 2 : 0)) | 1;  // odd: consecutive neighbours on distinct banks
     // kept of a neighbour for the weights: u, v, W0' r, the seven chain-rule functions
     static constexpr int LP = CH ? 11 : 3;
     // T_n at degrees n + 1 .. n + K, n = 1 .. K, then the further families' moments
@@ -134,7 +155,8 @@ template <int K, bool CH> struct Mom {
         return NT + K * f * (f + 1) / 2 + f * K * (K + 1) / 2;
     }
     static constexpr int NT = K * K * (K + 3) / 2 + K * K * (K + 1) / 2;
-    static constexpr int NLOW = CH ? NLOWFAM * K * (K + 1) / 2 + K * NLOWFAM * (NLOWFAM + 1) / 2 : 0;
+    // (behind the families' moments those of A2 at degree 2, which B3 needs)
+    static constexpr int NLOW = CH ? NLOWFAM * K * (K + 1) / 2 + K * NLOWFAM * (NLOWFAM + 1) / 2 + 3 : 0;
     static constexpr int PSZ = 2 * NBASE + NLOW;  // the sums of one part
     // position of (degree d, power s of x) behind the first entry of T_n (n = F for a further family)
     static __host__ __device__ constexpr int at(int n, int d, int s)
@@ -145,7 +167,58 @@ template <int K, bool CH> struct Mom {
     static __host__ __device__ constexpr int istart(int d) { return (2 * K + 1) * (2 * K + 2) / 2 - (d + 1) * (d + 2) / 2; }
 };
 static_assert(Mom<8, false>::NBASE == 108 && Mom<8, false>::NT == 640 && Mom<8, false>::toff(9) == 640, "moment counts");
-static_assert(Mom<8, true>::NIT == 152 && Mom<8, true>::NLOW == 224, "moment counts");
+static_assert(Mom<8, true>::NLOW == 227 && Mom<4, true>::NIT == 63 && Mom<5, true>::NIT == 87, "moment counts");
+
+// The chain rule's items: a monomial and up to NSLOT of the sums over it.  A warp's instruction takes the FP64 pipe's
+// time for all 32 lanes whether or not a lane needs it, and the middle degrees have up to four sums where the
+// others have one to three: in items of two sums all warps together take 6 FP64 instructions per neighbour at order 4, 9 at
+// order 5 and 12 at order 6, where an item per monomial, with all four families summed, took 12, 14 and 15.
+template <int K> struct ChainItems {
+    using M = Mom<K, true>;
+    static constexpr int NONE = 0xffff;
+    struct Item {
+        unsigned char s, t;              // powers of x and y (t = 255: no item)
+        unsigned char fn[M::NSLOT];      // the functions' places in the staged row
+        unsigned short to[M::NSLOT];     // the sums' places in a part, NONE: an unused slot
+    };
+    Item v[M::SPAN];
+};
+template <int K> constexpr ChainItems<K> make_chain_items()
+{
+    using M = Mom<K, true>;
+    ChainItems<K> T{};
+    for (int e = 0; e < M::SPAN; e++) {
+        T.v[e].t = 255;
+        for (int q = 0; q < M::NSLOT; q++) {
+            T.v[e].fn[q] = M::GO;
+            T.v[e].to[q] = ChainItems<K>::NONE;
+        }
+    }
+    int e = 0;
+    for (int d = 2 * K; d >= 1; d--)
+        for (int s = 0; s <= d; s++) {
+            int q = M::NSLOT;  // the current item's slots in use
+            e--;
+            auto put = [&](int fn, int to) {
+                if (q == M::NSLOT) {
+                    e++;
+                    q = 0;
+                    T.v[e].s = (unsigned char)s;
+                    T.v[e].t = (unsigned char)(d - s);
+                }
+                T.v[e].fn[q] = (unsigned char)fn;
+                T.v[e].to[q++] = (unsigned short)to;
+            };
+            if (d > K) put(M::GO + K - 1, M::istart(d) + s);
+            if (d > K && d < 2 * K) put(M::GO + d - K - 1, M::NBASE + M::istart(d) + s);
+            if (d == 2) put(M::FO, 2 * M::NBASE + M::NLOW - 3 + s);
+            for (int f = 2; f < NLOWFAM; f++)
+                if (d > f && d <= f + K) put(M::FO + f - 2, 2 * M::NBASE + M::loff(f) - M::NT + M::at(f, d, s));
+            e++;
+        }
+    return T;
+}
+template <int K> __device__ const ChainItems<K> chain_items = make_chain_items<K>();
 
 template <int K, int G, bool CH> struct Cfg {
     static constexpr int P = p_of_k(K);
@@ -153,12 +226,12 @@ template <int K, int G, bool CH> struct Cfg {
     static_assert(G % 32 == 0 && BUILD_THREADS % G == 0, "groups of whole warps");
     static constexpr size_t GROUP_SMEM = (SMEM_CTA / NG) / 16 * 16;
     static constexpr int LDA = P + MAX_OPS + 1;  // augmented row stride
-    static constexpr bool MOMENTS = K >= MOMENT_MIN_ORDER;
+    static constexpr bool MOMENTS = by_moments(K, CH);
     using M = Mom<K, CH>;
-    // orders 1-3: X and W of a neighbour, odd row stride (rows of consecutive neighbours on distinct banks);
+    // the others: X and W of a neighbour, odd row stride (rows of consecutive neighbours on distinct banks);
     // one tile of 1 x TN elements of M per thread
     static constexpr int LDX = (P + 3) / 4 * 4 + 1;
-    static constexpr int TN = K == 3 ? 3 : 1;
+    static constexpr int TN = K == 4 ? 7 : K == 3 ? 3 : 1;
     static constexpr int CG = (P + TN - 1) / TN;
     static_assert(MOMENTS || (P * CG <= 32 && CG * TN <= LDX), "one warp holds the tiles");
     // neighbours per staged chunk: what the group's share of the CTA's shared memory holds, <= 72
@@ -289,10 +362,8 @@ __device__ __forceinline__ void stage_neighbour(double x, double y, int rbf, dou
         keep[8] = b3 * x;
         keep[9] = b3 * y;
         if constexpr (ROW) {
-            row[M::FO] = b2;
-            row[M::FO + 1] = b3;
-            row[M::FO + 2] = a2;
-            row[M::FO + 3] = a3;
+            row[M::FO] = a2;
+            row[M::FO + 1] = a3;
         }
     }
     if constexpr (ROW) {
@@ -364,19 +435,36 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
         bool finite = true;  // of the entries of M this thread writes
         if constexpr (C::MOMENTS) {
             const double ihalf = 0.5 * ihi;
-            // this thread's item: the monomial of degree d with x^sx (d = -1: none)
+            // this thread's item: the monomial x^sx y^sy and the functions it is summed with (sy < 0: none)
             const int set = C::SETS > 1 ? tid / M::SPAN : 0;
-            int sx = C::SETS > 1 ? tid - set * M::SPAN : tid, d = 2 * K;
-            if (sx >= M::NIT || set >= C::SETS) d = -1;
-            while (d > 0 && sx > d) sx -= d-- + 1;
-            const bool hiK = d > K, hiN = d > K && d < 2 * K;
-            double accK[C::ACC], accN[C::ACC], accF[C::ACC][NLOWFAM];
+            const int item = C::SETS > 1 ? tid - set * M::SPAN : tid;
+            constexpr int NS = CH ? M::NSLOT : 2;
+            int sx = item, sy = -1, fn[NS], to[NS];
+            if (set < C::SETS && item < M::NIT) {
+                if constexpr (CH) {
+                    const auto it = chain_items<K>.v[item];
+                    sx = it.s;
+                    sy = it.t;
 #pragma unroll
-            for (int q = 0; q < C::ACC; q++) {
-                accK[q] = accN[q] = 0.0;
-#pragma unroll
-                for (int f = 0; f < NLOWFAM; f++) accF[q][f] = 0.0;
+                    for (int q = 0; q < NS; q++) {
+                        fn[q] = it.fn[q];
+                        to[q] = it.to[q];
+                    }
+                } else {
+                    int d = 2 * K;  // T_K, and up to degree 2K - 1 T_(d-K)
+                    while (sx > d) sx -= d-- + 1;
+                    sy = d - sx;
+                    fn[0] = M::GO + K - 1;
+                    to[0] = M::istart(d) + sx;
+                    fn[1] = M::GO + (d < 2 * K ? d - K - 1 : 0);
+                    to[1] = d < 2 * K ? M::NBASE + M::istart(d) + sx : ChainItems<K>::NONE;
+                }
             }
+            double acc[C::ACC][NS];
+#pragma unroll
+            for (int q = 0; q < C::ACC; q++)
+#pragma unroll
+                for (int f = 0; f < NS; f++) acc[q][f] = 0.0;
             for (int ch = 0; ch < nchunks; ch++) {
                 const int j0 = ch * NB, nj = min(NB, ni - j0);
                 if (ch > 0) gsync<G>(bar);
@@ -386,20 +474,16 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
                     stage_neighbour<K, CH, true>(dx * ihalf, dy * ihalf, A.rbf, rows + t * M::LD, keep + t * M::LP);
                 }
                 gsync<G>(bar);
-                // one product and one or two multiply-adds per item and neighbour (more at the few degrees
-                // that the further families share)
-                if (d > 0) {
-                    const double *rx = rows + M::XO + sx, *ry = rows + M::YO + (d - sx);
-                    const double *rg = rows + M::GO + (hiN ? d - K - 1 : 0);
+                // one product and NS multiply-adds per item and neighbour
+                if (sy >= 0) {
+                    const double *rx = rows + M::XO + sx, *ry = rows + M::YO + sy;
+                    const double *rf[NS];
+#pragma unroll
+                    for (int f = 0; f < NS; f++) rf[f] = rows + fn[f];
                     auto add = [&](int j, int q) {
                         const double m = rx[j * M::LD] * ry[j * M::LD];
-                        if (!CH || hiK) accK[q] = fma(m, rows[j * M::LD + M::GO + K - 1], accK[q]);
-                        if (hiN) accN[q] = fma(m, rg[j * M::LD], accN[q]);
-                        if constexpr (CH) {
 #pragma unroll
-                            for (int f = 0; f < NLOWFAM; f++)
-                                if (d > f && d <= f + K) accF[q][f] = fma(m, rows[j * M::LD + M::FO + f], accF[q][f]);
-                        }
+                        for (int f = 0; f < NS; f++) acc[q][f] = fma(m, rf[f][j * M::LD], acc[q][f]);
                     };
                     // (NB is even, so a neighbour's parity is that of its place in the chunk)
                     if constexpr (C::SETS == 2) {
@@ -417,20 +501,13 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
             }
             gsync<G>(bar);
             // the two parts' sums, over the staged rows
-            if (d > 0) {
+            if (sy >= 0) {
 #pragma unroll
                 for (int q = 0; q < C::ACC; q++) {
                     double *ps = rows + (C::SETS == 2 ? set : q) * M::PSZ;
-                    if (hiK) {
-                        ps[M::istart(d) + sx] = accK[q];
-                        ps[M::NBASE + M::istart(d) + sx] = accN[q];
-                    }
-                    if constexpr (CH) {
 #pragma unroll
-                        for (int f = 0; f < NLOWFAM; f++)
-                            if (d > f && d <= f + K)
-                                ps[2 * M::NBASE + M::loff(f) - M::NT + M::at(f, d, sx)] = accF[q][f];
-                    }
+                    for (int f = 0; f < NS; f++)
+                        if (to[f] != ChainItems<K>::NONE) ps[to[f]] = acc[q][f];
                 }
             }
             gsync<G>(bar);
@@ -456,10 +533,26 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
                     }
                 }
                 if constexpr (CH)
-                    for (int e = tid; e < M::NLOW; e += G)
+                    for (int e = M::loff(2) - M::NT + tid; e < M::NLOW; e += G)
                         T[M::NT + e] = rows[2 * M::NBASE + e] + rows[M::PSZ + 2 * M::NBASE + e];
             }
             gsync<G>(bar);
+            if constexpr (CH) {
+                // B2 at degrees 1 .. K and B3 at degrees 2 .. K + 1 (T_1 at degree 1 from T_2)
+                constexpr int NB2 = P, NB3 = P + K;
+                for (int e = tid; e < NB2 + NB3; e += G) {
+                    const bool b3 = e >= NB2;
+                    int dd = b3 ? 2 : 1, ds = b3 ? e - NB2 : e;
+                    while (ds > dd) ds -= dd++ + 1;
+                    const double *up = T + (b3 ? M::loff(3) + M::at(3, dd + 2, ds) : M::loff(2) + M::at(2, dd + 2, ds));
+                    double low;
+                    if (b3) low = 2.0 * (dd == 2 ? T[M::NT + M::NLOW - 3 + ds] : T[M::loff(2) + M::at(2, dd, ds)]);
+                    else if (dd == 1) low = T[M::toff(2) + M::at(2, 3, ds)] + T[M::toff(2) + M::at(2, 3, ds + 2)];
+                    else low = T[M::toff(1) + M::at(1, dd, ds)];
+                    T[b3 ? M::loff(1) + M::at(1, dd, ds) : M::loff(0) + M::at(0, dd, ds)] = (up[0] + up[2]) + low;
+                }
+                gsync<G>(bar);
+            }
             // M from the moments: a warp per row (a', b'), a lane per column (a, b)
             {
                 const int warp = tid >> 5, lane = tid & 31;
