@@ -196,17 +196,17 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_combine_sliced(int64_t n, Sel
 //   stage 1: acc += dt/3 F,     nxt = u + dt/2 F
 //   stage 2: acc += dt/3 F,     nxt = u + dt F
 //   stage 3: u = acc + dt/6 F
-// with ca the coefficient of acc (or u) and cn that of nxt, products formed on the host (in FP64 a product per thread
-// takes the pipe as long as a stencil entry of the warp).  The per-node update runs in the field type.
+// On double fields the coefficients are products formed on the host (in FP64 a product per thread takes the pipe as long
+// as a stencil entry of the warp).
 template <int CW, int UNR>
 __global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage_csr(int64_t n, const int64_t *__restrict__ row_ptr,
                                                              const int32_t *__restrict__ col,
                                                              const void *__restrict__ wc_raw,
                                                              const float *__restrict__ wc_lo,
-                                                             const float *src, float *__restrict__ u,
+                                                             const float *__restrict__ src, float *__restrict__ u,
                                                              float *__restrict__ acc_buf, float *__restrict__ nxt,
-                                                             const uint8_t *__restrict__ frozen, int stage, float ca,
-                                                             float cnx, int lg_g)
+                                                             const uint8_t *__restrict__ frozen, int stage, float dt,
+                                                             int lg_g)
 {
     const int2 *__restrict__ wcp = (const int2 *)wc_raw;
     const int G = 1 << lg_g;  // lanes per node, a power of two
@@ -214,11 +214,11 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage_csr(int64_t n, cons
     const int64_t i = ((int64_t)blockIdx.x * APPLY_THREADS + threadIdx.x) >> lg_g;
     const bool live = i < n;
     int64_t rs = 0, re = 0;
-    bool fixed = false;
+    float si = 0.0f;
     if (live) {
         rs = row_ptr[i];
         re = row_ptr[i + 1];
-        fixed = frozen && frozen[i];
+        si = src[i];
     }
     float acc = 0.0f;
     df accd{0.0f, 0.0f};
@@ -242,10 +242,9 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage_csr(int64_t n, cons
             }
         }
     };
-    if (rs < re) load_batch(rs);
-    const float si = live ? src[i] : 0.0f;
+    if (PIPE && rs < re) load_batch(rs);
     for (int64_t base = rs; base < re; base += (int64_t)G * UNR) {
-        if (!PIPE && base != rs) load_batch(base);
+        if (!PIPE) load_batch(base);
         int cj[UNR];
         float2 wv[UNR];
 #pragma unroll
@@ -277,14 +276,25 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_rk4_stage_csr(int64_t n, cons
         for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     }
     if (!live || lane != 0) return;
-    const float F = fixed ? 0.0f : acc;
-    if (stage == 3) {
-        u[i] = acc_buf[i] + ca * F;
-        return;
-    }
+    const float F = (frozen && frozen[i]) ? 0.0f : acc;
     const float ui = u[i];
-    acc_buf[i] = (stage == 0 ? ui : acc_buf[i]) + ca * F;
-    nxt[i] = ui + cnx * F;
+    switch (stage) {
+    case 0:
+        acc_buf[i] = ui + dt * (float)(1.0 / 6.0) * F;
+        nxt[i] = ui + dt * 0.5f * F;
+        break;
+    case 1:
+        acc_buf[i] = acc_buf[i] + dt * (float)(1.0 / 3.0) * F;
+        nxt[i] = ui + dt * 0.5f * F;
+        break;
+    case 2:
+        acc_buf[i] = acc_buf[i] + dt * (float)(1.0 / 3.0) * F;
+        nxt[i] = ui + dt * F;
+        break;
+    default:
+        u[i] = acc_buf[i] + dt * (float)(1.0 / 6.0) * F;
+        break;
+    }
 }
 
 // Coefficients of a step's stages
@@ -361,7 +371,7 @@ Shape default_shape(const labfm_ctx *ctx, int min_g)
 
 unsigned blocks_for(int64_t n, int G) { return (unsigned)((n * G + APPLY_THREADS - 1) / APPLY_THREADS); }
 
-// Coefficients of stage 0 .. 3 (see k_rk4_stage_csr)
+// Coefficients of stage 0 .. 3 of a Burgers run on float fields: of acc (or u), and of nxt
 float stage_ca(int stage, double dt) { return (float)dt * (float)(stage == 0 || stage == 3 ? 1.0 / 6.0 : 1.0 / 3.0); }
 float stage_cn(int stage, double dt) { return stage == 2 ? (float)dt : (float)dt * 0.5f; }
 
@@ -397,8 +407,7 @@ cudaError_t launch_stage_csr(labfm_ctx *ctx, Shape sh, const float *src, float *
     const float *wc_lo = CW == CW_DF ? reinterpret_cast<const float *>(ctx->wcomb.as<int2>() + ctx->nnz) : nullptr;
     auto args = [&](auto kern) {
         kern<<<blocks, APPLY_THREADS, 0, s>>>(ctx->n, ctx->row_ptr.as<int64_t>(), ctx->col.as<int32_t>(), wc, wc_lo, src, u,
-                                              acc, nxt, frozen, stage, stage_ca(stage, dt), stage_cn(stage, dt),
-                                              log2_of(sh.G));
+                                              acc, nxt, frozen, stage, (float)dt, log2_of(sh.G));
     };
     switch (sh.UNR) {
     case 2: args(k_rk4_stage_csr<CW, 2>); break;
@@ -726,8 +735,8 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_burg_combine_sliced(int64_t n
 template <class WT, int UNR>
 __global__ void __launch_bounds__(APPLY_THREADS) k_burgers_stage_csr(int64_t n, const int64_t *__restrict__ row_ptr,
                                                                  const int32_t *__restrict__ col,
-                                                                 const WT *__restrict__ wb, const float *su,
-                                                                 const float *sv, float *__restrict__ u,
+                                                                 const WT *__restrict__ wb, const float *__restrict__ su,
+                                                                 const float *__restrict__ sv, float *__restrict__ u,
                                                                  float *__restrict__ v, float *__restrict__ acc,
                                                                  float *__restrict__ nxt,
                                                                  const uint8_t *__restrict__ frozen, int stage, float ca,
@@ -739,11 +748,12 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_burgers_stage_csr(int64_t n, 
     const int64_t i = ((int64_t)blockIdx.x * APPLY_THREADS + threadIdx.x) >> lg_g;
     const bool live = i < n;
     int64_t rs = 0, re = 0;
-    bool fixed = false;
+    AT ui = 0, vi = 0;
     if (live) {
         rs = row_ptr[i];
         re = row_ptr[i + 1];
-        fixed = frozen && frozen[i];
+        ui = (AT)su[i];
+        vi = (AT)sv[i];
     }
     int cj[UNR];
     WT w0[UNR], w1[UNR], wl[UNR];
@@ -761,11 +771,9 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_burgers_stage_csr(int64_t n, 
             }
         }
     };
-    if (rs < re) load_batch(rs);
-    const AT ui = live ? (AT)su[i] : (AT)0, vi = live ? (AT)sv[i] : (AT)0;
     AT fu = 0, fv = 0;
     for (int64_t base = rs; base < re; base += (int64_t)G * UNR) {
-        if (base != rs) load_batch(base);
+        load_batch(base);
 #pragma unroll
         for (int q = 0; q < UNR; q++) {
             if (cj[q] >= 0) {
@@ -780,6 +788,7 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_burgers_stage_csr(int64_t n, 
         fv += __shfl_xor_sync(0xffffffffu, fv, o);
     }
     if (!live || lane != 0) return;
+    const bool fixed = frozen && frozen[i];
     const float Fu = fixed ? 0.0f : (float)fu;
     const float Fv = fixed ? 0.0f : (float)fv;
     if (stage == 3) {

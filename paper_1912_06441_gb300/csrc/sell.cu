@@ -69,9 +69,10 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l,
 
 }  // namespace
 
-// Lanes per node, as the power of two that gives the busiest SM the fewest FP64 instructions (a run gives every SM an
-// equal share of the slices): slices per SM, times two per entry of a lane, about four for the node and two per
-// combining step.  One lane for large sets; more where whole slices are too coarse a share.
+// Lanes per node, as the power of two with the least cost of a sweep on the busiest SM (a run gives every SM an equal
+// share of the slices): 16 cycles per FP64 instruction, two per entry of a lane, about four for the node and two per
+// combining step; and about 50 cycles per step for its loads, which the other warps hide on all but small sets.  One
+// lane for large sets, two at 161^2 nodes, eight at 41^2 (measured, heat: 2 lanes at 41^2 5.05 us a stage).
 static int sell_lanes_log2(int64_t n, int64_t nnz, int num_sms)
 {
     const int64_t deg = n > 0 ? (nnz + n - 1) / n : 0;
@@ -79,7 +80,7 @@ static int sell_lanes_log2(int64_t n, int64_t nnz, int num_sms)
     int64_t least = INT64_MAX;
     for (int lg = 0; lg <= 4; lg++) {
         const int64_t slices = ((n << lg) + 31) / 32, most = (slices + num_sms - 1) / num_sms;
-        const int64_t cost = most * (2 * ((deg + (1 << lg) - 1) >> lg) + 2 * lg + 4);
+        const int64_t steps = (deg + (1 << lg) - 1) >> lg, cost = 16 * most * (2 * steps + 2 * lg + 4) + 50 * steps;
         if (cost < least) {
             least = cost;
             best = lg;
