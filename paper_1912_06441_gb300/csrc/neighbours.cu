@@ -112,6 +112,24 @@ __global__ void k_cell_scatter(int64_t n, const double *__restrict__ xy, const i
     if (cell_xyf) cell_xyf[pos] = make_float2((float)x, (float)y);
 }
 
+// The up-to-3 distinct cell coordinates around c along one axis.
+__device__ __forceinline__ int axis_cells(int c, int nc, int periodic, int out[3])
+{
+    int m = 0;
+    for (int d = -1; d <= 1; d++) {
+        int v = c + d;
+        if (periodic) {
+            v = v < 0 ? v + nc : (v >= nc ? v - nc : v);
+        } else if (v < 0 || v >= nc) {
+            continue;
+        }
+        bool dup = false;
+        for (int t = 0; t < m; t++) dup |= (out[t] == v);
+        if (!dup) out[m++] = v;
+    }
+    return m;
+}
+
 // The exact distance test of Sec. 2 in IEEE double, explicitly rounded (no contraction).
 __device__ __forceinline__ bool within_exact(double qx, double qy, double xi, double yi, double R2, const Grid &g)
 {
@@ -415,10 +433,101 @@ __global__ void __launch_bounds__(NB_THREADS) k_sweep(int64_t n, const double *_
     if (!WRITE && lane < nodes) counts[my_i] = my_cnt;
 }
 
+// The same with a thread per node, in cell order, its row sorted by insertion: for large sets of few nodes to a cell, where
+// the rows are short and a warp's eight nodes lie in several cells.
+template <bool WRITE>
+__global__ void k_sweep_sparse(int64_t n, const double *__restrict__ h, Grid g,
+                        const int32_t *__restrict__ cell_of, const int64_t *__restrict__ cell_start,
+                        const int32_t *__restrict__ cell_nodes, const double2 *__restrict__ cell_xy,
+                        const float2 *__restrict__ cell_xyf, int32_t *__restrict__ counts,
+                        const int64_t *__restrict__ row_ptr, int32_t *__restrict__ col)
+{
+    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    int i = cell_nodes[t];
+    const double xi = cell_xy[t].x, yi = cell_xy[t].y;
+    double R = 2.0 * h[i];
+    double R2 = __dmul_rn(R, R);
+    // float classification only where the float wrap cannot flip a candidate near the radius
+    const bool filt = cell_xyf != nullptr && (!g.periodic || R2 <= g.r2_wrap_max);
+    const Prefilter pre((float)xi, (float)yi, (float)R2, g);
+    int c = cell_of[i];
+    int cx = c % g.nc[0], cy = c / g.nc[0];
+    int xs[3], ys[3];
+    int mx = axis_cells(cx, g.nc[0], g.periodic, xs);
+    int my = axis_cells(cy, g.nc[1], g.periodic, ys);
+    int cnt = 0;
+    int64_t base = WRITE ? row_ptr[i] : 0;
+    for (int a = 0; a < my; a++) {
+        for (int b = 0; b < mx; b++) {
+            int cc = ys[a] * g.nc[0] + xs[b];
+            int64_t s = cell_start[cc], e = cell_start[cc + 1];
+            for (int64_t p = s; p < e; p++) {
+                int j = cell_nodes[p];
+                if (j == i) continue;
+                bool in;
+                int decided = 0;  // 1: inside, 2: outside, 0: to the double test
+                if (filt) {
+                    bool inside, outside;
+                    pre.test(cell_xyf[p], g.periodic != 0, g, inside, outside);
+                    decided = inside ? 1 : (outside ? 2 : 0);
+                }
+                if (decided) {
+                    in = decided == 1;
+                } else {
+                    const double2 q = cell_xy[p];
+                    in = within_exact(q.x, q.y, xi, yi, R2, g);
+                }
+                if (in) {
+                    if (WRITE) col[base + cnt] = j;
+                    cnt++;
+                }
+            }
+        }
+    }
+    if (!WRITE) {
+        counts[i] = cnt;
+    } else {
+        // insertion sort of the row (stencils hold tens of entries)
+        int32_t *row = col + base;
+        for (int u = 1; u < cnt; u++) {
+            int32_t v = row[u];
+            int w = u - 1;
+            while (w >= 0 && row[w] > v) {
+                row[w + 1] = row[w];
+                w--;
+            }
+            row[w + 1] = v;
+        }
+    }
+}
+
+// Which of the two: whole searches take, with k_sweep_sparse and k_sweep, at 900^2 nodes 683 and 841 us at order 3 (6.8 nodes
+// a cell), 762 and 893 at order 4 (7.8), but 1,057 and 932 at order 5 (10.2); at 600^2 order 2 and 3 (5.8, 6.8) 422 and 478,
+// 443 and 470, at 450^2 364 and 335 at order 4; at 200^2 k_sweep wins at every order (194 against 259 at order 4).
+bool sparse_cells(int64_t n, const Grid &g)
+{
+    const double per_cell = (double)n / ((double)g.nc[0] * (double)g.nc[1]);
+    return per_cell < 7.5 ? n >= 200000 : per_cell < 9.0 && n >= 400000;
+}
+
 unsigned sweep_blocks(int64_t n)
 {
     const int64_t per = NB_THREADS / 32 * SWEEP_NODES;
     return (unsigned)((n + per - 1) / per);
+}
+
+template <bool WRITE>
+void launch_sweep(int64_t n, const double *h, const Grid &g, const int32_t *cell_of, const int64_t *cell_start,
+                  const int32_t *cell_nodes, const double2 *cell_xy, const float2 *cell_xyf, int32_t *counts,
+                  const int64_t *row_ptr, int32_t *col, cudaStream_t s)
+{
+    if (sparse_cells(n, g))
+        k_sweep_sparse<WRITE><<<(unsigned)((n + NB_THREADS - 1) / NB_THREADS), NB_THREADS, 0, s>>>(
+            n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, row_ptr, col);
+    else
+        k_sweep<WRITE><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf,
+                                                              counts, row_ptr, col);
 }
 
 }  // namespace
@@ -514,8 +623,7 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(cell_count, cell_start, ncells, ctx->scan_tmp, s));
     k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, cell_xyf);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
-    k_sweep<false><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts,
-                                              nullptr, nullptr);
+    launch_sweep<false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, nullptr, nullptr, s);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(counts, row_ptr, n, ctx->scan_tmp, s));
     int64_t *nnz_h = (int64_t *)ctx->host_small;
@@ -524,8 +632,7 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     int64_t nnz = *nnz_h;
     if (nnz >= ((int64_t)1 << 40)) return fail(ctx, LABFM_ERR_CAPACITY, "too many stencil entries");
     LABFM_CUDA_TRY(ctx, ctx->col.reserve(sizeof(int32_t) * (nnz > 0 ? nnz : 1)));
-    k_sweep<true><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr,
-                                             row_ptr, ctx->col.as<int32_t>());
+    launch_sweep<true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr, row_ptr, ctx->col.as<int32_t>(), s);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
     ctx->n = n;
@@ -670,8 +777,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
     // (the float pre-filter needs an array the fixed scratch does not hold: the double test alone)
     k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, nullptr);
     NA_TRY(cudaGetLastError());
-    k_sweep<false><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, counts,
-                                              nullptr, nullptr);
+    launch_sweep<false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, counts, nullptr, nullptr, s);
     NA_TRY(cudaGetLastError());
     NA_TRY(exclusive_scan_i32_to_i64_ws(counts, row_ptr, n, scan_tmp, NA_SCAN_ELEMS, s));
     int64_t nnz = 0;
@@ -680,8 +786,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
     *nnz_out = nnz;
     if (nnz > col_capacity) return LABFM_ERR_CAPACITY;
     if (nnz > 0) {
-        k_sweep<true><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr,
-                                                 nullptr, row_ptr, col);
+        launch_sweep<true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, nullptr, row_ptr, col, s);
         NA_TRY(cudaGetLastError());
     }
     NA_TRY(cudaStreamSynchronize(s));

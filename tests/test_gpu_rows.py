@@ -36,6 +36,20 @@ def test_rows_of_every_length(n, radius, periodic):
     assert np.array_equal(rp, orp) and np.array_equal(col, ocol)
 
 
+@pytest.mark.parametrize("periodic", [True, False])
+@pytest.mark.parametrize("n,spacings", [(200000, 2.3), (200001, 2.6), (400000, 2.9), (399999, 2.9)])
+def test_large_sets_of_few_nodes_a_cell(n, spacings, periodic):
+    """Random nodes around the sizes where the search changes its sweep, 5 to 8 nodes a cell on average."""
+    rng = np.random.default_rng(n)
+    xy = rng.random((n, 2))
+    h = 0.5 * spacings / np.sqrt(n) * (0.7 + 0.3 * rng.random(n))
+    rp, col = _search(xy, h, periodic)
+    q = np.sort(rng.choice(n, 3000, replace=False))
+    orp, ocol = oracle.neighbours_large(xy, h, periodic, queries=q)
+    assert np.array_equal(rp[q + 1] - rp[q], np.diff(orp))
+    assert np.array_equal(np.concatenate([col[rp[i]:rp[i + 1]] for i in q]), ocol)
+
+
 def test_row_offsets_of_many_blocks():
     """2898^2 lattice nodes (more than 4,096 blocks of the prefix sum), 2 h = 1.2 spacings: the four nearest nodes,
     fewer at the edges, known without a search."""
