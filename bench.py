@@ -57,6 +57,20 @@ def build_flops_per_node(k, ni, n_ops):
     return 2 * coef * ni + 2 * p * p * ni + (2.0 / 3.0) * p ** 3 + 2 * p * p * n_ops + 2 * p * ni * n_ops
 
 
+def moment_build_flops_per_node(k, ni, n_ops):
+    """FP64 flops of the FP64 build of orders 5 to 8 with the full chain rule, which forms M from moments: per neighbour
+    the powers, g_1 .. g_k and radial functions (about 4 k + k + 60), a product per monomial and a multiply-add per sum
+    (T_k over degrees k + 1 .. 2k, the highest degree of each other T_n, A2 over 2 .. k + 2, A3 over 4 .. k + 3), per operator
+    a polynomial of p terms and seven further functions; elimination as in build_flops_per_node."""
+    p = p_of_k(k)
+    top = 3 * k * (k + 1) // 2
+    fam = sum(d + 1 for d in range(2, k + 3)) + sum(d + 1 for d in range(4, k + 4))
+    sums = top + (top - (2 * k + 1)) + fam
+    monomials = sum(d + 1 for d in range(2, 2 * k + 1))
+    per_neighbour = 5 * k + 60 + monomials + 2 * sums + 2 * (p + 7) * n_ops
+    return per_neighbour * ni + (2.0 / 3.0) * p ** 3 + 2 * p * p * n_ops
+
+
 def apply_bytes(n, nnz, n_ops, wbytes=8, fbytes=8):
     """Algorithmic bytes of one application of n_ops operators: per stencil entry one int32
     index and n_ops weights; per node f_i, row pointer and n_ops outputs (the f_j gathers hit
@@ -69,7 +83,7 @@ def scan_launches(n):
     nb = (n + items - 1) // items
     if nb <= 1:
         return 1
-    return 2 + scan_launches(nb)
+    return 2 if nb <= 4096 else 2 + scan_launches(nb)
 
 
 def ncells_of(h, box=1.0):
@@ -79,8 +93,8 @@ def ncells_of(h, box=1.0):
 
 
 def nbr_launches(n, ncells):
-    # check, assign, scan(cells)+total, scatter, count sweep, scan(rows)+total, fill sweep
-    return 1 + 1 + scan_launches(ncells) + 1 + 1 + 1 + scan_launches(n) + 1 + 1
+    # check, assign, scan(cells), scatter, count sweep, scan(rows), fill sweep
+    return 1 + 1 + scan_launches(ncells) + 1 + 1 + scan_launches(n) + 1
 
 
 class ClockSampler:
@@ -305,7 +319,7 @@ def kernel_source_hash():
     import hashlib
 
     hsh = hashlib.sha256()
-    for f in ("build_fp64.cu", "abf.cuh"):
+    for f in ("build_node.cuh", "build_fp64.cu", "abf.cuh"):
         with open(os.path.join(ROOT, "paper_1912_06441_gb300", "csrc", f), "rb") as fh:
             hsh.update(fh.read())
     return hsh.hexdigest()
@@ -1006,7 +1020,7 @@ def run_labfm(args, rank, world, local_rank):
     build_ms = float(np.mean(phase[:, 1]))
     apply_ms = float(np.mean(phase[:, 2]))
     fp64_peak = measured_fp64_peak(torch, dev)
-    bflops = build_flops_per_node(K, ni, len(OPS)) * n
+    bflops = moment_build_flops_per_node(K, ni, len(OPS)) * n
     b_ach = bflops / (build_ms * 1e-3) / 1e12
     abytes = apply_bytes(n, nnz, len(OPS))
     a_ach = abytes / (apply_ms * 1e-3) / 1e9
@@ -1040,7 +1054,8 @@ def run_labfm(args, rank, world, local_rank):
                 "d2h_bytes_per_step": d2h},
         # per step: stencil search, one build launch (uniform order), one apply, and the RK4
         # step (operator combination + 4 stage kernels)
-        "gpu_launches": args.steps * (nbr_launches(n, ncells_of(HS / N_SIDE)) + 1 + 1 + 1 + 4),
+        "gpu_launches": args.steps * (nbr_launches(n, ncells_of(HS / N_SIDE)) + 1 + 1 + 1 + 2
+                                      + scan_launches(n // 32) + 1),
         "clocks": clk,
     }
     line["build_tuning"] = L.get_build_info()["fp64_group_threads"]

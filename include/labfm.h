@@ -239,9 +239,13 @@ labfm_status labfm_apply(labfm_ctx *ctx, uint32_t op_mask, const void *f, int fi
  * floats, ~48 bits) and the stencil sums run in double-float arithmetic on the FP32 pipes.
  * The per-node stage update is in double (in float when weights and field are FP32).
  * Nodes with frozen[i] != 0 keep their value
- * (Dirichlet nodes, Sec. 5.1).  The nsteps x 4 stage launches are recorded once into a
+ * (Dirichlet nodes, Sec. 5.1).  On FP64 fields the steps run in cooperative launches (a block
+ * per SM, a barrier over them between stages) on a layout of the stencils that the first
+ * such call after labfm_build_neighbours makes; a barrier that gives up (after about a second)
+ * makes the context's next call that reads weights return LABFM_ERR_TIMEOUT, the field is then
+ * undefined.  On FP32 fields the nsteps x 4 stage launches are recorded once into a
  * CUDA graph and replayed; it is recorded again when an argument other than beta, the
- * stencil count or size, the weight type or a context buffer changes.  The stage's launch
+ * stencil count or size, the weight type or a context buffer changes.  There the stage's launch
  * shape is tuned as for labfm_apply, on first-stage launches that read u and write only
  * context-owned buffers (u is not changed by the tuning).
  *   beta    host double[n_ops]
@@ -263,13 +267,11 @@ labfm_status labfm_step(labfm_ctx *ctx, const double *beta, void *u, int field_d
  * operators carry the linear terms: beta_2 = 1/Re on nabla^2, and e.g. a hyperviscosity
  * -alpha nabla^4 or alpha nabla^6 (Sec. 4.2) as another operator.  beta[0] and beta[1] are
  * not read.  The advection coefficients are the stage's own field values, so d/dx and d/dy
- * stay separate stencil sums; the linear operators are combined once into one weight per
+ * stay separate weights, joined per entry in the stage; the linear operators are combined once into one weight per
  * entry (summed in double, kept in the weight type, cached while beta[2..] and the weights are
  * unchanged).  Sums run in double unless field and weights are both LABFM_F32.
- * Nodes with frozen[i] != 0 keep their values of u and v.  The nsteps x 4 stage launches are
- * recorded once into a CUDA graph and replayed, under the same rules as labfm_step; the
- * stage's launch shape is tuned on first-stage launches that read u and v and write only
- * context-owned buffers.
+ * Nodes with frozen[i] != 0 keep their values of u and v.  Launches as in labfm_step: cooperative
+ * on FP64 fields, a CUDA graph with a tuned launch shape on FP32 fields.
  *   beta    host double[n_ops]
  *   u, v    device [n] of field_dtype, distinct, updated in place
  *   frozen  device uint8[n] or NULL
@@ -286,10 +288,9 @@ labfm_status labfm_step_burgers(labfm_ctx *ctx, const double *beta, void *u, voi
  * A_ij = 0, F_i = g_i), so that Phi_i = f[i] there.  The matrix is not formed: its products are
  * stencil sums over the context's stencils.  Stabilised bi-conjugate gradients (van der Vorst
  * 1992) with a Jacobi preconditioner (diag A), as in Sec. 5.2; all vectors and scalars in FP64 and
- * in device memory, iterations recorded in chunks of 16 into a CUDA graph with one host read of the
- * state per chunk.  The product's launch shape (lanes per node x entries in flight, 3 x 3 shapes)
- * is timed once per problem class (floor(log2 n), mean stencil size) on a context, as for
- * labfm_apply (n >= 4096, stream not capturing).
+ * in device memory, up to 256 iterations in one cooperative launch (a block per SM, barriers over
+ * them as in labfm_step; LABFM_ERR_TIMEOUT if one gives up) with one host read of the state
+ * per launch.
  * Stops when the recurrence residual ||r|| <= tol ||F||, or after max_iter iterations.  The
  * recurrence residual drifts from the true one ||F - A Phi|| in finite precision, so the true
  * residual is then formed; if it is above tol, the iteration restarts from the current Phi
