@@ -305,6 +305,8 @@ RkCoef rk_coef(double dt) { return RkCoef{dt * (1.0 / 6.0), dt * (1.0 / 3.0), dt
 
 // nsteps steps on double fields, sliced layout, one cooperative launch (see GridBarrier): a warp per slice (see SlicePipe),
 // the first steps of a sweep loaded before its barrier.  A lane adds into two sums in turn, because a dependent FP64 add waits several times the pipe's time for one.
+// 161^2 nodes, 49 entries each: 7.6 us a stage (9.0 as launches over CSR rows), 5.0 of them FP64 issue (two instructions an
+// entry), 1.55 the barrier.
 template <class VT>
 __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView S, const VT *__restrict__ wc, double *u,
                                                            double *acc_buf, double *sa, double *sb,
@@ -803,7 +805,7 @@ __global__ void __launch_bounds__(APPLY_THREADS) k_burgers_stage_csr(int64_t n, 
     nxt[n + i] = v0 + cnx * Fv;
 }
 
-// The same on double fields (see k_rk4_run)
+// The same on double fields (see k_rk4_run).  161^2 nodes: 17.0 us a stage (29.3 as launches), 14 of them FP64 issue.
 template <class VT>
 __global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellView S, const VT *__restrict__ wb, double *u,
                                                                double *v, double *acc, double *sa, double *sb,

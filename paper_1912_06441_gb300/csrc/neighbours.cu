@@ -306,7 +306,8 @@ struct Candidates {
 // consecutive nodes in cell order.  The nodes of a cell share their candidates, which the warp keeps in registers (up to
 // SWEEP_REGS per lane; more are read again for every node): per node there is the test of each candidate, a ballot
 // that gives the hits' places in the row, and the sort.  (A warp per node spent most of its time finding the
-// node's cells: 180 us a count and 254 us a write at 512^2, order 8.)
+// node's cells: 180 us a count and 254 us a write at 512^2, order 8, against 124 and 185 now; a thread per node took 102
+// and 817.)
 constexpr int SWEEP_NODES = 8;
 constexpr int SWEEP_REGS = 8;
 template <bool WRITE>
