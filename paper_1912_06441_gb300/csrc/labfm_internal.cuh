@@ -115,7 +115,7 @@ struct labfm_ctx {
     bool wburg_valid = false, wburg_sliced = false;
     labfm::StepGraph graph_burgers;
 
-    // implicit solves (BiCGStab): operator weights in the sliced layout, ten vectors, partial sums, and for Neumann
+    // implicit solves (BiCGStab): operator weights in the sliced layout, eleven vectors, partial sums, and for Neumann
     // ghost rows their map and the layout with their parents' stencils
     labfm::DevBuf sol_w, sol_vec, sol_part, sol_gmap;
     labfm::Sell sell_ghost;

@@ -10,6 +10,9 @@
 //   rho = (r^, r); beta = (rho / rho_old)(alpha / omega); p = r + beta (p - omega v); y = M^-1 p
 //   v = A y; alpha = rho / (r^, v); s = r - alpha v; z = M^-1 s; t = A z
 //   omega = (t, s) / (t, t); x += alpha y + omega z; r = s - omega t
+// The updates of x go to d, which is added to x when the iteration ends or starts afresh: added to x one by one, their
+// roundings (of x each, a hundred times and more) would set the residual that restarts can reach, up to 1.3e-13 ||F||
+// on 53^2 nodes.
 // The iterations of a solve are one cooperative launch (up to ITERS_MAX of them, see GridBarrier): every block keeps its
 // rows, a product is followed by a barrier, and a sum over the set rides on the barrier that its iteration needs in any
 // case: each block publishes its partial sum before it and adds up all blocks' after it, in a fixed order and so to
@@ -38,7 +41,7 @@ struct SolveState {
     double tol2;       // (tol ||b||)^2
     double resid2;     // ||b - A x||^2 at the end
     int done;          // 0 running, 1 converged, 2 breakdown, 3 iteration limit
-    int skip;          // ||s|| already within the tolerance: omega = 0, x += alpha y, r = s
+    int skip;          // ||s|| already within the tolerance: omega = 0, d += alpha y, r = s
     int iters;
     int max_iter;
 };
@@ -181,7 +184,7 @@ struct SolveArgs {
     const double *wd, *adiag, *dinv, *b;
     const uint8_t *dirichlet;
     GhostRows gr;
-    double *x, *r, *rhat, *p, *v, *y, *s, *z, *t;
+    double *x, *d, *r, *rhat, *p, *v, *y, *s, *z, *t;  // d: what the iteration has added to x since its start
     double *part;  // [NSLOT][blocks]
     SolveState *st;
     GridSync sync;
@@ -210,7 +213,10 @@ struct SolveBlock {
     // multiply-add per stencil entry (Dirichlet rows: x_i; a Neumann ghost row: the stencil of its parent b with the
     // ghost weights, and the diagonal term on x_b): fn(i, (A x)_i, own_i) on one lane per row, own_i read ahead.  The first
     // steps of the next product are on their way when it returns.
-    template <class Fn>
+    // DIFFERENCES: as sum_j w_ji (x_j - x_i), for true residuals.  The terms of the global form cancel (by a factor of
+    // about (L / h)^2 in a Laplacian of a smooth x), and its roundings, 1e-13 ||F|| on 41^2 nodes, made solves to that
+    // tolerance end or fail by the order of the sums; the differences hardly cancel.
+    template <bool DIFFERENCES, class Fn>
     __device__ __forceinline__ void product(const double *x, const double *own, Fn fn)
     {
         for (int64_t slice = s0 + warp; slice < s1; slice += RUN_THREADS / 32) {
@@ -223,20 +229,24 @@ struct SolveBlock {
             const bool row = i >= 0 && l.h == 0;
             double xi = 0.0, ai = 0.0, oi = 0.0;
             bool fixed = false;
-            if (row) {
-                oi = own[i];
+            if (row || (DIFFERENCES && i >= 0)) {
                 int64_t src = i;
                 if (A.gr.gmap && A.gr.gmap[i] >= 0) src = A.gr.parent[A.gr.gmap[i]];
                 xi = x[src];
-                ai = A.adiag[i];
+            }
+            if (row) {
+                oi = own[i];
+                if (!DIFFERENCES) ai = A.adiag[i];
                 fixed = A.dirichlet && A.dirichlet[i];
             }
             double sum[2] = {0.0, 0.0};
             pipe.run(l, lane, A.S, A.wd, [&](int j, double(&xv)[1]) { xv[0] = x[j]; },
-                     [&](int q, const double(&xv)[1], const double(&w)[1]) { sum[q & 1] = fma(xv[0], w[0], sum[q & 1]); });
+                     [&](int q, const double(&xv)[1], const double(&w)[1]) {
+                         sum[q & 1] = fma(DIFFERENCES ? xv[0] - xi : xv[0], w[0], sum[q & 1]);
+                     });
             double acc = sum[0] + sum[1];
             for (int o = (1 << A.S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (row) fn(i, fixed ? xi : fma(ai, xi, acc), oi);
+            if (row) fn(i, fixed ? xi : DIFFERENCES ? acc : fma(ai, xi, acc), oi);
         }
         pipe.preload(first, lane, A.S, A.wd);
     }
@@ -300,8 +310,9 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
     };
     if (start) {
         double rr = 0.0, bb = 0.0;
-        B.product(A.x, A.b, [&](int64_t i, double ax, double bi) {
+        B.product<true>(A.x, A.b, [&](int64_t i, double ax, double bi) {
             const double ri = bi - ax;
+            A.d[i] = 0.0;
             A.r[i] = ri;
             A.rhat[i] = ri;
             A.p[i] = 0.0;
@@ -325,7 +336,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
         if (!B.bar.wait()) return;
         // v = A y, (rhat, v) -> alpha
         double d0 = 0.0, d1 = 0.0;
-        B.product(A.y, A.rhat, [&](int64_t i, double vi, double hi) {
+        B.product<false>(A.y, A.rhat, [&](int64_t i, double vi, double hi) {
             A.v[i] = vi;
             d0 = fma(hi, vi, d0);
         });
@@ -347,7 +358,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
         if (threadIdx.x == 0) st.snorm2 = sum[0];
         // t = A z, (t, s), (t, t) -> omega
         d0 = 0.0;
-        B.product(A.z, A.s, [&](int64_t i, double ti, double si) {
+        B.product<false>(A.z, A.s, [&](int64_t i, double ti, double si) {
             A.t[i] = ti;
             d0 = fma(si, ti, d0);
             d1 = fma(ti, ti, d1);
@@ -355,12 +366,12 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
         if (!B.reduce<2>(2, d0, d1, sum)) return;
         scalars(4);
         if (st.done) break;
-        // x += alpha y + omega z; r = s - omega t; (rhat, r), (r, r) -> rho, beta, convergence
+        // d += alpha y + omega z; r = s - omega t; (rhat, r), (r, r) -> rho, beta, convergence
         d0 = d1 = 0.0;
         {
             const double alpha = st.alpha, omega = st.omega;
             for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
-                A.x[i] = fma(omega, A.z[i], fma(alpha, A.y[i], A.x[i]));
+                A.d[i] = fma(omega, A.z[i], fma(alpha, A.y[i], A.d[i]));
                 const double ri = fma(-omega, A.t[i], A.s[i]);
                 A.r[i] = ri;
                 d0 = fma(A.rhat[i], ri, d0);
@@ -371,8 +382,10 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
         scalars(5);
     }
     if (st.done) {
+        for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) A.x[i] += A.d[i];
+        if (!B.bar.wait()) return;
         double rr = 0.0, bb = 0.0;
-        B.product(A.x, A.b, [&](int64_t, double ax, double bi) {
+        B.product<true>(A.x, A.b, [&](int64_t, double ax, double bi) {
             const double ri = bi - ax;
             rr = fma(ri, ri, rr);
             bb = fma(bi, bi, bb);
@@ -428,12 +441,12 @@ labfm_status run_solve(labfm_ctx *ctx, int op, const double *f, double *phi, con
     if (ls != LABFM_OK) return ls;
     const SellView S = sell_view(L);
     LABFM_CUDA_TRY(ctx, ctx->sol_w.reserve(sizeof(double) * (L.places > 0 ? L.places : 1)));
-    LABFM_CUDA_TRY(ctx, ctx->sol_vec.reserve(sizeof(double) * 10 * n));
+    LABFM_CUDA_TRY(ctx, ctx->sol_vec.reserve(sizeof(double) * 11 * n));
     LABFM_CUDA_TRY(ctx, ctx->sol_part.reserve(sizeof(double) * NSLOT * (size_t)ctx->num_sms + sizeof(SolveState)));
     LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
     double *V = ctx->sol_vec.as<double>();
     double *dinv = V, *r = V + n, *rhat = V + 2 * n, *p = V + 3 * n, *v = V + 4 * n, *y = V + 5 * n, *sv = V + 6 * n,
-           *z = V + 7 * n, *t = V + 8 * n, *adiag = V + 9 * n;
+           *z = V + 7 * n, *t = V + 8 * n, *adiag = V + 9 * n, *d = V + 10 * n;
     double *part = ctx->sol_part.as<double>();
     SolveState *st = reinterpret_cast<SolveState *>(part + NSLOT * (size_t)ctx->num_sms);
     const double *wd = ctx->sol_w.as<double>();
@@ -453,7 +466,7 @@ labfm_status run_solve(labfm_ctx *ctx, int op, const double *f, double *phi, con
     init.tol2 = tol * tol;
     init.max_iter = max_iter;
     LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(st, &init, sizeof(SolveState), cudaMemcpyHostToDevice, s));
-    const SolveArgs args{n, S, wd, adiag, dinv, f, dirichlet, gr, phi, r, rhat, p, v, y, sv, z, t, part, st, grid_sync(ctx)};
+    const SolveArgs args{n, S, wd, adiag, dinv, f, dirichlet, gr, phi, d, r, rhat, p, v, y, sv, z, t, part, st, grid_sync(ctx)};
     const int most = (int)std::max<int64_t>(8, std::min<int64_t>(ITERS_MAX, (int64_t)1000000000 / (nnz + 100000)));
     // Launches until the state says that the iteration ended, with the true residual.  BiCGStab
     // restarts from the current iterate (r = F - A Phi, r^ = r), at most MAX_RESTARTS times
