@@ -303,7 +303,7 @@ struct RkCoef {
 };
 RkCoef rk_coef(double dt) { return RkCoef{dt * (1.0 / 6.0), dt * (1.0 / 3.0), dt * 0.5, dt}; }
 
-// nsteps steps on double fields, sliced layout, one cooperative launch (see GridBarrier): a warp per slice (see SlicePipe),
+// nsteps steps on double fields, sliced layout, one cooperative launch (see GridBarrier): a block's slices by its warps (see share_out),
 // the first steps of a sweep loaded before its barrier.  A lane adds into two sums in turn, because a dependent FP64 add waits several times the pipe's time for one.
 // 161^2 nodes, 49 entries each: 7.6 us a stage (9.0 as launches over CSR rows), 5.0 of them FP64 issue (two instructions an
 // entry), 1.55 the barrier.
@@ -313,43 +313,48 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView 
                                                            const uint8_t *__restrict__ frozen, int64_t nsteps, RkCoef rk,
                                                            GridSync sync)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t s0, s1;
-    slice_share(S.n_slices, s0, s1);
+    block_share(S, s0, s1);
     GridBarrier bar{sync};
-    const SellLane first(s0 + warp < s1 ? s0 + warp : S.n_slices, lane, n, S);
-    SlicePipe<4, 1, 1, VT> pipe;
-    pipe.preload(first, lane, S, wc);
+    struct Node {
+        double si, ui, ai, sum[2];
+        bool row, fixed;  // row: this lane updates the node; what it needs is read ahead
+    };
+    share_out(S, s0, s1);
+    SliceSweep<4, 1, 1, 1, VT> sweep;
+    sweep.preload(n, S, wc);
     for (int64_t it = 0; it < 4 * nsteps; it++) {
         const int stage = (int)(it & 3);
         const double *src = stage == 0 ? u : stage == 2 ? sb : sa;
-        for (int64_t slice = s0 + warp; slice < s1; slice += RUN_THREADS / 32) {
-            SellLane l = first;
-            if (slice != s0 + warp) {
-                l = SellLane(slice, lane, n, S);
-                pipe.preload(l, lane, S, wc);
-            }
-            const int64_t i = l.i;
-            const double si = i >= 0 ? src[i] : 0.0;
-            const bool row = i >= 0 && l.h == 0;  // this lane updates the node; what it needs is read ahead
-            const bool fixed = row && frozen && frozen[i];
-            const double ui = row && stage != 3 ? u[i] : 0.0, ai = row && stage != 0 ? acc_buf[i] : 0.0;
-            double sum[2] = {0.0, 0.0};
-            pipe.run(l, lane, S, wc, [&](int j, double(&x)[1]) { x[0] = src[j]; },
-                     [&](int q, const double(&x)[1], const VT(&w)[1]) { sum[q & 1] = fma(x[0] - si, (double)w[0], sum[q & 1]); });
-            double acc = sum[0] + sum[1];
-            for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (!row) continue;
-            const double F = fixed ? 0.0 : acc;
-            if (stage == 3) {
-                u[i] = ai + rk.sixth * F;
-                continue;
-            }
-            acc_buf[i] = stage == 0 ? ui + rk.sixth * F : ai + rk.third * F;
-            (stage == 1 ? sb : sa)[i] = ui + (stage == 2 ? rk.one : rk.half) * F;
-        }
+        sweep.run(
+            n, S, wc,
+            [&](const SellLane &l, bool own) {
+                Node v;
+                v.row = own && l.i >= 0 && l.h == 0;
+                v.si = l.i >= 0 ? src[l.i] : 0.0;
+                v.fixed = v.row && frozen && frozen[l.i];
+                v.ui = v.row && stage != 3 ? u[l.i] : 0.0;
+                v.ai = v.row && stage != 0 ? acc_buf[l.i] : 0.0;
+                v.sum[0] = v.sum[1] = 0.0;
+                return v;
+            },
+            [&](int j, double(&x)[1]) { x[0] = src[j]; },
+            [&](Node &v, int q, const double(&x)[1], const VT(&w)[1]) { v.sum[q & 1] = fma(x[0] - v.si, (double)w[0], v.sum[q & 1]); },
+            [&](const Node &v, double(&p)[1]) { p[0] = v.sum[0] + v.sum[1]; },
+            [&](const SellLane &l, const Node &v, const double(&p)[1]) {
+                double acc = p[0];
+                for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (!v.row) return;
+                const double F = v.fixed ? 0.0 : acc;
+                if (stage == 3) {
+                    u[l.i] = v.ai + rk.sixth * F;
+                    return;
+                }
+                acc_buf[l.i] = stage == 0 ? v.ui + rk.sixth * F : v.ai + rk.third * F;
+                (stage == 1 ? sb : sa)[l.i] = v.ui + (stage == 2 ? rk.one : rk.half) * F;
+            });
         if (it + 1 == 4 * nsteps) break;
-        pipe.preload(first, lane, S, wc);
+        sweep.preload(n, S, wc);
         if (!bar.wait()) return;
     }
 }
@@ -620,9 +625,9 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
         const SellView S = sell_view(ctx->sell);
         LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
         cudaError_t e = enqueue_runs(ctx, nsteps, [&](int64_t steps) {
-            return fmt == CW_S64 ? launch_run(ctx, S.n_slices, k_rk4_run<double>, n, S, ctx->wcomb.as<double>(), uu, acc, sa, sb,
+            return fmt == CW_S64 ? launch_run(ctx, S, k_rk4_run<double>, n, S, ctx->wcomb.as<double>(), uu, acc, sa, sb,
                                               frozen, steps, rk_coef(dt), grid_sync(ctx))
-                                 : launch_run(ctx, S.n_slices, k_rk4_run<float>, n, S, ctx->wcomb.as<float>(), uu, acc, sa, sb,
+                                 : launch_run(ctx, S, k_rk4_run<float>, n, S, ctx->wcomb.as<float>(), uu, acc, sa, sb,
                                               frozen, steps, rk_coef(dt), grid_sync(ctx));
         });
         return e == cudaSuccess ? LABFM_OK : cuda_fail(ctx, e, "RK4 run");
@@ -812,63 +817,70 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellV
                                                                const uint8_t *__restrict__ frozen, int64_t nsteps,
                                                                RkCoef rk, GridSync sync)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t s0, s1;
-    slice_share(S.n_slices, s0, s1);
+    block_share(S, s0, s1);
     GridBarrier bar{sync};
-    const SellLane first(s0 + warp < s1 ? s0 + warp : S.n_slices, lane, n, S);
-    SlicePipe<2, 3, 2, VT> pipe;
-    pipe.preload(first, lane, S, wb);
+    struct Node {
+        double s[2], u0[2], a0[2], f[2];
+        bool row, fixed;
+    };
+    share_out(S, s0, s1);
+    SliceSweep<2, 3, 2, 2, VT> sweep;
+    sweep.preload(n, S, wb);
     for (int64_t it = 0; it < 4 * nsteps; it++) {
         const int stage = (int)(it & 3);
         const double *su = stage == 0 ? u : stage == 2 ? sb : sa, *sv = stage == 0 ? v : su + n;
-        for (int64_t slice = s0 + warp; slice < s1; slice += RUN_THREADS / 32) {
-            SellLane l = first;
-            if (slice != s0 + warp) {
-                l = SellLane(slice, lane, n, S);
-                pipe.preload(l, lane, S, wb);
-            }
-            const int64_t i = l.i;
-            const double ui = i >= 0 ? su[i] : 0.0, vi = i >= 0 ? sv[i] : 0.0;
-            const bool row = i >= 0 && l.h == 0;
-            const bool fixed = row && frozen && frozen[i];
-            double *const field[2] = {u, v};
-            double u0[2] = {0.0, 0.0}, a0[2] = {0.0, 0.0};
+        double *const field[2] = {u, v};
+        sweep.run(
+            n, S, wb,
+            [&](const SellLane &l, bool own) {
+                Node b;
+                b.row = own && l.i >= 0 && l.h == 0;
+                b.fixed = b.row && frozen && frozen[l.i];
+                b.s[0] = l.i >= 0 ? su[l.i] : 0.0;
+                b.s[1] = l.i >= 0 ? sv[l.i] : 0.0;
 #pragma unroll
-            for (int c = 0; c < 2; c++) {
-                if (row && stage != 3) u0[c] = field[c][i];
-                if (row && stage != 0) a0[c] = acc[c * n + i];
-            }
-            double fu = 0.0, fv = 0.0;
-            pipe.run(l, lane, S, wb,
-                     [&](int j, double(&x)[2]) {
-                         x[0] = su[j];
-                         x[1] = sv[j];
-                     },
-                     [&](int, const double(&x)[2], const VT(&w)[3]) {
-                         const double c = fma(-vi, (double)w[1], fma(-ui, (double)w[0], (double)w[2]));
-                         fu = fma(x[0] - ui, c, fu);
-                         fv = fma(x[1] - vi, c, fv);
-                     });
-            for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) {
-                fu += __shfl_xor_sync(0xffffffffu, fu, o);
-                fv += __shfl_xor_sync(0xffffffffu, fv, o);
-            }
-            if (!row) continue;
-            const double F[2] = {fixed ? 0.0 : fu, fixed ? 0.0 : fv};
-            double *const nxt = stage == 1 ? sb : sa;
-#pragma unroll
-            for (int c = 0; c < 2; c++) {
-                if (stage == 3) {
-                    field[c][i] = a0[c] + rk.sixth * F[c];
-                    continue;
+                for (int c = 0; c < 2; c++) {
+                    b.u0[c] = b.row && stage != 3 ? field[c][l.i] : 0.0;
+                    b.a0[c] = b.row && stage != 0 ? acc[c * n + l.i] : 0.0;
+                    b.f[c] = 0.0;
                 }
-                acc[c * n + i] = stage == 0 ? u0[c] + rk.sixth * F[c] : a0[c] + rk.third * F[c];
-                nxt[c * n + i] = u0[c] + (stage == 2 ? rk.one : rk.half) * F[c];
-            }
-        }
+                return b;
+            },
+            [&](int j, double(&x)[2]) {
+                x[0] = su[j];
+                x[1] = sv[j];
+            },
+            [&](Node &b, int, const double(&x)[2], const VT(&w)[3]) {
+                const double c = fma(-b.s[1], (double)w[1], fma(-b.s[0], (double)w[0], (double)w[2]));
+                b.f[0] = fma(x[0] - b.s[0], c, b.f[0]);
+                b.f[1] = fma(x[1] - b.s[1], c, b.f[1]);
+            },
+            [&](const Node &b, double(&p)[2]) {
+                p[0] = b.f[0];
+                p[1] = b.f[1];
+            },
+            [&](const SellLane &l, const Node &b, const double(&p)[2]) {
+                double f[2] = {p[0], p[1]};
+                for (int o = (1 << S.lg_l) >> 1; o > 0; o >>= 1) {
+                    f[0] += __shfl_xor_sync(0xffffffffu, f[0], o);
+                    f[1] += __shfl_xor_sync(0xffffffffu, f[1], o);
+                }
+                if (!b.row) return;
+                double *const nxt = stage == 1 ? sb : sa;
+#pragma unroll
+                for (int c = 0; c < 2; c++) {
+                    const double F = b.fixed ? 0.0 : f[c];
+                    if (stage == 3) {
+                        field[c][l.i] = b.a0[c] + rk.sixth * F;
+                        continue;
+                    }
+                    acc[c * n + l.i] = stage == 0 ? b.u0[c] + rk.sixth * F : b.a0[c] + rk.third * F;
+                    nxt[c * n + l.i] = b.u0[c] + (stage == 2 ? rk.one : rk.half) * F;
+                }
+            });
         if (it + 1 == 4 * nsteps) break;
-        pipe.preload(first, lane, S, wb);
+        sweep.preload(n, S, wb);
         if (!bar.wait()) return;
     }
 }
@@ -970,9 +982,9 @@ labfm_status run_step_burgers(labfm_ctx *ctx, const double *beta, void *u, void 
         LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
         cudaError_t e = enqueue_runs(ctx, nsteps, [&](int64_t steps) {
             return ctx->wdtype == LABFM_F64
-                       ? launch_run(ctx, S.n_slices, k_burgers_run<double>, n, S, ctx->wburg.as<double>(), uu, vv, acc, sa, sb,
+                       ? launch_run(ctx, S, k_burgers_run<double>, n, S, ctx->wburg.as<double>(), uu, vv, acc, sa, sb,
                                     frozen, steps, rk_coef(dt), grid_sync(ctx))
-                       : launch_run(ctx, S.n_slices, k_burgers_run<float>, n, S, ctx->wburg.as<float>(), uu, vv, acc, sa, sb,
+                       : launch_run(ctx, S, k_burgers_run<float>, n, S, ctx->wburg.as<float>(), uu, vv, acc, sa, sb,
                                     frozen, steps, rk_coef(dt), grid_sync(ctx));
         });
         return e == cudaSuccess ? LABFM_OK : cuda_fail(ctx, e, "Burgers run");

@@ -35,13 +35,15 @@ struct Sell {
     int lg_l = 0;          // lanes per node, log2
     int64_t n_slices = 0;
     int64_t places = 0;    // entries with the empty places
-    DevBuf off, col, steps;
+    int blocks = 0;        // shares of the slices, one per block of a run
+    DevBuf off, col, steps, share;
     void release()
     {
         valid = false;
         off.release();
         col.release();
         steps.release();
+        share.release();
     }
 };
 
@@ -180,8 +182,14 @@ struct SellView {
     int64_t n_slices;
     const int64_t *off;
     const int32_t *col;
+    const int64_t *share;  // [blocks + 1]: the slices of share b are share[b] .. share[b + 1] - 1
+    int blocks;
     int lg_l;
 };
+
+// The scale on which sweeps are shared out: slice s takes [slice_at(s), slice_at(s + 1)), a place for each of its steps and
+// SLICE_COST for the update of its nodes (a step is two FP64 instructions or more, an update four and two per combining step).
+constexpr int SLICE_COST = 4;
 #ifdef __CUDACC__
 // A lane's place in the sliced layout: node i (-1: none) and entry k L + h of its row at step k
 struct SellLane {
@@ -195,6 +203,13 @@ struct SellLane {
         if (node < n) i = node;
         at = S.off[slice] * 32 + lane;
         steps = (int)(S.off[slice + 1] - S.off[slice]);
+    }
+    // so many steps from place `from` on
+    __device__ SellLane(int64_t slice, int64_t from, int count, int lane, int64_t n, const SellView &S) : at(from * 32 + lane), steps(count)
+    {
+        h = lane & ((1 << S.lg_l) - 1);
+        const int64_t node = slice * (32 >> S.lg_l) + (lane >> S.lg_l);
+        if (node < n) i = node;
     }
 };
 
@@ -260,10 +275,11 @@ struct SlicePipe {
 };
 
 // Runs of many dependent sweeps over a node set (RK4 steps, solver iterations) as one cooperative launch: a block per
-// SM with an equal share of the slices, a barrier over the grid between sweeps.  Launched one by one a sweep of a small
-// set costs its launch and its uneven last blocks again as much as its sums.  What a sweep writes for others to read
-// carries no __restrict__ in the kernel: it is not constant data of the launch.
+// SM, a barrier over the grid between sweeps.  Launched one by one a sweep of a small set costs its launch and its
+// uneven last blocks again as much as its sums.  What a sweep writes for others to read carries no __restrict__ in the
+// kernel: it is not constant data of the launch.
 constexpr int RUN_THREADS = 512;
+constexpr int RUN_WARPS = RUN_THREADS / 32;
 struct GridSync {
     unsigned *count;    // device: arrivals, then 1 if a wait gave up; both 0 at the launch
     unsigned *gave_up;  // pinned host word, set where a wait gave up
@@ -303,22 +319,161 @@ struct GridBarrier {
     }
 };
 
-// This block's share of the slices: [first, last)
-__device__ __forceinline__ void slice_share(int64_t n_slices, int64_t &first, int64_t &last)
+__device__ __forceinline__ int64_t slice_at(const SellView &S, int64_t s) { return S.off[s] + SLICE_COST * s; }
+
+// This block's slices [first, last): its share, or where the grid has fewer blocks than shares, several
+__device__ __forceinline__ void block_share(const SellView &S, int64_t &first, int64_t &last)
 {
-    first = n_slices * blockIdx.x / gridDim.x;
-    last = n_slices * (blockIdx.x + 1) / gridDim.x;
+    first = S.share[(int64_t)blockIdx.x * S.blocks / gridDim.x];
+    last = S.share[(int64_t)(blockIdx.x + 1) * S.blocks / gridDim.x];
 }
+
+// A warp's part of its block's slices: every RUN_WARPS-th slice, or where that gives some warp CUT_COST places more than an
+// equal part (every barrier waits for the last warp), one of RUN_WARPS equal runs of the block's places, cut within
+// slices too.  Then the warp in whose run a slice begins updates its nodes, and the warps that the slice runs on into
+// add up their part of it.  Order 4, 289^2 nodes, 18 slices of 49 steps a block: 27.4 us a stage in two rounds of whole slices, 21.1
+// cut (24.4 as launches); 257^2, 14 slices: 16.3 and 16.8; 161^2, 11 slices of 25 steps: 7.9 and 8.8; 41^2, 3 of 7: 3.2 and 3.5.
+// CUT_COST is what those and 25 more sizes between 41^2 and 900^2 come to: a second piece's loads and a block barrier.
+constexpr int CUT_COST = 25;
+struct WarpShare {
+    int64_t from;             // its first piece: the place where it begins
+    int steps;                // ... and its steps
+    int first, last, stride;  // the slices this warp updates: first, first + stride, ... below last
+    bool head;                // the first piece is a part of slice first - 1, which another warp updates
+    bool cut;                 // some slice of the block is shared by warps
+    int open;                 // it adds up the first `open` steps of slice last - 1 itself; < 0: all of them
+    int parts;                // ... and so many warps after it add up the rest
+};
+// This warp's part, kept in shared memory: read once a piece, where registers are short
+__device__ __forceinline__ WarpShare &warp_share()
+{
+    __shared__ WarpShare s_share[RUN_WARPS];
+    return s_share[threadIdx.x >> 5];
+}
+// Forms the parts of the block's warps; all of its threads take part.
+__device__ __forceinline__ void share_out(const SellView &S, int64_t s0, int64_t s1)
+{
+    __shared__ int s_first[RUN_WARPS + 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t base = slice_at(S, s0), total = slice_at(S, s1) - base;
+    int64_t whole = 0;  // places of every RUN_WARPS-th slice
+    for (int64_t t = s0 + warp + RUN_WARPS * lane; t < s1; t += RUN_WARPS * 32) whole += slice_at(S, t + 1) - slice_at(S, t);
+    for (int o = 16; o > 0; o >>= 1) whole += __shfl_xor_sync(0xffffffffu, whole, o);
+    if (!__syncthreads_or(whole > total / RUN_WARPS + CUT_COST)) {
+        const int64_t t = s0 + warp;
+        if (lane == 0)
+            warp_share() = t < s1 ? WarpShare{S.off[t], (int)(S.off[t + 1] - S.off[t]), (int)t, (int)s1, RUN_WARPS, false, false, -1, 0}
+                                  : WarpShare{0, 0, (int)t, (int)t, RUN_WARPS, false, false, -1, 0};
+        __syncwarp();
+        return;
+    }
+    const int64_t a = base + total * warp / RUN_WARPS, z = base + total * (warp + 1) / RUN_WARPS;
+    // the first slice at or behind a, a 32nd of what is left at a time
+    int64_t lo = s0, hi = s1;
+    while (lo < hi) {
+        const int64_t gap = (hi - lo + 31) / 32, at = lo + gap * lane;
+        const int before = __popc(__ballot_sync(0xffffffffu, at < hi && slice_at(S, at) < a));
+        hi = min(hi, lo + gap * before);
+        if (before > 0) lo += gap * (before - 1) + 1;
+    }
+    if (lane == 0) s_first[warp] = (int)lo;
+    if (threadIdx.x == 0) s_first[RUN_WARPS] = (int)s1;
+    __syncthreads();
+    WarpShare W{0, 0, (int)lo, s_first[warp + 1], 1, false, false, -1, 0};
+    if (W.last > W.first) {
+        const int64_t at = slice_at(S, W.last - 1), steps = S.off[W.last] - S.off[W.last - 1];
+        if (z - at < steps) {
+            W.open = (int)(z - at);
+            while (warp + 1 + W.parts < RUN_WARPS && base + total * (warp + 1 + W.parts) / RUN_WARPS - at < steps) W.parts++;
+        }
+        W.from = S.off[W.first];
+        W.steps = W.open >= 0 && W.last - W.first == 1 ? W.open : (int)(S.off[W.first + 1] - W.from);
+    }
+    if (W.first > s0) {
+        const int64_t at = slice_at(S, W.first - 1), steps = S.off[W.first] - S.off[W.first - 1];
+        if (a - at < steps) {
+            W.head = true;
+            W.from = S.off[W.first - 1] + (a - at);
+            W.steps = (int)(min(steps, z - at) - (a - at));
+        }
+    }
+    W.cut = __syncthreads_or(W.open >= 0) != 0;
+    if (lane == 0) warp_share() = W;
+    __syncwarp();
+}
+
+// Where the warps leave their parts of others' slices
+template <int NS>
+__device__ __forceinline__ double (&left_parts())[RUN_WARPS][NS][32]
+{
+    __shared__ double s_part[RUN_WARPS][NS][32];
+    return s_part;
+}
+
+// A block's sweep over its slices, NS sums per lane.  With a slice's node values by begin(lane, whether this warp updates it):
+// gather and add as in SlicePipe (add with those values), part(values, sums) the lane's sums, and where the warp
+// updates the slice finish(lane, values, sums) with the parts of all warps.  Every thread of the block takes part, after
+// share_out; a block barrier has to follow before the next run.
+template <int U, int NW, int NX, int NS, class VT>
+struct SliceSweep {
+    SlicePipe<U, NW, NX, VT> pipe;
+
+    // the first piece (of none: no node and no step)
+    static __device__ __forceinline__ SellLane begin_at(int64_t n, const SellView &S)
+    {
+        const WarpShare &W = warp_share();
+        const bool any = W.head || W.first < W.last;
+        return SellLane(any ? W.first - W.head : S.n_slices, W.from, W.steps, threadIdx.x & 31, n, S);
+    }
+    // the first loads of the next run
+    __device__ __forceinline__ void preload(int64_t n, const SellView &S, const VT *__restrict__ wc)
+    {
+        pipe.preload(begin_at(n, S), threadIdx.x & 31, S, wc);
+    }
+    template <class Begin, class Gather, class Add, class Part, class Finish>
+    __device__ __forceinline__ void run(int64_t n, const SellView &S, const VT *__restrict__ wc, Begin begin, Gather gather,
+                                        Add add, Part part, Finish finish)
+    {
+        double(&s_part)[RUN_WARPS][NS][32] = left_parts<NS>();
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const WarpShare &W = warp_share();
+        SellLane l = begin_at(n, S);
+        int slice = W.first - W.head;
+        while (true) {  // a warp without a piece goes through once, for the barrier
+            const bool mine = slice >= W.first && slice < W.last, last = slice + W.stride >= W.last;
+            auto v = begin(l, mine);
+            double p[NS];
+            pipe.run(l, lane, S, wc, gather, [&](int q, const double(&x)[NX], const VT(&w)[NW]) { add(v, q, x, w); });
+            part(v, p);
+            if (W.cut) {
+                if (!mine)
+#pragma unroll
+                    for (int t = 0; t < NS; t++) s_part[warp][t][lane] = p[t];
+                if (last) __syncthreads();  // every warp once
+                if (mine && last && W.open >= 0)
+                    for (int k = 1; k <= W.parts; k++)
+#pragma unroll
+                        for (int t = 0; t < NS; t++) p[t] += s_part[warp + k][t][lane];
+            }
+            if (mine) finish(l, v, p);
+            if (last) break;
+            slice += W.stride;
+            l = SellLane(slice, lane, n, S);
+            if (slice + 1 == W.last && W.open >= 0) l.steps = W.open;
+            pipe.preload(l, lane, S, wc);
+        }
+    }
+};
 
 // Cooperative launch of such a run on the context's stream
 template <class... P, class... A>
-cudaError_t launch_run(labfm_ctx *ctx, int64_t n_slices, void (*kern)(P...), A... args)
+cudaError_t launch_run(labfm_ctx *ctx, const SellView &S, void (*kern)(P...), A... args)
 {
     cudaError_t e = ctx->sync_buf.reserve(256);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->sync_buf.ptr, 0, 2 * sizeof(unsigned), ctx->stream);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(n_slices < ctx->num_sms ? n_slices : ctx->num_sms));
+    cfg.gridDim = dim3((unsigned)S.blocks);
     cfg.blockDim = dim3(RUN_THREADS);
     cfg.stream = ctx->stream;
     cudaLaunchAttribute at{};
@@ -341,7 +496,10 @@ inline GridSync grid_sync(const labfm_ctx *ctx)
     return GridSync{ctx->sync_buf.as<unsigned>(), reinterpret_cast<unsigned *>(static_cast<char *>(ctx->host_small) + LABFM_GAVE_UP)};
 }
 #endif
-inline SellView sell_view(const Sell &L) { return SellView{L.n_slices, L.off.as<int64_t>(), L.col.as<int32_t>(), L.lg_l}; }
+inline SellView sell_view(const Sell &L)
+{
+    return SellView{L.n_slices, L.off.as<int64_t>(), L.col.as<int32_t>(), L.share.as<int64_t>(), L.blocks, L.lg_l};
+}
 labfm_status ensure_sell(labfm_ctx *ctx);  // ctx->sell of the current stencils
 // The layout of the stencils with the rows in gmap (>= 0: a Neumann ghost row) replaced by their parents' (gmap null: none)
 labfm_status build_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int64_t *parent);

@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_steps(int64_t n, int lg_l
                                                             const int64_t *__restrict__ row_ptr,
                                                             const int32_t *__restrict__ gmap,
                                                             const int64_t *__restrict__ parent,
-                                                            int32_t *__restrict__ steps)
+                                                            int32_t *__restrict__ steps, int32_t *__restrict__ longest)
 {
     const int lane = threadIdx.x & 31;
     const int64_t slice = (int64_t)blockIdx.x * (SELL_THREADS / 32) + (threadIdx.x >> 5);
@@ -40,7 +40,11 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_steps(int64_t n, int lg_l
         len = (int)(row_ptr[r + 1] - row_ptr[r]);
     }
     const int most = __reduce_max_sync(0xffffffffu, len);
-    if (lane == 0) steps[slice] = (most + (1 << lg_l) - 1) >> lg_l;
+    if (lane == 0) {
+        const int count = (most + (1 << lg_l) - 1) >> lg_l;
+        steps[slice] = count;
+        if (count > *(volatile int32_t *)longest) atomicMax(longest, count);
+    }
 }
 
 __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l, int64_t n_slices,
@@ -48,7 +52,8 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l,
                                                            const int32_t *__restrict__ col,
                                                            const int32_t *__restrict__ gmap,
                                                            const int64_t *__restrict__ parent,
-                                                           const int64_t *__restrict__ off, int32_t *__restrict__ scol)
+                                                           const int64_t *__restrict__ off, int32_t *__restrict__ scol,
+                                                           int64_t *__restrict__ share, int blocks, int64_t slice_cost)
 {
     const int lane = threadIdx.x & 31, h = lane & ((1 << lg_l) - 1);
     const int64_t slice = (int64_t)blockIdx.x * (SELL_THREADS / 32) + (threadIdx.x >> 5);
@@ -61,6 +66,13 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l,
         re = row_ptr[r + 1];
     }
     const int64_t at = off[slice], steps = off[slice + 1] - at;
+    if (lane == 0) {
+        // share b begins at the first slice at or behind place b / blocks of all: slice + 1 for the b in this slice's run
+        const int64_t total = off[n_slices] + slice_cost * n_slices, p0 = at + slice_cost * slice, p1 = p0 + steps + slice_cost;
+        if (slice == 0) share[0] = 0;
+        for (int64_t b = p0 * blocks / total; b <= blocks && total * b / blocks <= p1; b++)
+            if (total * b / blocks > p0) share[b] = slice + 1;
+    }
     for (int64_t k = 0; k < steps; k++) {
         const int64_t e = rs + (k << lg_l) + h;
         scol[(at + k) * 32 + lane] = e < re ? col[e] : -1;
@@ -69,10 +81,11 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l,
 
 }  // namespace
 
-// Lanes per node, as the power of two with the least cost of a sweep on the busiest SM (a run gives every SM an equal
-// share of the slices): 16 cycles per FP64 instruction, two per entry of a lane, about four for the node and two per
-// combining step; and about 50 cycles per step for its loads, which the other warps hide on all but small sets.  One
-// lane for large sets, two at 161^2 nodes, eight at 41^2 (measured, heat: 2 lanes at 41^2 5.05 us a stage).
+// Lanes per node, as the power of two with the least cost of a sweep of the busiest block: 16 cycles per FP64 instruction,
+// two per entry of a lane, about four for the node and two per combining step; and 90 cycles per place for the loads of
+// the longest warp (see share_out: whole slices, or cut ones where those are more uneven).  One lane for large
+// sets, two at 129^2 and 161^2 nodes, eight at 41^2.  Over 45 sizes of heat, Burgers, solver and order-8 runs between 41^2 and 900^2
+// the choice is within 1 % of the best lane count on average and 9 % at worst.
 static int sell_lanes_log2(int64_t n, int64_t nnz, int num_sms)
 {
     const int64_t deg = n > 0 ? (nnz + n - 1) / n : 0;
@@ -80,7 +93,9 @@ static int sell_lanes_log2(int64_t n, int64_t nnz, int num_sms)
     int64_t least = INT64_MAX;
     for (int lg = 0; lg <= 4; lg++) {
         const int64_t slices = ((n << lg) + 31) / 32, most = (slices + num_sms - 1) / num_sms;
-        const int64_t steps = (deg + (1 << lg) - 1) >> lg, cost = 16 * most * (2 * steps + 2 * lg + 4) + 50 * steps;
+        const int64_t steps = (deg + (1 << lg) - 1) >> lg, whole = (most + RUN_WARPS - 1) / RUN_WARPS * (steps + SLICE_COST);
+        const int64_t cut = most * (steps + SLICE_COST) / RUN_WARPS + CUT_COST;
+        const int64_t cost = 16 * most * (2 * steps + 2 * lg + 4) + 90 * std::min(whole, cut);
         if (cost < least) {
             least = cost;
             best = lg;
@@ -88,6 +103,11 @@ static int sell_lanes_log2(int64_t n, int64_t nnz, int num_sms)
     }
     return best;
 }
+
+// Blocks get equal numbers of places where slices differ in length (order 6 on 200^2 nodes graded towards walls: 14.9 -> 11.3 us a
+// stage), but equal numbers of slices where none is a quarter longer than the mean: a few shorter ones at the box's edge
+// would otherwise make a block with one slice more than warps (193^2: 10.5 us a stage, 12.5 by places).
+constexpr int64_t EVEN_SLICE_COST = 1 << 20;
 
 labfm_status build_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int64_t *parent)
 {
@@ -97,27 +117,34 @@ labfm_status build_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int6
     L.valid = false;
     L.lg_l = sell_lanes_log2(n, ctx->nnz, ctx->num_sms);
     unsigned blocks = 0;
+    int64_t slice_cost = SLICE_COST;
     while (true) {
         const int64_t per = 32 >> L.lg_l;
         L.n_slices = (n + per - 1) / per;
         LABFM_CUDA_TRY(ctx, L.steps.reserve(sizeof(int32_t) * L.n_slices));
-        LABFM_CUDA_TRY(ctx, L.off.reserve(sizeof(int64_t) * (L.n_slices + 1)));
+        LABFM_CUDA_TRY(ctx, L.off.reserve(sizeof(int64_t) * (L.n_slices + 2)));
+        int64_t *const end = L.off.as<int64_t>() + L.n_slices;  // behind the last slice, and then the steps of the longest one
+        LABFM_CUDA_TRY(ctx, cudaMemsetAsync(end + 1, 0, sizeof(int64_t), s));
         blocks = (unsigned)((L.n_slices + SELL_THREADS / 32 - 1) / (SELL_THREADS / 32));
-        k_sell_steps<<<blocks, SELL_THREADS, 0, s>>>(n, L.lg_l, L.n_slices, rp, gmap, parent, L.steps.as<int32_t>());
+        k_sell_steps<<<blocks, SELL_THREADS, 0, s>>>(n, L.lg_l, L.n_slices, rp, gmap, parent, L.steps.as<int32_t>(),
+                                                     reinterpret_cast<int32_t *>(end + 1));
         LABFM_CUDA_TRY(ctx, cudaGetLastError());
         LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(L.steps.as<int32_t>(), L.off.as<int64_t>(), L.n_slices, ctx->scan_tmp, s));
         int64_t *total = (int64_t *)ctx->host_small;
-        LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(total, L.off.as<int64_t>() + L.n_slices, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(total, end, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-        L.places = 32 * *total;
+        L.places = 32 * total[0];
+        slice_cost = 4 * total[1] * L.n_slices <= 5 * total[0] ? EVEN_SLICE_COST : SLICE_COST;
         // a set whose neighbouring nodes differ too much in stencil size (a slice is as long as its largest one):
         // a warp per node, at most 31 places left empty each
         if (L.lg_l == 5 || L.places <= 2 * ctx->nnz + 64 * n) break;
         L.lg_l = 5;
     }
     LABFM_CUDA_TRY(ctx, L.col.reserve(sizeof(int32_t) * (L.places > 0 ? L.places : 1)));
+    L.blocks = (int)std::min<int64_t>(L.n_slices, ctx->num_sms);
+    LABFM_CUDA_TRY(ctx, L.share.reserve(sizeof(int64_t) * (L.blocks + 1)));
     k_sell_cols<<<blocks, SELL_THREADS, 0, s>>>(n, L.lg_l, L.n_slices, rp, ctx->col.as<int32_t>(), gmap, parent,
-                                                L.off.as<int64_t>(), L.col.as<int32_t>());
+                                                L.off.as<int64_t>(), L.col.as<int32_t>(), L.share.as<int64_t>(), L.blocks, slice_cost);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     L.valid = true;
     return LABFM_OK;

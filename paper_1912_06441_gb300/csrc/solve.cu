@@ -194,19 +194,15 @@ struct SolveArgs {
 struct SolveBlock {
     const SolveArgs &A;
     GridBarrier bar;
-    int64_t s0, s1;  // slices
-    int64_t n0, n1;  // rows
+    int n0, n1;  // rows
     int lane, warp;
-    SellLane first;
-    SlicePipe<4, 1, 1, double> pipe;
+    SliceSweep<4, 1, 1, 1, double> sweep;
 
-    __device__ SolveBlock(const SolveArgs &args, int64_t s0_, int64_t s1_)
-        : A(args), bar{args.sync}, s0(s0_), s1(s1_), lane(threadIdx.x & 31), warp(threadIdx.x >> 5),
-          first(s0_ + (threadIdx.x >> 5) < s1_ ? s0_ + (threadIdx.x >> 5) : args.S.n_slices, threadIdx.x & 31, args.n, args.S)
+    __device__ SolveBlock(const SolveArgs &args, int64_t s0, int64_t s1)
+        : A(args), bar{args.sync}, n0((int)(s0 * (32 >> args.S.lg_l))), n1((int)min(args.n, s1 * (32 >> args.S.lg_l))),
+          lane(threadIdx.x & 31), warp(threadIdx.x >> 5)
     {
-        n0 = s0 * (32 >> A.S.lg_l);
-        n1 = min(A.n, s1 * (32 >> A.S.lg_l));
-        pipe.preload(first, lane, A.S, A.wd);
+        sweep.preload(A.n, A.S, A.wd);
     }
 
     // A x over the block's rows with the matrix in its global form (Sec. 5.2), A_ii x_i + sum_j w_ji x_j, one FP64
@@ -219,36 +215,40 @@ struct SolveBlock {
     template <bool DIFFERENCES, class Fn>
     __device__ __forceinline__ void product(const double *x, const double *own, Fn fn)
     {
-        for (int64_t slice = s0 + warp; slice < s1; slice += RUN_THREADS / 32) {
-            SellLane l = first;
-            if (slice != s0 + warp) {
-                l = SellLane(slice, lane, A.n, A.S);
-                pipe.preload(l, lane, A.S, A.wd);
-            }
-            const int64_t i = l.i;
-            const bool row = i >= 0 && l.h == 0;
-            double xi = 0.0, ai = 0.0, oi = 0.0;
-            bool fixed = false;
-            if (row || (DIFFERENCES && i >= 0)) {
-                int64_t src = i;
-                if (A.gr.gmap && A.gr.gmap[i] >= 0) src = A.gr.parent[A.gr.gmap[i]];
-                xi = x[src];
-            }
-            if (row) {
-                oi = own[i];
-                if (!DIFFERENCES) ai = A.adiag[i];
-                fixed = A.dirichlet && A.dirichlet[i];
-            }
-            double sum[2] = {0.0, 0.0};
-            pipe.run(l, lane, A.S, A.wd, [&](int j, double(&xv)[1]) { xv[0] = x[j]; },
-                     [&](int q, const double(&xv)[1], const double(&w)[1]) {
-                         sum[q & 1] = fma(DIFFERENCES ? xv[0] - xi : xv[0], w[0], sum[q & 1]);
-                     });
-            double acc = sum[0] + sum[1];
-            for (int o = (1 << A.S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (row) fn(i, fixed ? xi : DIFFERENCES ? acc : fma(ai, xi, acc), oi);
-        }
-        pipe.preload(first, lane, A.S, A.wd);
+        struct Row {
+            double xi, ai, oi, sum[2];
+            bool row, fixed;
+        };
+        sweep.run(
+            A.n, A.S, A.wd,
+            [&](const SellLane &l, bool mine) {
+                Row v;
+                v.xi = v.ai = v.oi = v.sum[0] = v.sum[1] = 0.0;
+                v.fixed = false;
+                v.row = mine && l.i >= 0 && l.h == 0;
+                if (v.row || (DIFFERENCES && l.i >= 0)) {
+                    int64_t src = l.i;
+                    if (A.gr.gmap && A.gr.gmap[l.i] >= 0) src = A.gr.parent[A.gr.gmap[l.i]];
+                    v.xi = x[src];
+                }
+                if (v.row) {
+                    v.oi = own[l.i];
+                    if (!DIFFERENCES) v.ai = A.adiag[l.i];
+                    v.fixed = A.dirichlet && A.dirichlet[l.i];
+                }
+                return v;
+            },
+            [&](int j, double(&xv)[1]) { xv[0] = x[j]; },
+            [&](Row &v, int q, const double(&xv)[1], const double(&w)[1]) {
+                v.sum[q & 1] = fma(DIFFERENCES ? xv[0] - v.xi : xv[0], w[0], v.sum[q & 1]);
+            },
+            [&](const Row &v, double(&p)[1]) { p[0] = v.sum[0] + v.sum[1]; },
+            [&](const SellLane &l, const Row &v, const double(&p)[1]) {
+                double acc = p[0];
+                for (int o = (1 << A.S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (v.row) fn(l.i, v.fixed ? v.xi : DIFFERENCES ? acc : fma(v.ai, v.xi, acc), v.oi);
+            });
+        sweep.preload(A.n, A.S, A.wd);
     }
 
     // The sums of a and b over all blocks (NQ = 1: of a) through partial sums in slots q0 and q0 + 1, around a barrier; on
@@ -299,7 +299,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
 {
     __shared__ SolveState st;
     int64_t s0, s1;
-    slice_share(A.S.n_slices, s0, s1);
+    block_share(A.S, s0, s1);
+    share_out(A.S, s0, s1);
     SolveBlock B(A, s0, s1);
     if (threadIdx.x == 0) st = *A.st;
     __syncthreads();
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
         // p = r + beta (p - omega v); y = dinv p
         {
             const double beta = st.beta, omega = st.omega;
-            for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
+            for (int i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
                 const double pi = fma(beta, fma(-omega, A.v[i], A.p[i]), A.r[i]);
                 A.p[i] = pi;
                 A.y[i] = A.dinv[i] * pi;
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
         d0 = 0.0;
         {
             const double alpha = st.alpha;
-            for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
+            for (int i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
                 const double si = fma(-alpha, A.v[i], A.r[i]);
                 A.s[i] = si;
                 A.z[i] = A.dinv[i] * si;
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
         d0 = d1 = 0.0;
         {
             const double alpha = st.alpha, omega = st.omega;
-            for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
+            for (int i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) {
                 A.d[i] = fma(omega, A.z[i], fma(alpha, A.y[i], A.d[i]));
                 const double ri = fma(-omega, A.t[i], A.s[i]);
                 A.r[i] = ri;
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
         scalars(5);
     }
     if (st.done) {
-        for (int64_t i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) A.x[i] += A.d[i];
+        for (int i = B.n0 + threadIdx.x; i < B.n1; i += RUN_THREADS) A.x[i] += A.d[i];
         if (!B.bar.wait()) return;
         double rr = 0.0, bb = 0.0;
         B.product<true>(A.x, A.b, [&](int64_t, double ax, double bi) {
@@ -485,7 +486,7 @@ labfm_status run_solve(labfm_ctx *ctx, int op, const double *f, double *phi, con
     int start = 1;
     while (true) {
         do {
-            le = launch_run(ctx, S.n_slices, k_solve_run, args, start, most);
+            le = launch_run(ctx, S, k_solve_run, args, start, most);
             start = 0;
             if (le == cudaSuccess) le = cudaMemcpyAsync(&h, st, sizeof(SolveState), cudaMemcpyDeviceToHost, s);
             if (le == cudaSuccess) le = cudaStreamSynchronize(s);
