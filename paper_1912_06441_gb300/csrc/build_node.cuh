@@ -100,6 +100,7 @@ template <int P> struct NodeShared {
     double inv;
     int flag;                    // bit 0: zero/non-finite pivot, bit 1: non-finite weight, bit 2: non-finite M
     unsigned char perm[2][P];    // the elimination's rows by position (two lists, alternating)
+    unsigned ratios[BUILD_THREADS / 32];  // each warp's neighbours, see ratio_bit
 };
 
 // The CTA's dynamic shared memory (four CTAs fit an SM); a CTA of NG = 256 / G groups gives each group
@@ -333,6 +334,15 @@ __device__ __forceinline__ void offset_of(const BuildArgs &A, int64_t e, double 
     }
 }
 
+// A set of neighbours with |y| = 2^e |x| for one e (on a diagonal, say) has rows of X that are equal up to a power of two:
+// M is singular, and from X and W comes out so, its pivot exactly zero.  The products x^s y^t of the moments round
+// apart, so such sets are told by their offsets: bit e + 15 for a ratio 2^e, two bits for any other.
+__device__ __forceinline__ unsigned ratio_bit(double x, double y)
+{
+    const int r = (__double2hiint(x) & 0x7fffffff) - (__double2hiint(y) & 0x7fffffff), e = (r >> 20) + 15;
+    return __double2loint(x) == __double2loint(y) && (r & 0xfffff) == 0 && (unsigned)e <= 30u ? 1u << e : 3u;
+}
+
 // One neighbour at offset (x, y) in units of 2h (so every monomial is at most 1): what the weights need of it
 // into keep[], and with ROW its staged row for the moment sums.
 template <int K, bool CH, bool ROW>
@@ -465,12 +475,14 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
             for (int q = 0; q < C::ACC; q++)
 #pragma unroll
                 for (int f = 0; f < NS; f++) acc[q][f] = 0.0;
+            unsigned ratios = 0;
             for (int ch = 0; ch < nchunks; ch++) {
                 const int j0 = ch * NB, nj = min(NB, ni - j0);
                 if (ch > 0) gsync<G>(bar);
                 for (int t = tid; t < nj; t += G) {
                     double dx, dy;
                     offset_of(A, rs + j0 + t, xi, yi, dx, dy);
+                    ratios |= ratio_bit(dx, dy);
                     stage_neighbour<K, CH, true>(dx * ihalf, dy * ihalf, A.rbf, rows + t * M::LD, keep + t * M::LP);
                 }
                 gsync<G>(bar);
@@ -499,6 +511,8 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
                     }
                 }
             }
+            ratios = __reduce_or_sync(0xffffffffu, ratios);
+            if ((tid & 31) == 0) sh.ratios[tid >> 5] = ratios;
             gsync<G>(bar);
             // the two parts' sums, over the staged rows
             if (sy >= 0) {
@@ -752,7 +766,14 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
             }
             gsync<G>(bar);
         }
-        const bool singular = (s_flag & 5) != 0;  // no weights from a failed elimination
+        bool one_ratio = false;
+        if constexpr (C::MOMENTS) {
+            unsigned ratios = 0;
+#pragma unroll
+            for (int w = 0; w < G / 32; w++) ratios |= sh.ratios[w];
+            one_ratio = __popc(ratios) == 1;
+        }
+        const bool singular = (s_flag & 5) != 0 || one_ratio;  // no weights from a failed elimination
         for (int t = tid; t < P * n_ops; t += G) {
             const int m = t / n_ops, d = t - m * n_ops;
             double v = 0.0;  // a non-finite M gives no weights, and no position list is formed
@@ -828,7 +849,7 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
         }
         if (tid == 0) {
             int st = (flag & 4)   ? LABFM_NODE_NONFINITE
-                     : (flag & 1) ? LABFM_NODE_SINGULAR
+                     : (flag & 1) || one_ratio ? LABFM_NODE_SINGULAR
                      : (flag & 2) ? LABFM_NODE_NONFINITE
                                   : LABFM_NODE_OK;
             if (A.node_status) A.node_status[i] = st;
