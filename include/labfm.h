@@ -241,9 +241,12 @@ labfm_status labfm_apply(labfm_ctx *ctx, uint32_t op_mask, const void *f, int fi
  * Nodes with frozen[i] != 0 keep their value
  * (Dirichlet nodes, Sec. 5.1).  On FP64 fields the steps run in cooperative launches (a block
  * per SM, a barrier over them between stages) on a layout of the stencils that the first
- * such call after labfm_build_neighbours makes; a barrier that gives up (after about a second)
- * makes the context's next call that reads weights return LABFM_ERR_TIMEOUT, the field is then
- * undefined.  On FP32 fields the nsteps x 4 stage launches are recorded once into a
+ * such call after labfm_build_neighbours makes.  A barrier that gives up (after 2^21 reads of its
+ * count, of the order of a second) ends the run, its field is then undefined, and runs enqueued
+ * behind it leave their fields as they are, until a call has reported it: that call does nothing
+ * else and returns LABFM_ERR_TIMEOUT.  It is the first call to apply, step or solve after the run
+ * has ended on the device, or a search, build or solve that waited for it.  labfm_step with
+ * nsteps 0 after a synchronisation of the stream only asks.  On FP32 fields the nsteps x 4 stage launches are recorded once into a
  * CUDA graph and replayed; it is recorded again when an argument other than beta, the
  * stencil count or size, the weight type or a context buffer changes.  There the stage's launch
  * shape is tuned as for labfm_apply, on first-stage launches that read u and write only
@@ -289,8 +292,8 @@ labfm_status labfm_step_burgers(labfm_ctx *ctx, const double *beta, void *u, voi
  * stencil sums over the context's stencils.  Stabilised bi-conjugate gradients (van der Vorst
  * 1992) with a Jacobi preconditioner (diag A), as in Sec. 5.2; all vectors and scalars in FP64 and
  * in device memory, up to 256 iterations in one cooperative launch (a block per SM, barriers over
- * them as in labfm_step; LABFM_ERR_TIMEOUT if one gives up) with one host read of the state
- * per launch.
+ * them as in labfm_step; LABFM_ERR_TIMEOUT if one gives up, phi is then undefined) with one host
+ * read of the state per launch.
  * Stops when the recurrence residual ||r|| <= tol ||F||, or after max_iter iterations.  The
  * recurrence residual drifts from the true one ||F - A Phi|| in finite precision, so the true
  * residual is then formed; if it is above tol, the iteration restarts from the current Phi

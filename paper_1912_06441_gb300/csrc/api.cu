@@ -240,7 +240,10 @@ labfm_status labfm_build_neighbours(labfm_ctx *ctx, int64_t n, const double *xy,
     ctx->have_weights = false;
     ctx->wcomb_valid = false;
     ctx->sell.valid = false;
-    return run_neighbours(ctx, n, xy, h, periodic ? 1 : 0, box_lo, box_hi, nnz_out);
+    const labfm_status st = run_neighbours(ctx, n, xy, h, periodic ? 1 : 0, box_lo, box_hi, nnz_out);
+    const labfm_status rs = run_gave_up(ctx);  // (every run has ended: the search waited for the stream)
+    if (rs != LABFM_OK) ctx->n = 0;            // its positions may come from that run
+    return rs != LABFM_OK ? rs : st;
 }
 
 labfm_status labfm_get_neighbours(labfm_ctx *ctx, const int64_t **row_ptr, const int32_t **col, int64_t *n,
@@ -287,6 +290,7 @@ labfm_status labfm_build_weights(labfm_ctx *ctx, const int8_t *order, int unifor
     ctx->wburg_valid = false;
     labfm_status st =
         run_build(ctx, order, uniform_order, rbf, n_ops, C, precision, weight_dtype, node_status, n_bad_out);
+    if (const labfm_status rs = run_gave_up(ctx)) return rs;
     if (st == LABFM_OK || st == LABFM_ERR_SINGULAR) {
         ctx->have_weights = true;
         ctx->n_ops = n_ops;
@@ -329,7 +333,7 @@ labfm_status labfm_apply(labfm_ctx *ctx, uint32_t op_mask, const void *f, int fi
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
-    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
+    if (const labfm_status rs = run_gave_up(ctx)) return rs;
     if (!f || !out) return fail(ctx, LABFM_ERR_ARG, "null field or output");
     if (field_dtype != LABFM_F64 && field_dtype != LABFM_F32) return fail(ctx, LABFM_ERR_ARG, "bad field_dtype");
     if (op_mask == 0 || (op_mask >> ctx->n_ops) != 0) return fail(ctx, LABFM_ERR_ARG, "op_mask selects no or unknown operators");
@@ -344,7 +348,7 @@ labfm_status labfm_step(labfm_ctx *ctx, const double *beta, void *u, int field_d
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
-    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
+    if (const labfm_status rs = run_gave_up(ctx)) return rs;
     if (!beta || !u) return fail(ctx, LABFM_ERR_ARG, "null beta or u");
     if (field_dtype != LABFM_F64 && field_dtype != LABFM_F32) return fail(ctx, LABFM_ERR_ARG, "bad field_dtype");
     if (!std::isfinite(dt) || nsteps < 0) return fail(ctx, LABFM_ERR_ARG, "dt must be finite and nsteps >= 0");
@@ -360,7 +364,7 @@ labfm_status labfm_solve(labfm_ctx *ctx, int op, const double *f, double *phi, c
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
-    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
+    if (const labfm_status rs = run_gave_up(ctx)) return rs;
     if (op < 0 || op >= ctx->n_ops) return fail(ctx, LABFM_ERR_ARG, "op must index a built operator");
     if (!f || !phi) return fail(ctx, LABFM_ERR_ARG, "null f or phi");
     if ((const void *)f == (const void *)phi) return fail(ctx, LABFM_ERR_ARG, "f and phi must be distinct buffers");
@@ -375,7 +379,7 @@ labfm_status labfm_solve_neumann(labfm_ctx *ctx, int op, const double *f, double
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
-    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
+    if (const labfm_status rs = run_gave_up(ctx)) return rs;
     if (op < 0 || op >= ctx->n_ops) return fail(ctx, LABFM_ERR_ARG, "op must index a built operator");
     if (!f || !phi) return fail(ctx, LABFM_ERR_ARG, "null f or phi");
     if ((const void *)f == (const void *)phi) return fail(ctx, LABFM_ERR_ARG, "f and phi must be distinct buffers");
@@ -402,7 +406,7 @@ labfm_status labfm_step_burgers(labfm_ctx *ctx, const double *beta, void *u, voi
     if (!ctx) return LABFM_ERR_ARG;
     ctx->err.clear();
     if (!ctx->have_weights) return fail(ctx, LABFM_ERR_STATE, "labfm_build_weights must come first");
-    if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: its fields are not valid");
+    if (const labfm_status rs = run_gave_up(ctx)) return rs;
     if (!ctx->grad01) return fail(ctx, LABFM_ERR_ARG, "operators 0 and 1 of the weights must be d/dx and d/dy");
     if (!beta || !u || !v) return fail(ctx, LABFM_ERR_ARG, "null beta, u or v");
     if (u == v) return fail(ctx, LABFM_ERR_ARG, "u and v must be distinct buffers");

@@ -316,11 +316,13 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView 
     int64_t s0, s1;
     block_share(S, s0, s1);
     GridBarrier bar{sync};
+    bar.check();
     struct Node {
         double si, ui, ai, sum[2];
         bool row, fixed;  // row: this lane updates the node; what it needs is read ahead
     };
     share_out(S, s0, s1);
+    if (bar.stopped()) return;
     SliceSweep<4, 1, 1, 1, VT> sweep;
     sweep.preload(n, S, wc);
     for (int64_t it = 0; it < 4 * nsteps; it++) {
@@ -623,12 +625,12 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
     if (cw_sliced(fmt)) {
         double *uu = (double *)u, *acc = ctx->rk_acc.as<double>(), *sa = ctx->rk_stage_a.as<double>(), *sb = ctx->rk_stage_b.as<double>();
         const SellView S = sell_view(ctx->sell);
-        LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
+        LABFM_CUDA_TRY(ctx, ensure_sync(ctx));
         cudaError_t e = enqueue_runs(ctx, nsteps, [&](int64_t steps) {
             return fmt == CW_S64 ? launch_run(ctx, S, k_rk4_run<double>, n, S, ctx->wcomb.as<double>(), uu, acc, sa, sb,
-                                              frozen, steps, rk_coef(dt), grid_sync(ctx))
+                                              frozen, steps, rk_coef(dt), grid_sync(ctx, LABFM_GAVE_UP))
                                  : launch_run(ctx, S, k_rk4_run<float>, n, S, ctx->wcomb.as<float>(), uu, acc, sa, sb,
-                                              frozen, steps, rk_coef(dt), grid_sync(ctx));
+                                              frozen, steps, rk_coef(dt), grid_sync(ctx, LABFM_GAVE_UP));
         });
         return e == cudaSuccess ? LABFM_OK : cuda_fail(ctx, e, "RK4 run");
     }
@@ -820,11 +822,13 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellV
     int64_t s0, s1;
     block_share(S, s0, s1);
     GridBarrier bar{sync};
+    bar.check();
     struct Node {
         double s[2], u0[2], a0[2], f[2];
         bool row, fixed;
     };
     share_out(S, s0, s1);
+    if (bar.stopped()) return;
     SliceSweep<2, 3, 2, 2, VT> sweep;
     sweep.preload(n, S, wb);
     for (int64_t it = 0; it < 4 * nsteps; it++) {
@@ -979,13 +983,13 @@ labfm_status run_step_burgers(labfm_ctx *ctx, const double *beta, void *u, void 
         double *uu = (double *)u, *vv = (double *)v, *acc = ctx->bu_acc.as<double>();
         double *sa = ctx->bu_stage_a.as<double>(), *sb = ctx->bu_stage_b.as<double>();
         const SellView S = sell_view(ctx->sell);
-        LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
+        LABFM_CUDA_TRY(ctx, ensure_sync(ctx));
         cudaError_t e = enqueue_runs(ctx, nsteps, [&](int64_t steps) {
             return ctx->wdtype == LABFM_F64
                        ? launch_run(ctx, S, k_burgers_run<double>, n, S, ctx->wburg.as<double>(), uu, vv, acc, sa, sb,
-                                    frozen, steps, rk_coef(dt), grid_sync(ctx))
+                                    frozen, steps, rk_coef(dt), grid_sync(ctx, LABFM_GAVE_UP))
                        : launch_run(ctx, S, k_burgers_run<float>, n, S, ctx->wburg.as<float>(), uu, vv, acc, sa, sb,
-                                    frozen, steps, rk_coef(dt), grid_sync(ctx));
+                                    frozen, steps, rk_coef(dt), grid_sync(ctx, LABFM_GAVE_UP));
         });
         return e == cudaSuccess ? LABFM_OK : cuda_fail(ctx, e, "Burgers run");
     }

@@ -65,7 +65,8 @@ struct StepGraph {
 
 }  // namespace labfm
 
-constexpr int LABFM_GAVE_UP = 1000;  // byte of the context's host words
+// Bytes of the context's host words: a wait of a run (a solve) gave up
+constexpr int LABFM_GAVE_UP = 1000, LABFM_SOLVE_GAVE_UP = 1004;
 
 struct labfm_ctx {
     int device = 0;
@@ -81,7 +82,7 @@ struct labfm_ctx {
     labfm::DevBuf node_xy, node_h;  // context copies of the node positions and h
     labfm::DevBuf row_ptr, col;
     labfm::Sell sell;  // of these stencils, for the FP64 products
-    labfm::DevBuf sync_buf;  // barrier counter of the cooperative runs
+    labfm::DevBuf sync_buf;  // barrier words of the cooperative runs
     // scratch of the neighbour search
     labfm::DevBuf cell_of, cell_count, cell_start, cell_nodes, counts, scan_tmp, misc;
 
@@ -126,7 +127,7 @@ struct labfm_ctx {
     // key (kind, n_ops, dtypes, size class of n, mean stencil size) -> (G << 8) | UNR
     std::unordered_map<uint64_t, uint32_t> tuned;
 
-    // pinned host words for status read-back; at byte LABFM_GAVE_UP: a barrier of an earlier run gave up
+    // pinned host words for status read-back; at bytes LABFM_GAVE_UP, LABFM_SOLVE_GAVE_UP: a barrier gave up
     void *host_small = nullptr;
 };
 
@@ -281,14 +282,31 @@ struct SlicePipe {
 constexpr int RUN_THREADS = 512;
 constexpr int RUN_WARPS = RUN_THREADS / 32;
 struct GridSync {
-    unsigned *count;    // device: arrivals, then 1 if a wait gave up; both 0 at the launch
+    unsigned *count;    // device: arrivals, 0 at the launch; then 1 once a wait gave up, until the host has reported it
     unsigned *gave_up;  // pinned host word, set where a wait gave up
 };
-constexpr unsigned SYNC_POLLS = 1u << 21;  // about a second
+// Reads of the count that a wait makes before it gives up: of the order of a second.  Set at compile time for tests (a
+// limit that came with the launch cost 0.05 to 0.1 us a barrier).
+#ifndef LABFM_SYNC_POLLS
+#define LABFM_SYNC_POLLS (1u << 21)
+#endif
+constexpr unsigned SYNC_POLLS = LABFM_SYNC_POLLS;
 
 struct GridBarrier {
     GridSync g;
     unsigned target = 0;
+    // Whether an earlier run, or a block of this one, gave up: the fields are not valid, and the run leaves them as they
+    // are.  check comes before a block barrier, stopped behind it.
+    static __device__ __forceinline__ int &stop_word()
+    {
+        __shared__ int s_stop;
+        return s_stop;
+    }
+    __device__ __forceinline__ void check() const
+    {
+        if (threadIdx.x == 0) stop_word() = *(volatile unsigned *)(g.count + 1) != 0;
+    }
+    static __device__ __forceinline__ bool stopped() { return stop_word() != 0; }
     // Waits until every block has arrived; what they wrote before is visible after.  false: a block did not arrive
     // within SYNC_POLLS reads (or another block has found so): the caller returns.
     __device__ bool wait()
@@ -469,8 +487,7 @@ struct SliceSweep {
 template <class... P, class... A>
 cudaError_t launch_run(labfm_ctx *ctx, const SellView &S, void (*kern)(P...), A... args)
 {
-    cudaError_t e = ctx->sync_buf.reserve(256);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->sync_buf.ptr, 0, 2 * sizeof(unsigned), ctx->stream);
+    cudaError_t e = cudaMemsetAsync(ctx->sync_buf.ptr, 0, sizeof(unsigned), ctx->stream);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)S.blocks);
@@ -483,19 +500,37 @@ cudaError_t launch_run(labfm_ctx *ctx, const SellView &S, void (*kern)(P...), A.
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
-// Whether a barrier of an earlier run gave up (its results are not valid); the word is cleared.
-inline bool run_gave_up(labfm_ctx *ctx)
+// The barrier words, before the first launch
+inline cudaError_t ensure_sync(labfm_ctx *ctx)
 {
-    volatile unsigned *w = reinterpret_cast<unsigned *>(static_cast<char *>(ctx->host_small) + LABFM_GAVE_UP);
-    const bool gave_up = *w != 0;
-    *w = 0;
-    return gave_up;
+    if (ctx->sync_buf.ptr) return cudaSuccess;
+    const cudaError_t e = ctx->sync_buf.reserve(256);
+    return e == cudaSuccess ? cudaMemsetAsync(ctx->sync_buf.ptr, 0, 256, ctx->stream) : e;
 }
-inline GridSync grid_sync(const labfm_ctx *ctx)
+inline unsigned *gave_up_word(const labfm_ctx *ctx, int byte)
 {
-    return GridSync{ctx->sync_buf.as<unsigned>(), reinterpret_cast<unsigned *>(static_cast<char *>(ctx->host_small) + LABFM_GAVE_UP)};
+    return reinterpret_cast<unsigned *>(static_cast<char *>(ctx->host_small) + byte);
+}
+inline GridSync grid_sync(const labfm_ctx *ctx, int byte)
+{
+    return GridSync{ctx->sync_buf.as<unsigned>(), gave_up_word(ctx, byte)};
 }
 #endif
+// Whether a wait of a run (byte LABFM_GAVE_UP) or solve that has ended gave up; launches from here on run again.
+inline bool gave_up(labfm_ctx *ctx, int byte)
+{
+    volatile unsigned *w = reinterpret_cast<unsigned *>(static_cast<char *>(ctx->host_small) + byte);
+    if (*w == 0) return false;
+    *w = 0;
+    cudaMemsetAsync(ctx->sync_buf.as<unsigned>() + 1, 0, sizeof(unsigned), ctx->stream);
+    return true;
+}
+inline labfm_status run_gave_up(labfm_ctx *ctx)
+{
+    return gave_up(ctx, LABFM_GAVE_UP)
+               ? fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the blocks of an earlier run gave up: the fields of the runs since are not valid")
+               : LABFM_OK;
+}
 inline SellView sell_view(const Sell &L)
 {
     return SellView{L.n_slices, L.off.as<int64_t>(), L.col.as<int32_t>(), L.share.as<int64_t>(), L.blocks, L.lg_l};

@@ -300,7 +300,12 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_solve_run(SolveArgs A, int s
     __shared__ SolveState st;
     int64_t s0, s1;
     block_share(A.S, s0, s1);
+    GridBarrier{A.sync}.check();
     share_out(A.S, s0, s1);
+    if (GridBarrier::stopped()) {
+        if (threadIdx.x == 0) *(volatile unsigned *)A.sync.gave_up = 1u;  // the host learns that no iteration was made
+        return;
+    }
     SolveBlock B(A, s0, s1);
     if (threadIdx.x == 0) st = *A.st;
     __syncthreads();
@@ -444,7 +449,7 @@ labfm_status run_solve(labfm_ctx *ctx, int op, const double *f, double *phi, con
     LABFM_CUDA_TRY(ctx, ctx->sol_w.reserve(sizeof(double) * (L.places > 0 ? L.places : 1)));
     LABFM_CUDA_TRY(ctx, ctx->sol_vec.reserve(sizeof(double) * 11 * n));
     LABFM_CUDA_TRY(ctx, ctx->sol_part.reserve(sizeof(double) * NSLOT * (size_t)ctx->num_sms + sizeof(SolveState)));
-    LABFM_CUDA_TRY(ctx, ctx->sync_buf.reserve(256));
+    LABFM_CUDA_TRY(ctx, ensure_sync(ctx));
     double *V = ctx->sol_vec.as<double>();
     double *dinv = V, *r = V + n, *rhat = V + 2 * n, *p = V + 3 * n, *v = V + 4 * n, *y = V + 5 * n, *sv = V + 6 * n,
            *z = V + 7 * n, *t = V + 8 * n, *adiag = V + 9 * n, *d = V + 10 * n;
@@ -467,7 +472,7 @@ labfm_status run_solve(labfm_ctx *ctx, int op, const double *f, double *phi, con
     init.tol2 = tol * tol;
     init.max_iter = max_iter;
     LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(st, &init, sizeof(SolveState), cudaMemcpyHostToDevice, s));
-    const SolveArgs args{n, S, wd, adiag, dinv, f, dirichlet, gr, phi, d, r, rhat, p, v, y, sv, z, t, part, st, grid_sync(ctx)};
+    const SolveArgs args{n, S, wd, adiag, dinv, f, dirichlet, gr, phi, d, r, rhat, p, v, y, sv, z, t, part, st, grid_sync(ctx, LABFM_SOLVE_GAVE_UP)};
     const int most = (int)std::max<int64_t>(8, std::min<int64_t>(ITERS_MAX, (int64_t)1000000000 / (nnz + 100000)));
     // Launches until the state says that the iteration ended, with the true residual.  BiCGStab
     // restarts from the current iterate (r = F - A Phi, r^ = r), at most MAX_RESTARTS times
@@ -491,7 +496,9 @@ labfm_status run_solve(labfm_ctx *ctx, int op, const double *f, double *phi, con
             if (le == cudaSuccess) le = cudaMemcpyAsync(&h, st, sizeof(SolveState), cudaMemcpyDeviceToHost, s);
             if (le == cudaSuccess) le = cudaStreamSynchronize(s);
             if (le != cudaSuccess) return cuda_fail(ctx, le, "BiCGStab iterations");
-            if (run_gave_up(ctx)) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the solver's blocks gave up");
+            const bool mine = gave_up(ctx, LABFM_SOLVE_GAVE_UP);
+            if (const labfm_status rs = run_gave_up(ctx)) return rs;
+            if (mine) return fail(ctx, LABFM_ERR_TIMEOUT, "a wait between the solver's blocks gave up");
         } while (!h.done);
         total += h.iters;
         resid = std::sqrt(h.resid2) / (h.bnorm2 > 0.0 ? std::sqrt(h.bnorm2) : 1.0);
