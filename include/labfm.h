@@ -240,7 +240,8 @@ labfm_status labfm_apply(labfm_ctx *ctx, uint32_t op_mask, const void *f, int fi
  * The per-node stage update is in double (in float when weights and field are FP32).
  * Nodes with frozen[i] != 0 keep their value
  * (Dirichlet nodes, Sec. 5.1).  On FP64 fields the steps run in cooperative launches (a block
- * per SM, a barrier over them between stages) on a layout of the stencils that the first
+ * per SM of the stream, or as many as fit, a barrier over them between stages; up to some tens of
+ * milliseconds each, in which no other launch shares those SMs) on a layout of the stencils that the first
  * such call after labfm_build_neighbours makes.  A barrier that gives up (after 2^21 reads of its
  * count, of the order of a second) ends the run, its field is then undefined, and runs enqueued
  * behind it leave their fields as they are, until a call has reported it: that call does nothing

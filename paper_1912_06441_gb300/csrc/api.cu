@@ -186,6 +186,7 @@ labfm_status labfm_create(labfm_ctx **out, int device, void *stream)
     ctx->device = device;
     ctx->stream = (cudaStream_t)stream;
     cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
+    ctx->run_blocks = ctx->num_sms;
     if (cudaMallocHost(&ctx->host_small, 1024) != cudaSuccess) {  // status words read back by the calls
         delete ctx;
         return LABFM_ERR_NOMEM;
@@ -221,6 +222,7 @@ labfm_status labfm_set_stream(labfm_ctx *ctx, void *stream)
 {
     if (!ctx) return LABFM_ERR_ARG;
     ctx->stream = (cudaStream_t)stream;
+    ctx->run_blocks = ctx->num_sms;
     ctx->graph.release();
     ctx->graph_burgers.release();
     return LABFM_OK;

@@ -83,6 +83,7 @@ struct labfm_ctx {
     labfm::DevBuf row_ptr, col;
     labfm::Sell sell;  // of these stencils, for the FP64 products
     labfm::DevBuf sync_buf;  // barrier words of the cooperative runs
+    int run_blocks = 0;      // blocks that fit the context's stream at once
     // scratch of the neighbour search
     labfm::DevBuf cell_of, cell_count, cell_start, cell_nodes, counts, scan_tmp, misc;
 
@@ -483,14 +484,14 @@ struct SliceSweep {
     }
 };
 
-// Cooperative launch of such a run on the context's stream
+// Cooperative launch of such a run on the context's stream.  Its blocks have to fit the SMs together: where the stream has
+// fewer of them than the device (a green context, a share of the device), with half as many blocks, and so on.
 template <class... P, class... A>
 cudaError_t launch_run(labfm_ctx *ctx, const SellView &S, void (*kern)(P...), A... args)
 {
     cudaError_t e = cudaMemsetAsync(ctx->sync_buf.ptr, 0, sizeof(unsigned), ctx->stream);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)S.blocks);
     cfg.blockDim = dim3(RUN_THREADS);
     cfg.stream = ctx->stream;
     cudaLaunchAttribute at{};
@@ -498,7 +499,13 @@ cudaError_t launch_run(labfm_ctx *ctx, const SellView &S, void (*kern)(P...), A.
     at.val.cooperative = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    while (true) {
+        cfg.gridDim = dim3((unsigned)(S.blocks < ctx->run_blocks ? S.blocks : ctx->run_blocks));
+        e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
+        if (e != cudaErrorCooperativeLaunchTooLarge || cfg.gridDim.x == 1) return e;
+        cudaGetLastError();
+        ctx->run_blocks = (int)(cfg.gridDim.x + 1) / 2;
+    }
 }
 // The barrier words, before the first launch
 inline cudaError_t ensure_sync(labfm_ctx *ctx)
