@@ -26,7 +26,7 @@ struct Grid {
     double lo[2], L[2], halfL[2], inv_cs[2];
     int nc[2];
     int periodic;
-    // float pre-filter of the distance test (used where cell_xyf is given): box sides and half
+    // float pre-filter of the distance test: box sides and half
     // sides in float, the bound E on |dx_float - dx| (roundings of the coordinates, the
     // difference and the wrap), and the largest (2h)^2 for which the float wrap cannot differ
     // from the double one on a candidate near the radius
@@ -302,6 +302,17 @@ struct Candidates {
     }
 };
 
+// Float coordinates of the node at p in cell order, from the float copy, or where there is none (the search on a fixed
+// scratch array) the same values converted again: 360^2 nodes at order 4 in 224 us, 838 with the double test alone.  (The
+// sweeps test the copy against null although it is there: left out, the search took 2 to 3 % longer.)
+template <bool COPY>
+__device__ __forceinline__ float2 float_at(int64_t p, const double2 *__restrict__ cell_xy, const float2 *__restrict__ cell_xyf)
+{
+    if (COPY) return cell_xyf[p];
+    const double2 q = cell_xy[p];
+    return make_float2((float)q.x, (float)q.y);
+}
+
 // One sweep over the candidates of every node; WRITE = false: count; true: write col[].  A warp takes SWEEP_NODES
 // consecutive nodes in cell order.  The nodes of a cell share their candidates, which the warp keeps in registers (up to
 // SWEEP_REGS per lane; more are read again for every node): per node there is the test of each candidate, a ballot
@@ -310,7 +321,7 @@ struct Candidates {
 // and 817.)
 constexpr int SWEEP_NODES = 8;
 constexpr int SWEEP_REGS = 8;
-template <bool WRITE>
+template <bool WRITE, bool COPY>
 __global__ void __launch_bounds__(NB_THREADS) k_sweep(int64_t n, const double *__restrict__ h, Grid g,
                                                       const int32_t *__restrict__ cell_of,
                                                       const int64_t *__restrict__ cell_start,
@@ -343,7 +354,7 @@ __global__ void __launch_bounds__(NB_THREADS) k_sweep(int64_t n, const double *_
     }
     const float my_xf = (float)my_at.x, my_yf = (float)my_at.y, my_R2f = (float)my_R2;
     // float classification only where the float wrap cannot flip a candidate near the radius
-    const int my_filt = cell_xyf != nullptr && (!g.periodic || my_R2 <= g.r2_wrap_max);
+    const int my_filt = (!COPY || cell_xyf != nullptr) && (!g.periodic || my_R2 <= g.r2_wrap_max);
     for (int k0 = 0; k0 < nodes;) {
         const int c = __shfl_sync(all, my_cell, k0);
         const Candidates cand(c, g, cell_start);
@@ -360,7 +371,7 @@ __global__ void __launch_bounds__(NB_THREADS) k_sweep(int64_t n, const double *_
                 if (q < cand.total) {
                     const int p = cand.place(q);
                     cj[r] = cell_nodes[p];
-                    if (cell_xyf) cq[r] = cell_xyf[p];
+                    if (!COPY || cell_xyf) cq[r] = float_at<COPY>(p, cell_xy, cell_xyf);
                     valid |= 1u << r;
                 }
             }
@@ -436,7 +447,7 @@ __global__ void __launch_bounds__(NB_THREADS) k_sweep(int64_t n, const double *_
 
 // The same with a thread per node, in cell order, its row sorted by insertion: for large sets of few nodes to a cell, where
 // the rows are short and a warp's eight nodes lie in several cells.
-template <bool WRITE>
+template <bool WRITE, bool COPY>
 __global__ void k_sweep_sparse(int64_t n, const double *__restrict__ h, Grid g,
                         const int32_t *__restrict__ cell_of, const int64_t *__restrict__ cell_start,
                         const int32_t *__restrict__ cell_nodes, const double2 *__restrict__ cell_xy,
@@ -450,7 +461,7 @@ __global__ void k_sweep_sparse(int64_t n, const double *__restrict__ h, Grid g,
     double R = 2.0 * h[i];
     double R2 = __dmul_rn(R, R);
     // float classification only where the float wrap cannot flip a candidate near the radius
-    const bool filt = cell_xyf != nullptr && (!g.periodic || R2 <= g.r2_wrap_max);
+    const bool filt = (!COPY || cell_xyf != nullptr) && (!g.periodic || R2 <= g.r2_wrap_max);
     const Prefilter pre((float)xi, (float)yi, (float)R2, g);
     int c = cell_of[i];
     int cx = c % g.nc[0], cy = c / g.nc[0];
@@ -470,7 +481,7 @@ __global__ void k_sweep_sparse(int64_t n, const double *__restrict__ h, Grid g,
                 int decided = 0;  // 1: inside, 2: outside, 0: to the double test
                 if (filt) {
                     bool inside, outside;
-                    pre.test(cell_xyf[p], g.periodic != 0, g, inside, outside);
+                    pre.test(float_at<COPY>(p, cell_xy, cell_xyf), g.periodic != 0, g, inside, outside);
                     decided = inside ? 1 : (outside ? 2 : 0);
                 }
                 if (decided) {
@@ -518,16 +529,16 @@ unsigned sweep_blocks(int64_t n)
     return (unsigned)((n + per - 1) / per);
 }
 
-template <bool WRITE>
+template <bool WRITE, bool COPY>
 void launch_sweep(int64_t n, const double *h, const Grid &g, const int32_t *cell_of, const int64_t *cell_start,
                   const int32_t *cell_nodes, const double2 *cell_xy, const float2 *cell_xyf, int32_t *counts,
                   const int64_t *row_ptr, int32_t *col, cudaStream_t s)
 {
     if (sparse_cells(n, g))
-        k_sweep_sparse<WRITE><<<(unsigned)((n + NB_THREADS - 1) / NB_THREADS), NB_THREADS, 0, s>>>(
+        k_sweep_sparse<WRITE, COPY><<<(unsigned)((n + NB_THREADS - 1) / NB_THREADS), NB_THREADS, 0, s>>>(
             n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, row_ptr, col);
     else
-        k_sweep<WRITE><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf,
+        k_sweep<WRITE, COPY><<<sweep_blocks(n), NB_THREADS, 0, s>>>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf,
                                                               counts, row_ptr, col);
 }
 
@@ -624,7 +635,7 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(cell_count, cell_start, ncells, ctx->scan_tmp, s));
     k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, cell_xyf);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
-    launch_sweep<false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, nullptr, nullptr, s);
+    launch_sweep<false, true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, nullptr, nullptr, s);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(counts, row_ptr, n, ctx->scan_tmp, s));
     int64_t *nnz_h = (int64_t *)ctx->host_small;
@@ -633,7 +644,7 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     int64_t nnz = *nnz_h;
     if (nnz >= ((int64_t)1 << 40)) return fail(ctx, LABFM_ERR_CAPACITY, "too many stencil entries");
     LABFM_CUDA_TRY(ctx, ctx->col.reserve(sizeof(int32_t) * (nnz > 0 ? nnz : 1)));
-    launch_sweep<true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr, row_ptr, ctx->col.as<int32_t>(), s);
+    launch_sweep<true, true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr, row_ptr, ctx->col.as<int32_t>(), s);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
     ctx->n = n;
@@ -767,6 +778,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
         g.nc[d] = (int)ncell_d[d];
         g.inv_cs[d] = (double)g.nc[d] / g.L[d];
     }
+    set_float_filter(g, box_lo, box_hi);
     const int64_t ncells = (int64_t)g.nc[0] * g.nc[1];
     if (ncells > NA_MAXC) return LABFM_ERR_CAPACITY;
 
@@ -775,10 +787,10 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
     k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count, counts);  // counts: the ranks until the sweep
     NA_TRY(cudaGetLastError());
     NA_TRY(exclusive_scan_i32_to_i64_ws(cell_count, cell_start, ncells, scan_tmp, NA_SCAN_ELEMS, s));
-    // (the float pre-filter needs an array the fixed scratch does not hold: the double test alone)
+    // (the float pre-filter's coordinates are converted where they are read: the fixed scratch holds no copy of them)
     k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, nullptr);
     NA_TRY(cudaGetLastError());
-    launch_sweep<false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, counts, nullptr, nullptr, s);
+    launch_sweep<false, false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, counts, nullptr, nullptr, s);
     NA_TRY(cudaGetLastError());
     NA_TRY(exclusive_scan_i32_to_i64_ws(counts, row_ptr, n, scan_tmp, NA_SCAN_ELEMS, s));
     int64_t nnz = 0;
@@ -787,7 +799,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
     *nnz_out = nnz;
     if (nnz > col_capacity) return LABFM_ERR_CAPACITY;
     if (nnz > 0) {
-        launch_sweep<true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, nullptr, row_ptr, col, s);
+        launch_sweep<true, false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, nullptr, row_ptr, col, s);
         NA_TRY(cudaGetLastError());
     }
     NA_TRY(cudaStreamSynchronize(s));
