@@ -517,9 +517,14 @@ __global__ void k_sweep_sparse(int64_t n, const double *__restrict__ h, Grid g,
 // Which of the two: whole searches take, with k_sweep_sparse and k_sweep, at 900^2 nodes 683 and 841 us at order 3 (6.8 nodes
 // a cell), 762 and 893 at order 4 (7.8), but 1,057 and 932 at order 5 (10.2); at 600^2 order 2 and 3 (5.8, 6.8) 422 and 478,
 // 443 and 470, at 450^2 364 and 335 at order 4; at 200^2 k_sweep wins at every order (194 against 259 at order 4).
-bool sparse_cells(int64_t n, const Grid &g)
+// That mean counts empty cells too.  Rows of twice the pi nodes a node of the mean cell that a uniform set has at most (nnz, known
+// to the write sweep, else 0) are those of a set that fills a part of its box, with many nodes in each cell: whole
+// searches of 200,000 nodes, 100 to each of 5 % of the cells, took 3.4 ms with both sweeps by a thread per node, 0.8 with
+// this one by k_sweep; 300 to each of 2 %, 28 and 4.3.
+bool sparse_cells(int64_t n, const Grid &g, int64_t nnz)
 {
     const double per_cell = (double)n / ((double)g.nc[0] * (double)g.nc[1]);
+    if ((double)nnz > 2.0 * 3.15 * per_cell * (double)n) return false;
     return per_cell < 7.5 ? n >= 200000 : per_cell < 9.0 && n >= 400000;
 }
 
@@ -532,9 +537,9 @@ unsigned sweep_blocks(int64_t n)
 template <bool WRITE, bool COPY>
 void launch_sweep(int64_t n, const double *h, const Grid &g, const int32_t *cell_of, const int64_t *cell_start,
                   const int32_t *cell_nodes, const double2 *cell_xy, const float2 *cell_xyf, int32_t *counts,
-                  const int64_t *row_ptr, int32_t *col, cudaStream_t s)
+                  const int64_t *row_ptr, int32_t *col, int64_t nnz, cudaStream_t s)
 {
-    if (sparse_cells(n, g))
+    if (sparse_cells(n, g, nnz))
         k_sweep_sparse<WRITE, COPY><<<(unsigned)((n + NB_THREADS - 1) / NB_THREADS), NB_THREADS, 0, s>>>(
             n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, row_ptr, col);
     else
@@ -635,7 +640,7 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(cell_count, cell_start, ncells, ctx->scan_tmp, s));
     k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, cell_xyf);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
-    launch_sweep<false, true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, nullptr, nullptr, s);
+    launch_sweep<false, true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, nullptr, nullptr, 0, s);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(counts, row_ptr, n, ctx->scan_tmp, s));
     int64_t *nnz_h = (int64_t *)ctx->host_small;
@@ -644,7 +649,7 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     int64_t nnz = *nnz_h;
     if (nnz >= ((int64_t)1 << 40)) return fail(ctx, LABFM_ERR_CAPACITY, "too many stencil entries");
     LABFM_CUDA_TRY(ctx, ctx->col.reserve(sizeof(int32_t) * (nnz > 0 ? nnz : 1)));
-    launch_sweep<true, true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr, row_ptr, ctx->col.as<int32_t>(), s);
+    launch_sweep<true, true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr, row_ptr, ctx->col.as<int32_t>(), nnz, s);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
     ctx->n = n;
@@ -790,7 +795,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
     // (the float pre-filter's coordinates are converted where they are read: the fixed scratch holds no copy of them)
     k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, nullptr);
     NA_TRY(cudaGetLastError());
-    launch_sweep<false, false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, counts, nullptr, nullptr, s);
+    launch_sweep<false, false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, counts, nullptr, nullptr, 0, s);
     NA_TRY(cudaGetLastError());
     NA_TRY(exclusive_scan_i32_to_i64_ws(counts, row_ptr, n, scan_tmp, NA_SCAN_ELEMS, s));
     int64_t nnz = 0;
@@ -799,7 +804,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
     *nnz_out = nnz;
     if (nnz > col_capacity) return LABFM_ERR_CAPACITY;
     if (nnz > 0) {
-        launch_sweep<true, false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, nullptr, row_ptr, col, s);
+        launch_sweep<true, false>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, nullptr, nullptr, row_ptr, col, nnz, s);
         NA_TRY(cudaGetLastError());
     }
     NA_TRY(cudaStreamSynchronize(s));
