@@ -156,6 +156,8 @@ labfm_status run_build(labfm_ctx *ctx, const int8_t *order, int uniform_order, i
     // Group size of the FP64 kernel per order: timed once per (order, mean stencil size, n_ops)
     // on up to 16,384 of the order's real nodes (the autotuner of the build), kept in the
     // context's table.  Not while the caller's stream is being captured, nor below 4,096 nodes.
+    // (The form of the ABFs is not in the key, and the untimed choice of a small set is kept: both forms' timings come out
+    // as that choice, 64 threads at orders 1 to 4, 128 at 5 and 6, at 200^2 nodes.)
     auto group_for = [&](int k, const int32_t *list, int64_t cnt, double deg, int &G) -> cudaError_t {
         G = k <= 4 ? 64 : (k <= 6 ? 128 : 256);
         const uint64_t dkey = (uint64_t)std::min(deg + 0.5, 65535.0);
