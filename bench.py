@@ -1052,10 +1052,10 @@ def run_labfm(args, rank, world, local_rank):
         "build_mnodes_per_s": n / (build_ms * 1e-3) / 1e6,
         "e2e": {"value": replicas_throughput(world, n, e2e_ms), "unit": "Mnodes/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
-        # per step: stencil search, one build launch (uniform order), one apply, and the RK4
-        # step (operator combination + 4 stage kernels)
-        "gpu_launches": args.steps * (nbr_launches(n, ncells_of(HS / N_SIDE)) + 1 + 1 + 1 + 2
-                                      + scan_launches(n // 32) + 1),
+        # per step: stencil search, one build launch (uniform order), one apply, and the RK4 step (shape of the sliced
+        # layout, its prefix sum, its columns and combined weights, and the four stages as one run)
+        "gpu_launches": args.steps * (nbr_launches(n, ncells_of(HS / N_SIDE)) + 1 + 1 + 1
+                                      + scan_launches(n // 32) + 1 + 1),
         "clocks": clk,
     }
     line["build_tuning"] = L.get_build_info()["fp64_group_threads"]

@@ -17,7 +17,9 @@
  *    destroyed or the buffer is rebuilt.
  *  - Work is enqueued on the context stream.  Calls that return counts or
  *    statuses (labfm_build_neighbours, labfm_build_weights) synchronise that
- *    stream before returning; labfm_apply and labfm_step do not.
+ *    stream before returning; labfm_apply and labfm_step do not (the first labfm_step or
+ *    labfm_step_burgers on FP64 fields after a search does where the longest stencil is more than
+ *    about twice the mean).
  *  - No C++ exception crosses the ABI; failures return a labfm_status and
  *    labfm_last_error() gives a message.  Invalid arguments are rejected on the
  *    host before any kernel is launched.

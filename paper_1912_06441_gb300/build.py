@@ -18,7 +18,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "liblabfm.so")
 SOURCES = ["api.cu", "neighbours.cu", "build_fp64.cu", "build_fp64_dw0.cu", "build_fp64_chain.cu", "build_mixed.cu", "sell.cu", "apply.cu", "solve.cu"]
-HEADERS = ["labfm_internal.cuh", "abf.cuh", "build_node.cuh", "df64.cuh"]
+HEADERS = ["labfm_internal.cuh", "abf.cuh", "build_node.cuh", "df64.cuh", "sell_fill.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I", os.path.join(ROOT, "include"), "-I", CSRC]

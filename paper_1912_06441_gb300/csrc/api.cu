@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_sums(const Tin *__restric
 // sums: the sums of the blocks' runs, or with `scanned` their exclusive scan; null for a single block
 template <class Tin>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const Tin *__restrict__ in, int64_t *__restrict__ out, int64_t n,
-                                                             const int64_t *__restrict__ sums, int scanned)
+                                                             const int64_t *__restrict__ sums, int scanned,
+                                                             unsigned long long *__restrict__ largest)
 {
     __shared__ int64_t sh[32];
     int64_t before = 0;  // the sum of all earlier blocks' runs
@@ -116,12 +117,16 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const Tin *__restri
     if (g < n) out[g] = at;
     if (g + 1 < n) out[g + 1] = at + a;
     if (g < n && g + 2 >= n) out[n] = at + a + b;  // the thread of the last element
+    if (largest) {
+        const unsigned most = __reduce_max_sync(0xffffffffu, (unsigned)max(a, b));
+        if (lane == 0 && most > *(volatile unsigned long long *)largest) atomicMax(largest, (unsigned long long)most);
+    }
 }
 
 __global__ void k_scan_empty(int64_t *out) { out[0] = 0; }
 
 template <class Tin>
-static cudaError_t scan_rec(const Tin *in, int64_t *out, int64_t n, int64_t *tmp, cudaStream_t s)
+static cudaError_t scan_rec(const Tin *in, int64_t *out, int64_t n, int64_t *tmp, cudaStream_t s, unsigned long long *largest)
 {
     const int64_t nb = (n + SCAN_ITEMS - 1) / SCAN_ITEMS;
     int64_t *sums = nullptr;
@@ -132,11 +137,11 @@ static cudaError_t scan_rec(const Tin *in, int64_t *out, int64_t n, int64_t *tmp
         if (e != cudaSuccess) return e;
         if (nb > SCAN_DIRECT) {
             int64_t *scanned = tmp + nb;  // nb + 1 elements
-            if ((e = scan_rec<int64_t>(sums, scanned, nb, tmp + 2 * nb + 1, s)) != cudaSuccess) return e;
+            if ((e = scan_rec<int64_t>(sums, scanned, nb, tmp + 2 * nb + 1, s, nullptr)) != cudaSuccess) return e;
             sums = scanned;
         }
     }
-    k_scan_apply<Tin><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, sums, nb > SCAN_DIRECT ? 1 : 0);
+    k_scan_apply<Tin><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, out, n, sums, nb > SCAN_DIRECT ? 1 : 0, largest);
     return cudaGetLastError();
 }
 
@@ -153,19 +158,20 @@ size_t scan_workspace_elems(int64_t n)
 }
 
 cudaError_t exclusive_scan_i32_to_i64_ws(const int32_t *in, int64_t *out, int64_t n, int64_t *tmp, size_t tmp_elems,
-                                         cudaStream_t s)
+                                         cudaStream_t s, unsigned long long *largest)
 {
     if (scan_workspace_elems(n) > tmp_elems) return cudaErrorInvalidValue;
-    if (n > 0) return scan_rec<int32_t>(in, out, n, tmp, s);
+    if (n > 0) return scan_rec<int32_t>(in, out, n, tmp, s, largest);
     k_scan_empty<<<1, 1, 0, s>>>(out);
     return cudaGetLastError();
 }
 
-cudaError_t exclusive_scan_i32_to_i64(const int32_t *in, int64_t *out, int64_t n, DevBuf &tmp, cudaStream_t s)
+cudaError_t exclusive_scan_i32_to_i64(const int32_t *in, int64_t *out, int64_t n, DevBuf &tmp, cudaStream_t s,
+                                      unsigned long long *largest)
 {
     const size_t elems = scan_workspace_elems(n);
     cudaError_t e = tmp.reserve(elems * sizeof(int64_t));
-    return e == cudaSuccess ? exclusive_scan_i32_to_i64_ws(in, out, n, tmp.as<int64_t>(), elems, s) : e;
+    return e == cudaSuccess ? exclusive_scan_i32_to_i64_ws(in, out, n, tmp.as<int64_t>(), elems, s, largest) : e;
 }
 
 }  // namespace labfm
@@ -241,7 +247,7 @@ labfm_status labfm_build_neighbours(labfm_ctx *ctx, int64_t n, const double *xy,
     if (cudaSetDevice(ctx->device) != cudaSuccess) return fail(ctx, LABFM_ERR_CUDA, "cudaSetDevice failed");
     ctx->have_weights = false;
     ctx->wcomb_valid = false;
-    ctx->sell.valid = false;
+    ctx->sell.shaped = ctx->sell.valid = false;
     const labfm_status st = run_neighbours(ctx, n, xy, h, periodic ? 1 : 0, box_lo, box_hi, nnz_out);
     const labfm_status rs = run_gave_up(ctx);  // (every run has ended: the search waited for the stream)
     if (rs != LABFM_OK) ctx->n = 0;            // its positions may come from that run

@@ -20,7 +20,7 @@
 #include <type_traits>
 
 #include "df64.cuh"
-#include "labfm_internal.cuh"
+#include "sell_fill.cuh"
 
 namespace labfm {
 namespace {
@@ -174,22 +174,19 @@ __global__ void k_combine(int64_t nnz, int n_ops, const WT *__restrict__ w, cons
     }
 }
 
-// wc in the sliced layout (a warp per slice): 0 where there is no entry
-template <class WT, class VT>
-__global__ void __launch_bounds__(APPLY_THREADS) k_combine_sliced(int64_t n, SellView S,
-                                                                 const int64_t *__restrict__ row_ptr, int n_ops,
-                                                                 const WT *__restrict__ w, VT *__restrict__ wc, Beta b)
-{
-    const SellLane l((int64_t)blockIdx.x * (APPLY_THREADS / 32) + (threadIdx.x >> 5), threadIdx.x & 31, n, S);
-    const int64_t rs = l.i >= 0 ? row_ptr[l.i] : 0, re = l.i >= 0 ? row_ptr[l.i + 1] : 0;
-    for (int k = 0; k < l.steps; k++) {
-        const int64_t e = rs + ((int64_t)k << S.lg_l) + l.h;
+// wc of an entry, for the sliced layout
+template <class WT>
+struct Combined {
+    const WT *__restrict__ w;
+    int n_ops;
+    Beta b;
+    __device__ __forceinline__ void operator()(int64_t e, WT *v) const
+    {
         double s = 0.0;
-        if (e < re)
-            for (int d = 0; d < n_ops; d++) s = fma(b.v[d], (double)w[e * n_ops + d], s);
-        wc[l.at + 32 * (int64_t)k] = (VT)s;
+        for (int d = 0; d < n_ops; d++) s = fma(b.v[d], (double)w[e * n_ops + d], s);
+        v[0] = (WT)s;
     }
-}
+};
 
 // One RK4 stage.  F_i = sum_j (src_j - src_i) wc_ji (0 on frozen nodes), then
 //   stage 0: acc = u + dt/6 F,  nxt = u + dt/2 F
@@ -426,8 +423,6 @@ cudaError_t launch_stage_csr(labfm_ctx *ctx, Shape sh, const float *src, float *
     return cudaGetLastError();
 }
 
-unsigned slice_blocks(const labfm_ctx *ctx, int threads) { return (unsigned)((ctx->sell.n_slices * 32 + threads - 1) / threads); }
-
 // Time every shape with `run` (which enqueues one launch on ctx->stream) and keep the fastest.
 template <class RunFn>
 cudaError_t autotune(labfm_ctx *ctx, uint64_t key, int min_g, RunFn run, Shape &best)
@@ -581,7 +576,7 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
     size_t fsz = fdt == LABFM_F64 ? 8 : 4;
     const int fmt = cw_format(fdt, ctx->wdtype);
     if (cw_sliced(fmt)) {
-        labfm_status st = ensure_sell(ctx);
+        labfm_status st = ensure_sell_shape(ctx);
         if (st != LABFM_OK) return st;
     }
     // combined weight, cached while beta, the weights and the storage format are unchanged
@@ -592,18 +587,17 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
         LABFM_CUDA_TRY(ctx, ctx->wcomb.reserve(bytes > 0 ? bytes : 8));
         Beta b{};
         for (int d = 0; d < ctx->n_ops; d++) b.v[d] = beta[d];
-        const int64_t *rp = ctx->row_ptr.as<int64_t>();
         const int32_t *cl = ctx->col.as<int32_t>();
-        const unsigned blocks = (unsigned)((nnz + 255) / 256), sb = slice_blocks(ctx, APPLY_THREADS);
+        const unsigned blocks = (unsigned)((nnz + 255) / 256);
         if (nnz > 0) {
             switch (fmt) {
             case CW_S64:
-                k_combine_sliced<double, double><<<sb, APPLY_THREADS, 0, s>>>(n, sell_view(ctx->sell), rp, ctx->n_ops,
-                                                                             ctx->w.as<double>(), ctx->wcomb.as<double>(), b);
+                LABFM_CUDA_TRY(ctx, (launch_sell_fill<double, 1>(ctx, ctx->sell, ctx->wcomb.as<double>(),
+                                                                Combined<double>{ctx->w.as<double>(), ctx->n_ops, b})));
                 break;
             case CW_S32:
-                k_combine_sliced<float, float><<<sb, APPLY_THREADS, 0, s>>>(n, sell_view(ctx->sell), rp, ctx->n_ops,
-                                                                           ctx->w.as<float>(), ctx->wcomb.as<float>(), b);
+                LABFM_CUDA_TRY(ctx, (launch_sell_fill<float, 1>(ctx, ctx->sell, ctx->wcomb.as<float>(),
+                                                               Combined<float>{ctx->w.as<float>(), ctx->n_ops, b})));
                 break;
             case CW_DF:
                 k_combine<double><<<blocks, 256, 0, s>>>(nnz, ctx->n_ops, ctx->w.as<double>(), cl, ctx->wcomb.ptr, fmt, b);
@@ -623,6 +617,8 @@ labfm_status run_step(labfm_ctx *ctx, const double *beta, void *u, int fdt, doub
     LABFM_CUDA_TRY(ctx, ctx->rk_stage_b.reserve(fsz * n));
 
     if (cw_sliced(fmt)) {
+        labfm_status st = ensure_sell(ctx);
+        if (st != LABFM_OK) return st;
         double *uu = (double *)u, *acc = ctx->rk_acc.as<double>(), *sa = ctx->rk_stage_a.as<double>(), *sb = ctx->rk_stage_b.as<double>();
         const SellView S = sell_view(ctx->sell);
         LABFM_CUDA_TRY(ctx, ensure_sync(ctx));
@@ -714,25 +710,20 @@ __global__ void k_burg_combine(int64_t nnz, int n_ops, const WT *__restrict__ w,
 }
 
 template <class WT>
-__global__ void __launch_bounds__(APPLY_THREADS) k_burg_combine_sliced(int64_t n, SellView S,
-                                                                      const int64_t *__restrict__ row_ptr, int n_ops,
-                                                                      const WT *__restrict__ w, WT *__restrict__ wb, Beta b)
-{
-    const int lane = threadIdx.x & 31;
-    const SellLane l((int64_t)blockIdx.x * (APPLY_THREADS / 32) + (threadIdx.x >> 5), lane, n, S);
-    const int64_t rs = l.i >= 0 ? row_ptr[l.i] : 0, re = l.i >= 0 ? row_ptr[l.i + 1] : 0;
-    WT *out = wb + 3 * (l.at - lane) + lane;
-    for (int k = 0; k < l.steps; k++, out += 96) {
-        const int64_t e = rs + ((int64_t)k << S.lg_l) + l.h;
+struct BurgersWeights {
+    const WT *__restrict__ w;
+    int n_ops;
+    Beta b;
+    __device__ __forceinline__ void operator()(int64_t e, WT *v) const
+    {
         const WT *we = w + e * n_ops;
         double s = 0.0;
-        if (e < re)
-            for (int d = 2; d < n_ops; d++) s += b.v[d] * (double)we[d];
-        out[0] = e < re ? we[0] : (WT)0;
-        out[32] = e < re ? we[1] : (WT)0;
-        out[64] = (WT)s;
+        for (int d = 2; d < n_ops; d++) s += b.v[d] * (double)we[d];
+        v[0] = we[0];
+        v[1] = we[1];
+        v[2] = (WT)s;
     }
-}
+};
 
 // One RK4 stage for the pair (u, v).  With the stage's source fields (su, sv), the advection weights of node i join
 // the linear one per entry, c_ji = wl_ji - su_i w^0_ji - sv_i w^1_ji, and
@@ -946,7 +937,7 @@ labfm_status run_step_burgers(labfm_ctx *ctx, const double *beta, void *u, void 
     const size_t fsz = fdt == LABFM_F64 ? 8 : 4, wsz = ctx->wdtype == LABFM_F64 ? 8 : 4;
     const bool sliced = fdt == LABFM_F64;
     if (sliced) {
-        labfm_status st = ensure_sell(ctx);
+        labfm_status st = ensure_sell_shape(ctx);
         if (st != LABFM_OK) return st;
     }
     bool same_beta = ctx->wburg_valid && ctx->wburg_sliced == sliced;
@@ -957,19 +948,16 @@ labfm_status run_step_burgers(labfm_ctx *ctx, const double *beta, void *u, void 
         Beta b{};
         for (int d = 2; d < ctx->n_ops; d++) b.v[d] = beta[d];
         if (nnz > 0) {
-            auto combine = [&](auto wt) {
+            auto combine = [&](auto wt) -> cudaError_t {
                 using WT = decltype(wt);
                 if (sliced)
-                    k_burg_combine_sliced<WT><<<slice_blocks(ctx, APPLY_THREADS), APPLY_THREADS, 0, s>>>(
-                        n, sell_view(ctx->sell), ctx->row_ptr.as<int64_t>(), ctx->n_ops, ctx->w.as<WT>(),
-                        ctx->wburg.as<WT>(), b);
-                else
-                    k_burg_combine<WT><<<(unsigned)std::min<int64_t>((nnz + 255) / 256, (int64_t)ctx->num_sms * 32), 256, 0,
-                                         s>>>(nnz, ctx->n_ops, ctx->w.as<WT>(), ctx->wburg.as<WT>(), b);
+                    return launch_sell_fill<WT, 3>(ctx, ctx->sell, ctx->wburg.as<WT>(),
+                                                   BurgersWeights<WT>{ctx->w.as<WT>(), ctx->n_ops, b});
+                k_burg_combine<WT><<<(unsigned)std::min<int64_t>((nnz + 255) / 256, (int64_t)ctx->num_sms * 32), 256, 0, s>>>(
+                    nnz, ctx->n_ops, ctx->w.as<WT>(), ctx->wburg.as<WT>(), b);
+                return cudaGetLastError();
             };
-            if (ctx->wdtype == LABFM_F64) combine(0.0);
-            else combine(0.0f);
-            LABFM_CUDA_TRY(ctx, cudaGetLastError());
+            LABFM_CUDA_TRY(ctx, ctx->wdtype == LABFM_F64 ? combine(0.0) : combine(0.0f));
         }
         ctx->wburg_sliced = sliced;
         for (int d = 2; d < ctx->n_ops; d++) ctx->beta_burg[d] = beta[d];
@@ -980,6 +968,8 @@ labfm_status run_step_burgers(labfm_ctx *ctx, const double *beta, void *u, void 
     LABFM_CUDA_TRY(ctx, ctx->bu_stage_b.reserve(2 * fsz * n));
 
     if (sliced) {
+        labfm_status st = ensure_sell(ctx);
+        if (st != LABFM_OK) return st;
         double *uu = (double *)u, *vv = (double *)v, *acc = ctx->bu_acc.as<double>();
         double *sa = ctx->bu_stage_a.as<double>(), *sb = ctx->bu_stage_b.as<double>();
         const SellView S = sell_view(ctx->sell);

@@ -31,15 +31,17 @@ struct DevBuf {
 
 // The sliced layout of the stencils (see sell.cu), built once per stencil search by the first call that reads it.
 struct Sell {
-    bool valid = false;
+    bool shaped = false;   // lg_l .. off are those of the stencils
+    bool valid = false;    // ... and col and share
     int lg_l = 0;          // lanes per node, log2
     int64_t n_slices = 0;
-    int64_t places = 0;    // entries with the empty places
+    int64_t places = 0;    // entries with the empty places, at most
     int blocks = 0;        // shares of the slices, one per block of a run
+    int64_t slice_cost = 0;  // what a slice counts besides its steps in the shares
     DevBuf off, col, steps, share;
     void release()
     {
-        valid = false;
+        shaped = valid = false;
         off.release();
         col.release();
         steps.release();
@@ -77,6 +79,7 @@ struct labfm_ctx {
     // stencils
     int64_t n = 0;
     int64_t nnz = 0;
+    int64_t longest = 0;  // entries of the longest row
     int periodic = 0;
     double lo[2] = {0, 0}, hi[2] = {0, 0};
     labfm::DevBuf node_xy, node_h;  // context copies of the node positions and h
@@ -137,12 +140,14 @@ namespace labfm {
 labfm_status fail(labfm_ctx *ctx, labfm_status st, const std::string &msg);
 labfm_status cuda_fail(labfm_ctx *ctx, cudaError_t e, const char *where);
 
-// Exclusive prefix sum of in[0..n) into out[0..n]; out[n] = total.  `tmp` is scratch.
-cudaError_t exclusive_scan_i32_to_i64(const int32_t *in, int64_t *out, int64_t n, DevBuf &tmp, cudaStream_t s);
+// Exclusive prefix sum of in[0..n) into out[0..n]; out[n] = total.  `tmp` is scratch.  *largest (0 before) becomes the largest
+// in[i] (non-negative); null: not wanted.
+cudaError_t exclusive_scan_i32_to_i64(const int32_t *in, int64_t *out, int64_t n, DevBuf &tmp, cudaStream_t s,
+                                      unsigned long long *largest = nullptr);
 // The same scan on a caller-provided workspace of tmp_elems int64 (at least scan_workspace_elems(n)).
 size_t scan_workspace_elems(int64_t n);
 cudaError_t exclusive_scan_i32_to_i64_ws(const int32_t *in, int64_t *out, int64_t n, int64_t *tmp, size_t tmp_elems,
-                                         cudaStream_t s);
+                                         cudaStream_t s, unsigned long long *largest = nullptr);
 
 // Arguments of the mixed-precision build kernel (see build_mixed.cu).
 struct MixedArgsPublic {
@@ -542,7 +547,8 @@ inline SellView sell_view(const Sell &L)
 {
     return SellView{L.n_slices, L.off.as<int64_t>(), L.col.as<int32_t>(), L.share.as<int64_t>(), L.blocks, L.lg_l};
 }
-labfm_status ensure_sell(labfm_ctx *ctx);  // ctx->sell of the current stencils
+labfm_status ensure_sell_shape(labfm_ctx *ctx);  // ctx->sell of the current stencils, col and share still to come (sell_fill.cuh)
+labfm_status ensure_sell(labfm_ctx *ctx);        // all of it
 // The layout of the stencils with the rows in gmap (>= 0: a Neumann ghost row) replaced by their parents' (gmap null: none)
 labfm_status build_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int64_t *parent);
 

@@ -86,9 +86,10 @@ __device__ __forceinline__ int cell_coord(double x, double lo, double inv_cs, in
 }
 
 __global__ void k_cell_assign(int64_t n, const double *__restrict__ xy, Grid g, int32_t *__restrict__ cell_of,
-                              int32_t *__restrict__ cell_count, int32_t *__restrict__ rank)
+                              int32_t *__restrict__ cell_count, int32_t *__restrict__ rank, int64_t *__restrict__ longest)
 {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0 && longest) *longest = 0;  // until the rows' offsets are formed
     if (i >= n) return;
     int cx = cell_coord(xy[2 * i], g.lo[0], g.inv_cs[0], g.nc[0]);
     int cy = cell_coord(xy[2 * i + 1], g.lo[1], g.inv_cs[1], g.nc[1]);
@@ -622,7 +623,7 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
     LABFM_CUDA_TRY(ctx, ctx->cell_start.reserve(sizeof(int64_t) * (ncells + 1)));
     LABFM_CUDA_TRY(ctx, ctx->cell_nodes.reserve(sizeof(int32_t) * n + sizeof(double2) * n + sizeof(float2) * n + 64));
     LABFM_CUDA_TRY(ctx, ctx->counts.reserve(sizeof(int32_t) * n));
-    LABFM_CUDA_TRY(ctx, ctx->row_ptr.reserve(sizeof(int64_t) * (n + 1)));
+    LABFM_CUDA_TRY(ctx, ctx->row_ptr.reserve(sizeof(int64_t) * (n + 2)));
     int32_t *cell_of = ctx->cell_of.as<int32_t>();
     int32_t *cell_count = ctx->cell_count.as<int32_t>();
     int64_t *cell_start = ctx->cell_start.as<int64_t>();
@@ -635,18 +636,20 @@ labfm_status run_neighbours(labfm_ctx *ctx, int64_t n, const double *xy, const d
 
     int nbn = (int)((n + NB_THREADS - 1) / NB_THREADS);
     LABFM_CUDA_TRY(ctx, cudaMemsetAsync(cell_count, 0, sizeof(int32_t) * ncells, s));
-    k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count, counts);  // counts: the ranks until the sweep
+    // counts: the ranks until the sweep; behind the row offsets: the longest row
+    k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count, counts, row_ptr + n + 1);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(cell_count, cell_start, ncells, ctx->scan_tmp, s));
     k_cell_scatter<<<nbn, NB_THREADS, 0, s>>>(n, xy, cell_of, cell_start, counts, cell_nodes, cell_xy, cell_xyf);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     launch_sweep<false, true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, counts, nullptr, nullptr, 0, s);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
-    LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(counts, row_ptr, n, ctx->scan_tmp, s));
+    LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(counts, row_ptr, n, ctx->scan_tmp, s, reinterpret_cast<unsigned long long *>(row_ptr + n + 1)));
     int64_t *nnz_h = (int64_t *)ctx->host_small;
-    LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(nnz_h, row_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+    LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(nnz_h, row_ptr + n, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    int64_t nnz = *nnz_h;
+    const int64_t nnz = nnz_h[0];
+    ctx->longest = nnz_h[1];
     if (nnz >= ((int64_t)1 << 40)) return fail(ctx, LABFM_ERR_CAPACITY, "too many stencil entries");
     LABFM_CUDA_TRY(ctx, ctx->col.reserve(sizeof(int32_t) * (nnz > 0 ? nnz : 1)));
     launch_sweep<true, true>(n, h, g, cell_of, cell_start, cell_nodes, cell_xy, cell_xyf, nullptr, row_ptr, ctx->col.as<int32_t>(), nnz, s);
@@ -789,7 +792,7 @@ extern "C" labfm_status labfm_build_neighbours_noalloc(int device, void *stream,
 
     int nbn = (int)((n + NB_THREADS - 1) / NB_THREADS);
     NA_TRY(cudaMemsetAsync(cell_count, 0, sizeof(int32_t) * ncells, s));
-    k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count, counts);  // counts: the ranks until the sweep
+    k_cell_assign<<<nbn, NB_THREADS, 0, s>>>(n, xy, g, cell_of, cell_count, counts, nullptr);  // counts: the ranks until the sweep
     NA_TRY(cudaGetLastError());
     NA_TRY(exclusive_scan_i32_to_i64_ws(cell_count, cell_start, ncells, scan_tmp, NA_SCAN_ELEMS, s));
     // (the float pre-filter's coordinates are converted where they are read: the fixed scratch holds no copy of them)

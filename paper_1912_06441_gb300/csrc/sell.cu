@@ -8,7 +8,7 @@
 // (2 lanes per SM and clock) as long as an entry of all 32.  With one or two lanes a node they are a few percent.
 #include <algorithm>
 
-#include "labfm_internal.cuh"
+#include "sell_fill.cuh"
 
 namespace labfm {
 namespace {
@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_steps(int64_t n, int lg_l
                                                             const int64_t *__restrict__ row_ptr,
                                                             const int32_t *__restrict__ gmap,
                                                             const int64_t *__restrict__ parent,
-                                                            int32_t *__restrict__ steps, int32_t *__restrict__ longest)
+                                                            int32_t *__restrict__ steps)
 {
     const int lane = threadIdx.x & 31;
     const int64_t slice = (int64_t)blockIdx.x * (SELL_THREADS / 32) + (threadIdx.x >> 5);
@@ -40,13 +40,10 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_steps(int64_t n, int lg_l
         len = (int)(row_ptr[r + 1] - row_ptr[r]);
     }
     const int most = __reduce_max_sync(0xffffffffu, len);
-    if (lane == 0) {
-        const int count = (most + (1 << lg_l) - 1) >> lg_l;
-        steps[slice] = count;
-        if (count > *(volatile int32_t *)longest) atomicMax(longest, count);
-    }
+    if (lane == 0) steps[slice] = (most + (1 << lg_l) - 1) >> lg_l;
 }
 
+// columns and shares of a layout with ghost rows (a warp per slice)
 __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l, int64_t n_slices,
                                                            const int64_t *__restrict__ row_ptr,
                                                            const int32_t *__restrict__ col,
@@ -66,13 +63,7 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l,
         re = row_ptr[r + 1];
     }
     const int64_t at = off[slice], steps = off[slice + 1] - at;
-    if (lane == 0) {
-        // share b begins at the first slice at or behind place b / blocks of all: slice + 1 for the b in this slice's run
-        const int64_t total = off[n_slices] + slice_cost * n_slices, p0 = at + slice_cost * slice, p1 = p0 + steps + slice_cost;
-        if (slice == 0) share[0] = 0;
-        for (int64_t b = p0 * blocks / total; b <= blocks && total * b / blocks <= p1; b++)
-            if (total * b / blocks > p0) share[b] = slice + 1;
-    }
+    if (lane == 0) note_shares(slice, n_slices, off, share, blocks, slice_cost);
     for (int64_t k = 0; k < steps; k++) {
         const int64_t e = rs + (k << lg_l) + h;
         scol[(at + k) * 32 + lane] = e < re ? col[e] : -1;
@@ -105,54 +96,71 @@ static int sell_lanes_log2(int64_t n, int64_t nnz, int num_sms)
 }
 
 // Blocks get equal numbers of places where slices differ in length (order 6 on 200^2 nodes graded towards walls: 14.9 -> 11.3 us a
-// stage), but equal numbers of slices where none is a quarter longer than the mean: a few shorter ones at the box's edge
-// would otherwise make a block with one slice more than warps (193^2: 10.5 us a stage, 12.5 by places).
+// stage), but equal numbers of slices where no row is half as long again as the mean: a few shorter ones at the box's
+// edge would otherwise make a block with one slice more than warps (193^2: 10.5 us a stage, 12.5 by places).
 constexpr int64_t EVEN_SLICE_COST = 1 << 20;
 
-labfm_status build_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int64_t *parent)
+// The layout's shape: lanes per node and the places of the slices.  The longest row, which the search has counted, bounds
+// the places of ordinary sets, so that their number need not be waited for.
+static labfm_status shape_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int64_t *parent)
 {
     cudaStream_t s = ctx->stream;
-    const int64_t n = ctx->n;
-    const int64_t *rp = ctx->row_ptr.as<int64_t>();
-    L.valid = false;
+    const int64_t n = ctx->n, most_places = 2 * ctx->nnz + 64 * n;
+    L.shaped = L.valid = false;
     L.lg_l = sell_lanes_log2(n, ctx->nnz, ctx->num_sms);
-    unsigned blocks = 0;
-    int64_t slice_cost = SLICE_COST;
     while (true) {
         const int64_t per = 32 >> L.lg_l;
         L.n_slices = (n + per - 1) / per;
         LABFM_CUDA_TRY(ctx, L.steps.reserve(sizeof(int32_t) * L.n_slices));
-        LABFM_CUDA_TRY(ctx, L.off.reserve(sizeof(int64_t) * (L.n_slices + 2)));
-        int64_t *const end = L.off.as<int64_t>() + L.n_slices;  // behind the last slice, and then the steps of the longest one
-        LABFM_CUDA_TRY(ctx, cudaMemsetAsync(end + 1, 0, sizeof(int64_t), s));
-        blocks = (unsigned)((L.n_slices + SELL_THREADS / 32 - 1) / (SELL_THREADS / 32));
-        k_sell_steps<<<blocks, SELL_THREADS, 0, s>>>(n, L.lg_l, L.n_slices, rp, gmap, parent, L.steps.as<int32_t>(),
-                                                     reinterpret_cast<int32_t *>(end + 1));
+        LABFM_CUDA_TRY(ctx, L.off.reserve(sizeof(int64_t) * (L.n_slices + 1)));
+        k_sell_steps<<<(unsigned)((L.n_slices + SELL_THREADS / 32 - 1) / (SELL_THREADS / 32)), SELL_THREADS, 0, s>>>(
+            n, L.lg_l, L.n_slices, ctx->row_ptr.as<int64_t>(), gmap, parent, L.steps.as<int32_t>());
         LABFM_CUDA_TRY(ctx, cudaGetLastError());
         LABFM_CUDA_TRY(ctx, exclusive_scan_i32_to_i64(L.steps.as<int32_t>(), L.off.as<int64_t>(), L.n_slices, ctx->scan_tmp, s));
+        L.places = 32 * L.n_slices * ((ctx->longest + (1 << L.lg_l) - 1) >> L.lg_l);
+        if (L.places <= most_places) break;
         int64_t *total = (int64_t *)ctx->host_small;
-        LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(total, end, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        LABFM_CUDA_TRY(ctx, cudaMemcpyAsync(total, L.off.as<int64_t>() + L.n_slices, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         LABFM_CUDA_TRY(ctx, cudaStreamSynchronize(s));
-        L.places = 32 * total[0];
-        slice_cost = 4 * total[1] * L.n_slices <= 5 * total[0] ? EVEN_SLICE_COST : SLICE_COST;
+        L.places = 32 * *total;
         // a set whose neighbouring nodes differ too much in stencil size (a slice is as long as its largest one):
         // a warp per node, at most 31 places left empty each
-        if (L.lg_l == 5 || L.places <= 2 * ctx->nnz + 64 * n) break;
+        if (L.lg_l == 5 || L.places <= most_places) break;
         L.lg_l = 5;
     }
-    LABFM_CUDA_TRY(ctx, L.col.reserve(sizeof(int32_t) * (L.places > 0 ? L.places : 1)));
+    L.slice_cost = 2 * ctx->longest * n <= 3 * ctx->nnz ? EVEN_SLICE_COST : SLICE_COST;
     L.blocks = (int)std::min<int64_t>(L.n_slices, ctx->num_sms);
+    LABFM_CUDA_TRY(ctx, L.col.reserve(sizeof(int32_t) * (L.places > 0 ? L.places : 1)));
     LABFM_CUDA_TRY(ctx, L.share.reserve(sizeof(int64_t) * (L.blocks + 1)));
-    k_sell_cols<<<blocks, SELL_THREADS, 0, s>>>(n, L.lg_l, L.n_slices, rp, ctx->col.as<int32_t>(), gmap, parent,
-                                                L.off.as<int64_t>(), L.col.as<int32_t>(), L.share.as<int64_t>(), L.blocks, slice_cost);
+    L.shaped = true;
+    return LABFM_OK;
+}
+
+labfm_status build_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int64_t *parent)
+{
+    const labfm_status st = shape_sell(ctx, L, gmap, parent);
+    if (st != LABFM_OK) return st;
+    k_sell_cols<<<(unsigned)((L.n_slices + SELL_THREADS / 32 - 1) / (SELL_THREADS / 32)), SELL_THREADS, 0, ctx->stream>>>(
+        ctx->n, L.lg_l, L.n_slices, ctx->row_ptr.as<int64_t>(), ctx->col.as<int32_t>(), gmap, parent, L.off.as<int64_t>(),
+        L.col.as<int32_t>(), L.share.as<int64_t>(), L.blocks, L.slice_cost);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     L.valid = true;
     return LABFM_OK;
 }
 
+labfm_status ensure_sell_shape(labfm_ctx *ctx)
+{
+    return ctx->sell.shaped ? LABFM_OK : shape_sell(ctx, ctx->sell, nullptr, nullptr);
+}
+
+struct ColumnsOnly {};
+
 labfm_status ensure_sell(labfm_ctx *ctx)
 {
-    return ctx->sell.valid ? LABFM_OK : build_sell(ctx, ctx->sell, nullptr, nullptr);
+    const labfm_status st = ensure_sell_shape(ctx);
+    if (st != LABFM_OK || ctx->sell.valid) return st;
+    LABFM_CUDA_TRY(ctx, (launch_sell_fill<int32_t, 0>(ctx, ctx->sell, (int32_t *)nullptr, ColumnsOnly{})));
+    return LABFM_OK;
 }
 
 }  // namespace labfm

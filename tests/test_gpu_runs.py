@@ -123,3 +123,31 @@ def test_stage_time_of_just_more_slices_than_warps():
         return best
 
     assert stage_us(289) <= 1.5 * stage_us(257)
+
+
+@pytest.mark.parametrize("kind", ["step", "burgers"])
+def test_the_first_step_after_a_search_does_not_wait(kind):
+    """On a context that has done the same before (its buffers are there), with 50 ms of other work on the stream."""
+    import time
+
+    import torch
+
+    m = 100
+    at = np.arange(m * m)
+    xy, h = np.stack([(at % m + 0.5) / m, (at // m + 0.5) / m], 1), np.full(m * m, 1.999 / m)
+    X, H = torch.from_numpy(xy).to("cuda"), torch.from_numpy(h).to("cuda")
+    L = _context(xy, h, ("dx", "dy", "lap"), "f64")[0]
+    C = np.stack([S.op_c_vector(o, 2) for o in ("dx", "dy", "lap")])
+    u, v = (torch.from_numpy(np.random.default_rng(i).random(m * m)).to("cuda") for i in (0, 1))
+    run = (lambda: L.step([0.0] * 3, u, 1e-9, 1)) if kind == "step" else (lambda: L.step_burgers([0.0] * 3, u, v, 1e-9, 1))
+    for _ in range(3):
+        L.build_neighbours(X, H, False)
+        L.build_weights(C, uniform_order=2)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(100000000)
+        t = time.perf_counter()
+        run()
+        t = time.perf_counter() - t
+        torch.cuda.synchronize()
+    assert t < 0.02
+    L.close()
