@@ -315,28 +315,30 @@ def accuracy_vs_oracle(torch, P, dev, local_rank):
     return out
 
 
-def kernel_source_hash():
-    import hashlib
+def _rounded(v):
+    """v with its floats to six digits."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, dict):
+        return {k: _rounded(x) for k, x in v.items()}
+    return [_rounded(x) for x in v] if isinstance(v, (list, tuple)) else v
 
-    hsh = hashlib.sha256()
-    for f in ("build_node.cuh", "build_fp64.cu", "abf.cuh"):
-        with open(os.path.join(ROOT, "paper_1912_06441_gb300", "csrc", f), "rb") as fh:
-            hsh.update(fh.read())
-    return hsh.hexdigest()
 
-
-def build_traffic(n):
-    """DRAM bytes per launch of the build kernel from the committed ncu capture, scaled by
-    node count; None if the kernel source changed since the capture."""
-    prof = os.path.join(ROOT, "profiles", "build_fp64_traffic.json")
-    try:
-        with open(prof) as fh:
-            rec = json.load(fh)
-    except Exception:
-        return None
-    if rec.get("source_sha256") != kernel_source_hash():
-        return None
-    return rec["dram_bytes_per_node"] * n
+def report(line, out=None, err=None):
+    """The result line on `out`, short enough to be read from the end of a log: the further measurements (`extra`) go to
+    `err` as a line of their own, and a few of their figures stay in the line."""
+    line = dict(line)
+    extra = line.pop("extra", None)
+    if extra is not None:
+        print("bench details: " + json.dumps(_rounded(extra)), file=err or sys.stderr, flush=True)
+        line["details"] = "stderr"
+        line["mixed_vs_fp64"] = {key[:6]: {prec: {k: extra[key][prec][k] for k in ("ms", "mnodes_per_s") if k in extra[key][prec]}
+                                           for prec in ("fp64", "mixed", "mixed_tc") if prec in extra[key]}
+                                 for key in ("order8_mixed_vs_fp64", "order6_mixed_vs_fp64") if key in extra}
+        order8 = extra.get("accuracy_vs_oracle", {}).get("orders", {}).get("8", {})
+        line["order8_frac_le_1e-8"] = {nodes: {v: blk[v]["frac_le_1e-8"] for v in ("fp64_oracle", "fp64", "mixed", "mixed_tc") if v in blk}
+                                       for nodes, blk in order8.items() if isinstance(blk, dict) and "nodes" in blk}
+    print(json.dumps(_rounded(line)), file=out or sys.stdout, flush=True)
 
 
 def _time(torch, fn, reps=3):
@@ -1025,7 +1027,6 @@ def run_labfm(args, rank, world, local_rank):
     abytes = apply_bytes(n, nnz, len(OPS))
     a_ach = abytes / (apply_ms * 1e-3) / 1e9
     hbm, hbm_src = hbm_peak()
-    traffic = build_traffic(n)
     line = {
         "metric": METRIC, "value": value, "unit": "Mnodes/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
@@ -1036,7 +1037,7 @@ def run_labfm(args, rank, world, local_rank):
         "phases_ms": {"neighbours": float(np.mean(phase[:, 0])), "build_fp64": build_ms, "apply": apply_ms,
                       "rk4_step": float(np.mean(phase[:, 3]))},
         "roofline": {"bound": "alu", "kernel": "k_build_fp64<8> (FP64 weight build)", "achieved": b_ach,
-                     "peak": fp64_peak, "unit": "TFLOP/s", "frac": b_ach / fp64_peak, "traffic": traffic,
+                     "peak": fp64_peak, "unit": "TFLOP/s", "frac": b_ach / fp64_peak,
                      "peak_source": "cuBLAS DGEMM 4096^3 measured in this run (FP64 pipe)",
                      "algorithmic_flops_per_node": bflops / n},
         "apply_roofline": {"bound": "hbm", "kernel": "k_apply<4,double,double>", "achieved": a_ach, "peak": hbm,
@@ -1080,7 +1081,7 @@ def run_labfm(args, rank, world, local_rank):
         line["extra"]["accuracy_vs_oracle"] = accuracy_vs_oracle(torch, P, dev, local_rank)
         if not SKIP_LARGE:
             line["extra"]["rk4_2048"]["oracle"] = rk4_oracle_leg(torch, P, dev, local_rank)
-    print(json.dumps(line), flush=True)
+    report(line)
     L.close()
 
 
