@@ -320,7 +320,8 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_rk4_run(int64_t n, SellView 
     };
     share_out(S, s0, s1);
     if (bar.stopped()) return;
-    SliceSweep<4, 1, 1, 1, VT> sweep;
+    SliceSweep<4, 1, 1, 1, true, VT> sweep;
+    sweep.place(n, S);
     sweep.preload(n, S, wc);
     for (int64_t it = 0; it < 4 * nsteps; it++) {
         const int stage = (int)(it & 3);
@@ -820,7 +821,7 @@ __global__ void __launch_bounds__(RUN_THREADS, 1) k_burgers_run(int64_t n, SellV
     };
     share_out(S, s0, s1);
     if (bar.stopped()) return;
-    SliceSweep<2, 3, 2, 2, VT> sweep;
+    SliceSweep<2, 3, 2, 2, false, VT> sweep;
     sweep.preload(n, S, wb);
     for (int64_t it = 0; it < 4 * nsteps; it++) {
         const int stage = (int)(it & 3);

@@ -37,7 +37,8 @@ struct Sell {
     int64_t n_slices = 0;
     int64_t places = 0;    // entries with the empty places, at most
     int blocks = 0;        // shares of the slices, one per block of a run
-    int64_t slice_cost = 0;  // what a slice counts besides its steps in the shares
+    bool even = false;     // shares of equal numbers of slices
+    bool whole = false;    // ... none of which can be worth a cut
     DevBuf off, col, steps, share;
     void release()
     {
@@ -189,9 +190,12 @@ struct SellView {
     int64_t n_slices;
     const int64_t *off;
     const int32_t *col;
-    const int64_t *share;  // [blocks + 1]: the slices of share b are share[b] .. share[b + 1] - 1
+    const int64_t *share;  // [blocks + 1]: the slices of share b are share[b] .. share[b + 1] - 1; null: equal numbers,
+    int each, more;        // `each`, and `more` in all besides, spread evenly
+    unsigned recip;        // 2^32 / blocks, rounded up
     int blocks;
     int lg_l;
+    bool whole;            // no block can have a slice to cut
 };
 
 // The scale on which sweeps are shared out: slice s takes [slice_at(s), slice_at(s + 1)), a place for each of its steps and
@@ -202,6 +206,7 @@ constexpr int SLICE_COST = 4;
 struct SellLane {
     int64_t i = -1, at = 0;
     int steps = 0, h;
+    SellLane() = default;
     __device__ SellLane(int64_t slice, int lane, int64_t n, const SellView &S)
     {
         h = lane & ((1 << S.lg_l) - 1);
@@ -348,8 +353,19 @@ __device__ __forceinline__ int64_t slice_at(const SellView &S, int64_t s) { retu
 // This block's slices [first, last): its share, or where the grid has fewer blocks than shares, several
 __device__ __forceinline__ void block_share(const SellView &S, int64_t &first, int64_t &last)
 {
-    first = S.share[(int64_t)blockIdx.x * S.blocks / gridDim.x];
-    last = S.share[(int64_t)(blockIdx.x + 1) * S.blocks / gridDim.x];
+    int b0 = blockIdx.x, b1 = blockIdx.x + 1;
+    if (gridDim.x != S.blocks) {
+        b0 = b0 * S.blocks / gridDim.x;
+        b1 = b1 * S.blocks / gridDim.x;
+    }
+    if (S.share) {
+        first = S.share[b0];
+        last = S.share[b1];
+    } else {
+        // (b more / blocks, by the reciprocal: exact up to some 250 blocks)
+        first = (int64_t)S.each * b0 + __umulhi((unsigned)(S.more * b0), S.recip);
+        last = (int64_t)S.each * b1 + __umulhi((unsigned)(S.more * b1), S.recip);
+    }
 }
 
 // A warp's part of its block's slices: every RUN_WARPS-th slice, or where that gives some warp CUT_COST places more than an
@@ -379,15 +395,23 @@ __device__ __forceinline__ void share_out(const SellView &S, int64_t s0, int64_t
 {
     __shared__ int s_first[RUN_WARPS + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto whole_slices = [&] {
+        const int64_t t = s0 + warp;
+        if (lane == 0)
+            warp_share() = t < s1 ? WarpShare{S.off[t], (int)(S.off[t + 1] - S.off[t]), (int)t, (int)s1, RUN_WARPS, false, false, -1, 0}
+                                  : WarpShare{0, 0, (int)t, (int)t, RUN_WARPS, false, false, -1, 0};
+    };
+    if (S.whole) {  // (a run of two steps on 64^2 nodes would take 7 % longer for finding that out)
+        whole_slices();
+        __syncthreads();
+        return;
+    }
     const int64_t base = slice_at(S, s0), total = slice_at(S, s1) - base;
     int64_t whole = 0;  // places of every RUN_WARPS-th slice
     for (int64_t t = s0 + warp + RUN_WARPS * lane; t < s1; t += RUN_WARPS * 32) whole += slice_at(S, t + 1) - slice_at(S, t);
     for (int o = 16; o > 0; o >>= 1) whole += __shfl_xor_sync(0xffffffffu, whole, o);
     if (!__syncthreads_or(whole > total / RUN_WARPS + CUT_COST)) {
-        const int64_t t = s0 + warp;
-        if (lane == 0)
-            warp_share() = t < s1 ? WarpShare{S.off[t], (int)(S.off[t + 1] - S.off[t]), (int)t, (int)s1, RUN_WARPS, false, false, -1, 0}
-                                  : WarpShare{0, 0, (int)t, (int)t, RUN_WARPS, false, false, -1, 0};
+        whole_slices();
         __syncwarp();
         return;
     }
@@ -438,9 +462,15 @@ __device__ __forceinline__ double (&left_parts())[RUN_WARPS][NS][32]
 // gather and add as in SlicePipe (add with those values), part(values, sums) the lane's sums, and where the warp
 // updates the slice finish(lane, values, sums) with the parts of all warps.  Every thread of the block takes part, after
 // share_out; a block barrier has to follow before the next run.
-template <int U, int NW, int NX, int NS, class VT>
+// KEEP: the first piece is kept in registers, found by place() once or, where registers are short, before every preload; else it
+// is read again from the warp's share.  (Burgers runs are 3 to 4 % faster without, 161^2: 68.4 us a step against 70.4; heat
+// and solves up to 4 % with, 41^2: 11.9 us a step against 12.5.)
+template <int U, int NW, int NX, int NS, bool KEEP, class VT>
 struct SliceSweep {
     SlicePipe<U, NW, NX, VT> pipe;
+    SellLane kept_at;
+    int kept_slice;
+    bool kept_mine, kept_last;  // this warp updates it; it has no further one
 
     // the first piece (of none: no node and no step)
     static __device__ __forceinline__ SellLane begin_at(int64_t n, const SellView &S)
@@ -449,10 +479,20 @@ struct SliceSweep {
         const bool any = W.head || W.first < W.last;
         return SellLane(any ? W.first - W.head : S.n_slices, W.from, W.steps, threadIdx.x & 31, n, S);
     }
+    __device__ __forceinline__ void place(int64_t n, const SellView &S)
+    {
+        static_assert(KEEP, "nothing is kept");
+        const WarpShare &W = warp_share();
+        kept_slice = W.first - W.head;
+        kept_mine = kept_slice >= W.first && kept_slice < W.last;
+        kept_last = kept_slice + W.stride >= W.last;
+        kept_at = begin_at(n, S);
+    }
     // the first loads of the next run
     __device__ __forceinline__ void preload(int64_t n, const SellView &S, const VT *__restrict__ wc)
     {
-        pipe.preload(begin_at(n, S), threadIdx.x & 31, S, wc);
+        if constexpr (KEEP) pipe.preload(kept_at, threadIdx.x & 31, S, wc);
+        else pipe.preload(begin_at(n, S), threadIdx.x & 31, S, wc);
     }
     template <class Begin, class Gather, class Add, class Part, class Finish>
     __device__ __forceinline__ void run(int64_t n, const SellView &S, const VT *__restrict__ wc, Begin begin, Gather gather,
@@ -461,10 +501,23 @@ struct SliceSweep {
         double(&s_part)[RUN_WARPS][NS][32] = left_parts<NS>();
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         const WarpShare &W = warp_share();
-        SellLane l = begin_at(n, S);
-        int slice = W.first - W.head;
+        SellLane l;
+        int slice;
+        bool mine, last;
+        if constexpr (KEEP) {
+            l = kept_at;
+            slice = kept_slice;
+            mine = kept_mine;
+            last = kept_last;
+        } else {
+            l = begin_at(n, S);
+            slice = W.first - W.head;
+        }
         while (true) {  // a warp without a piece goes through once, for the barrier
-            const bool mine = slice >= W.first && slice < W.last, last = slice + W.stride >= W.last;
+            if constexpr (!KEEP) {
+                mine = slice >= W.first && slice < W.last;
+                last = slice + W.stride >= W.last;
+            }
             auto v = begin(l, mine);
             double p[NS];
             pipe.run(l, lane, S, wc, gather, [&](int q, const double(&x)[NX], const VT(&w)[NW]) { add(v, q, x, w); });
@@ -482,6 +535,10 @@ struct SliceSweep {
             if (mine) finish(l, v, p);
             if (last) break;
             slice += W.stride;
+            if constexpr (KEEP) {
+                mine = true;
+                last = slice + W.stride >= W.last;
+            }
             l = SellLane(slice, lane, n, S);
             if (slice + 1 == W.last && W.open >= 0) l.steps = W.open;
             pipe.preload(l, lane, S, wc);
@@ -545,7 +602,10 @@ inline labfm_status run_gave_up(labfm_ctx *ctx)
 }
 inline SellView sell_view(const Sell &L)
 {
-    return SellView{L.n_slices, L.off.as<int64_t>(), L.col.as<int32_t>(), L.share.as<int64_t>(), L.blocks, L.lg_l};
+    const int each = (int)(L.n_slices / L.blocks), more = (int)(L.n_slices % L.blocks);
+    const unsigned recip = (unsigned)(((1ull << 32) + L.blocks - 1) / L.blocks);  // (one block: 0, and more = 0)
+    return SellView{L.n_slices, L.off.as<int64_t>(), L.col.as<int32_t>(), L.even ? nullptr : L.share.as<int64_t>(), each, more,
+                    recip, L.blocks, L.lg_l, L.whole};
 }
 labfm_status ensure_sell_shape(labfm_ctx *ctx);  // ctx->sell of the current stencils, col and share still to come (sell_fill.cuh)
 labfm_status ensure_sell(labfm_ctx *ctx);        // all of it

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l,
                                                            const int32_t *__restrict__ gmap,
                                                            const int64_t *__restrict__ parent,
                                                            const int64_t *__restrict__ off, int32_t *__restrict__ scol,
-                                                           int64_t *__restrict__ share, int blocks, int64_t slice_cost)
+                                                           int64_t *__restrict__ share, int blocks)
 {
     const int lane = threadIdx.x & 31, h = lane & ((1 << lg_l) - 1);
     const int64_t slice = (int64_t)blockIdx.x * (SELL_THREADS / 32) + (threadIdx.x >> 5);
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l,
         re = row_ptr[r + 1];
     }
     const int64_t at = off[slice], steps = off[slice + 1] - at;
-    if (lane == 0) note_shares(slice, n_slices, off, share, blocks, slice_cost);
+    if (lane == 0 && share) note_shares(slice, n_slices, off, share, blocks);
     for (int64_t k = 0; k < steps; k++) {
         const int64_t e = rs + (k << lg_l) + h;
         scol[(at + k) * 32 + lane] = e < re ? col[e] : -1;
@@ -72,22 +72,24 @@ __global__ void __launch_bounds__(SELL_THREADS) k_sell_cols(int64_t n, int lg_l,
 
 }  // namespace
 
-// Lanes per node, as the power of two with the least cost of a sweep of the busiest block: 16 cycles per FP64 instruction,
-// two per entry of a lane, about four for the node and two per combining step; and 90 cycles per place for the loads of
-// the longest warp (see share_out: whole slices, or cut ones where those are more uneven).  One lane for large
-// sets, two at 129^2 and 161^2 nodes, eight at 41^2.  Over 45 sizes of heat, Burgers, solver and order-8 runs between 41^2 and 900^2
-// the choice is within 1 % of the best lane count on average and 9 % at worst.
+// Lanes per node, as the power of two with the least cost of a sweep of the busiest block.  It is the larger of two, in cycles:
+// 16 per FP64 instruction, two per entry of a lane, about four for the node and two per combining step; and 210 per
+// place of the longest warp for its loads (see share_out: whole slices, or cut ones where those are more uneven); of
+// the same size they add up, about as the fourth root of the sum of fourth powers.  One lane for large sets, two at 129^2 and
+// 161^2 nodes, sixteen at 41^2.  Over 45 sizes of heat, Burgers, solver and order-8 runs between 41^2 and 900^2 the
+// choice is within 0.3 % of the best lane count on average and 4 % at worst.
 static int sell_lanes_log2(int64_t n, int64_t nnz, int num_sms)
 {
     const int64_t deg = n > 0 ? (nnz + n - 1) / n : 0;
     int best = 0;
-    int64_t least = INT64_MAX;
+    double least = 0.0;
     for (int lg = 0; lg <= 4; lg++) {
         const int64_t slices = ((n << lg) + 31) / 32, most = (slices + num_sms - 1) / num_sms;
         const int64_t steps = (deg + (1 << lg) - 1) >> lg, whole = (most + RUN_WARPS - 1) / RUN_WARPS * (steps + SLICE_COST);
         const int64_t cut = most * (steps + SLICE_COST) / RUN_WARPS + CUT_COST;
-        const int64_t cost = 16 * most * (2 * steps + 2 * lg + 4) + 90 * std::min(whole, cut);
-        if (cost < least) {
+        const double issue = 16.0 * (double)(most * (2 * steps + 2 * lg + 4)), loads = 210.0 * (double)std::min(whole, cut);
+        const double cost = issue * issue * issue * issue + loads * loads * loads * loads;
+        if (lg == 0 || cost < least) {
             least = cost;
             best = lg;
         }
@@ -98,7 +100,7 @@ static int sell_lanes_log2(int64_t n, int64_t nnz, int num_sms)
 // Blocks get equal numbers of places where slices differ in length (order 6 on 200^2 nodes graded towards walls: 14.9 -> 11.3 us a
 // stage), but equal numbers of slices where no row is half as long again as the mean: a few shorter ones at the box's
 // edge would otherwise make a block with one slice more than warps (193^2: 10.5 us a stage, 12.5 by places).
-constexpr int64_t EVEN_SLICE_COST = 1 << 20;
+static bool even_rows(const labfm_ctx *ctx) { return 2 * ctx->longest * ctx->n <= 3 * ctx->nnz; }
 
 // The layout's shape: lanes per node and the places of the slices.  The longest row, which the search has counted, bounds
 // the places of ordinary sets, so that their number need not be waited for.
@@ -128,8 +130,10 @@ static labfm_status shape_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, con
         if (L.lg_l == 5 || L.places <= most_places) break;
         L.lg_l = 5;
     }
-    L.slice_cost = 2 * ctx->longest * n <= 3 * ctx->nnz ? EVEN_SLICE_COST : SLICE_COST;
     L.blocks = (int)std::min<int64_t>(L.n_slices, ctx->num_sms);
+    L.even = even_rows(ctx) && L.blocks <= 250;
+    const int64_t rounds = ((L.n_slices + L.blocks - 1) / L.blocks + RUN_WARPS - 1) / RUN_WARPS;
+    L.whole = L.even && rounds * (((ctx->longest + (1 << L.lg_l) - 1) >> L.lg_l) + SLICE_COST) <= CUT_COST;
     LABFM_CUDA_TRY(ctx, L.col.reserve(sizeof(int32_t) * (L.places > 0 ? L.places : 1)));
     LABFM_CUDA_TRY(ctx, L.share.reserve(sizeof(int64_t) * (L.blocks + 1)));
     L.shaped = true;
@@ -142,7 +146,7 @@ labfm_status build_sell(labfm_ctx *ctx, Sell &L, const int32_t *gmap, const int6
     if (st != LABFM_OK) return st;
     k_sell_cols<<<(unsigned)((L.n_slices + SELL_THREADS / 32 - 1) / (SELL_THREADS / 32)), SELL_THREADS, 0, ctx->stream>>>(
         ctx->n, L.lg_l, L.n_slices, ctx->row_ptr.as<int64_t>(), ctx->col.as<int32_t>(), gmap, parent, L.off.as<int64_t>(),
-        L.col.as<int32_t>(), L.share.as<int64_t>(), L.blocks, L.slice_cost);
+        L.col.as<int32_t>(), L.even ? nullptr : L.share.as<int64_t>(), L.blocks);
     LABFM_CUDA_TRY(ctx, cudaGetLastError());
     L.valid = true;
     return LABFM_OK;

@@ -22,17 +22,15 @@ struct SellFill {
     const int64_t *off, *row_ptr;
     const int32_t *col;
     int32_t *scol;   // null: the columns are there
-    int64_t *share;
+    int64_t *share;  // null: equal numbers of slices
     int blocks;
-    int64_t slice_cost;
 };
 
 // Where share b of the blocks begins: at the first slice at or behind place b / blocks of all (slice s: those that are s + 1).
-__device__ __forceinline__ void note_shares(int64_t slice, int64_t n_slices, const int64_t *off, int64_t *share, int blocks,
-                                            int64_t slice_cost)
+__device__ __forceinline__ void note_shares(int64_t slice, int64_t n_slices, const int64_t *off, int64_t *share, int blocks)
 {
-    const int64_t total = off[n_slices] + slice_cost * n_slices;
-    const int64_t p0 = off[slice] + slice_cost * slice, p1 = off[slice + 1] + slice_cost * (slice + 1);
+    const int64_t total = off[n_slices] + SLICE_COST * n_slices;
+    const int64_t p0 = off[slice] + SLICE_COST * slice, p1 = off[slice + 1] + SLICE_COST * (slice + 1);
     if (slice == 0) share[0] = 0;
     for (int64_t b = p0 * blocks / total; b <= blocks && total * b / blocks <= p1; b++)
         if (total * b / blocks > p0) share[b] = slice + 1;
@@ -69,7 +67,7 @@ __global__ void __launch_bounds__(FILL_THREADS) k_sell_fill(const __grid_constan
         s_len[lane] = len;
         s_at[lane] = end - room;
         if (lane == 31) s_at[32] = end;
-        if (lane == 0 && F.scol) note_shares(slice, F.n_slices, F.off, F.share, F.blocks, F.slice_cost);
+        if (lane == 0 && F.share) note_shares(slice, F.n_slices, F.off, F.share, F.blocks);
     }
     const int64_t at = F.off[slice], steps = F.off[slice + 1] - at;
     __syncthreads();
@@ -115,7 +113,7 @@ cudaError_t launch_sell_fill(labfm_ctx *ctx, Sell &L, VT *out, Fn fn)
     const int64_t want = (int64_t)(32 >> L.lg_l) * (ctx->longest | 1) + 32;
     const int cap = (int)(want * (int64_t)per_entry <= FILL_SMEM ? want : FILL_SMEM / per_entry) / 2 * 2;
     const SellFill F{ctx->n, L.n_slices, L.lg_l, cap, L.off.as<int64_t>(), ctx->row_ptr.as<int64_t>(), ctx->col.as<int32_t>(),
-                     cols ? L.col.as<int32_t>() : nullptr, L.share.as<int64_t>(), L.blocks, L.slice_cost};
+                     cols ? L.col.as<int32_t>() : nullptr, cols && !L.even ? L.share.as<int64_t>() : nullptr, L.blocks};
     cudaError_t e = cudaSuccess;
     if (cap * per_entry > 47 * 1024)
         e = cudaFuncSetAttribute(k_sell_fill<VT, NV, Fn>, cudaFuncAttributeMaxDynamicSharedMemorySize, FILL_SMEM);

@@ -196,12 +196,13 @@ struct SolveBlock {
     GridBarrier bar;
     int n0, n1;  // rows
     int lane, warp;
-    SliceSweep<4, 1, 1, 1, double> sweep;
+    SliceSweep<4, 1, 1, 1, true, double> sweep;
 
     __device__ SolveBlock(const SolveArgs &args, int64_t s0, int64_t s1)
         : A(args), bar{args.sync}, n0((int)(s0 * (32 >> args.S.lg_l))), n1((int)min(args.n, s1 * (32 >> args.S.lg_l))),
           lane(threadIdx.x & 31), warp(threadIdx.x >> 5)
     {
+        sweep.place(A.n, A.S);
         sweep.preload(A.n, A.S, A.wd);
     }
 
@@ -248,6 +249,7 @@ struct SolveBlock {
                 for (int o = (1 << A.S.lg_l) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
                 if (v.row) fn(l.i, v.fixed ? v.xi : DIFFERENCES ? acc : fma(v.ai, v.xi, acc), v.oi);
             });
+        sweep.place(A.n, A.S);
         sweep.preload(A.n, A.S, A.wd);
     }
 
