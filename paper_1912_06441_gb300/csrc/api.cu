@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const Tin *__restri
                                                              unsigned long long *__restrict__ largest)
 {
     __shared__ int64_t sh[32];
+    __shared__ unsigned sh_max[32];
     int64_t before = 0;  // the sum of all earlier blocks' runs
     if (sums && scanned) {
         before = sums[blockIdx.x];
@@ -110,6 +111,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const Tin *__restri
         if (lane >= o) v += w;
     }
     if (lane == 31) sh[warp] = v;
+    if (largest) sh_max[warp] = __reduce_max_sync(0xffffffffu, (unsigned)max(a, b));
     __syncthreads();
     int64_t ws = lane < warp ? sh[lane] : 0;
     for (int o = 16; o > 0; o >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, o);
@@ -117,9 +119,9 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(const Tin *__restri
     if (g < n) out[g] = at;
     if (g + 1 < n) out[g + 1] = at + a;
     if (g < n && g + 2 >= n) out[n] = at + a + b;  // the thread of the last element
-    if (largest) {
-        const unsigned most = __reduce_max_sync(0xffffffffu, (unsigned)max(a, b));
-        if (lane == 0 && most > *(volatile unsigned long long *)largest) atomicMax(largest, (unsigned long long)most);
+    if (largest && warp == 0) {
+        const unsigned most = __reduce_max_sync(0xffffffffu, sh_max[lane]);
+        if (lane == 0) atomicMax(largest, (unsigned long long)most);
     }
 }
 
