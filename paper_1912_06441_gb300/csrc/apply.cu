@@ -731,7 +731,7 @@ struct BurgersWeights {
 //   F_u = sum_j (su_j - su_i) c_ji,   F_v = sum_j (sv_j - sv_i) c_ji
 // (0 on frozen nodes): six FP64 instructions per entry and two sums to combine, where the sums with w^0, w^1 and wl
 // apart take eight and six; the FP64 pipe bounds the stage on sets that fit the L2 cache.  Then the stage updates
-// of k_rk4_stage for both fields; acc and nxt hold u in [0, n) and v in [n, 2n).  Sums in double unless fields and
+// of k_rk4_stage_csr for both fields; acc and nxt hold u in [0, n) and v in [n, 2n).  Sums in double unless fields and
 // weights are both float.
 template <class WT, int UNR>
 __global__ void __launch_bounds__(APPLY_THREADS) k_burgers_stage_csr(int64_t n, const int64_t *__restrict__ row_ptr,

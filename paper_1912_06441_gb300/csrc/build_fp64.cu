@@ -44,7 +44,7 @@ bool chain_rule(int rbf) { return (rbf & LABFM_ABF_DW0_ONLY) == 0; }
 
 cudaError_t launch_fp64_order(int k, int G, const BuildArgs &a, int num_sms, cudaStream_t s)
 {
-    return (k >= MOMENT_MIN_ORDER && chain_rule(a.rbf) ? launch_order_chain : launch_order_dw0)(k, G, a, num_sms, s);
+    return (k >= FORM_MIN_ORDER && chain_rule(a.rbf) ? launch_order_chain : launch_order_dw0)(k, G, a, num_sms, s);
 }
 
 }  // namespace
@@ -150,7 +150,10 @@ labfm_status run_build(labfm_ctx *ctx, const int8_t *order, int uniform_order, i
     // Orders that the FP64 kernel builds: all of them for LABFM_PREC_FP64; for the mixed builds the
     // orders below MIXED_MIN_ORDER, whose p x p systems (p <= 14) are small and well conditioned:
     // there the cost is latency, which the grouped FP64 kernel hides better than the four-kernel
-    // mixed pipeline, and FP64 arithmetic is accurate to the floor.
+    // mixed pipeline, and FP64 arithmetic is accurate to the floor.  (From moments the FP64 kernel is the faster one at
+    // the orders above too, 23.5 against 29.6 and 30.7 ms at order 6, 56.2 against 69.7 and 63.3 at order 8, 512^2 nodes;
+    // there the mixed builds stay for the accuracy that their refinement asks for: errors at order 8 of 1e-12 against
+    // 2e-9 in the median.)
     auto fp64_route = [&](int k) { return !mixed || k < MIXED_MIN_ORDER; };
 
     // Group size of the FP64 kernel per order: timed once per (order, mean stencil size, n_ops)

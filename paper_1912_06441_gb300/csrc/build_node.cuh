@@ -8,13 +8,13 @@
 // barrier), where the p x p system is small and a whole CTA would spend its time in barrier
 // latency with most threads idle.  G per order is chosen by timing (build autotuner).
 //
-// Orders 1-3, and 4 with the full chain rule, form M from X and W themselves.  Orders 4-8 use two facts about the ABFs of Sec. 3.2:
+// Orders 1-3, and 4 with the full chain rule, form M from X and W themselves.  The others use two facts about the ABFs of Sec. 3.2:
 //
 // (1) The weights depend only on the space that the ABFs span: w_j = W_j . Psi with sum_j X_j w_j = C is
 //     the same for every basis of that space.  The elements of degree n whose ABF is dW0/dr d^alpha|r|
 //     are W0'(q) q^(1-2n) P_alpha(x, y) with the n + 1 independent homogeneous polynomials P_alpha of degree
 //     n, so they span g_n x^a y^b, a + b = n, g_n = W0' q^(1-2n).  (With the full chain rule the elements of
-//     degree 2 and 3 span five other functions times harmonics instead, see LowFam.)
+//     degree 2 and 3 span four other radial functions times harmonics instead, see NLOWFAM.)
 // (2) In that basis M_(a',b'),(a,b) = sum_j g_n x^(a+a') y^(b+b') = T_n(a + a', b + b'): its entries are moments,
 //     and T_n(s, t) = T_(n+1)(s + 2, t) + T_(n+1)(s, t + 2), because g_n = g_(n+1) (x^2 + y^2).  So T_K at degrees
 //     K + 1 .. 2K and the highest degree n + K of each other T_n are all the sums over neighbours there are:
@@ -25,7 +25,7 @@
 // formed.  The FP64 pipe bounds the build (two lanes per SM and clock on GB300), and this takes its work at
 // order 8 from 181 k to about 80 k multiply-adds per node.  The basis g_n x^a y^b is also better conditioned
 // than the ABFs (median condition number at order 8, +-0.3 s noise: 1e10 against 3e12), so the weights come out
-// closer to the exact ones (order 8: about ten times).  Orders 1-3 keep X and W: their systems are so small that
+// closer to the exact ones (order 8: about ten times).  The orders below keep X and W: their systems are so small that
 // nothing is gained, and the rounding of the recurrence shows there (5e-16 against 4e-16).
 //
 // Per-node orders (walls and variable resolution, Sec. 4.1) run in one persistent launch over
@@ -77,7 +77,7 @@ struct OrderItems {
 };
 
 constexpr int BUILD_THREADS = 256;
-constexpr int MOMENT_MIN_ORDER = 4;  // orders whose kernels differ by the form of the ABFs
+constexpr int FORM_MIN_ORDER = 4;  // from here on the kernels differ by the form of the ABFs (order 4 is built from moments in one of them)
 
 // Orders built from moments: from 5 up, and order 4 where every ABF is dW0/dr d^alpha|r| (256^2 nodes: 1.55 ms against
 // 2.08 from X and W; with the full chain rule, where half of the 14 elements are further functions, 2.29 against 2.13).
@@ -404,7 +404,7 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
     using M = Mom<K, CH>;
     constexpr int P = C::P, NB = C::NB, LDA = C::LDA;
     double *Am = smem;  // [P][LDA]  augmented [M | Chat], over the staged rows
-    // moments: rows [NB][LD], kept values [NB][LP], T; orders 1-3: Xs, Ws [NB][LDX]
+    // moments: rows [NB][LD], kept values [NB][LP], T; from X and W: Xs, Ws [NB][LDX]
     double *rows = smem;
     double *keep = rows + NB * M::LD;
     double *T = keep + NB * M::LP;
@@ -786,7 +786,7 @@ __device__ __forceinline__ void build_node(const BuildArgs &A, int64_t i, double
         }
         gsync<G>(bar);
 
-        // weights: w_j^d = W0' r sum Phi_ab u^a v^b (+ the chain-rule functions), or W_j . Psi^d at orders 1-3
+        // weights: w_j^d = W0' r sum Phi_ab u^a v^b (+ the chain-rule functions), or W_j . Psi^d
         for (int ch = 0; ch < nchunks; ch++) {
             const int j0 = ch * NB;
             const int nj = min(NB, ni - j0);
