@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(FILL_THREADS) k_sell_fill(const __grid_constan
             rs = F.row_ptr[i];
             len = (int)(F.row_ptr[i + 1] - rs);
         }
-        const int room = len | 1;  // odd: rows of equal length begin on different banks
+        const int room = min(len | 1, 1 << 24);  // odd: rows of equal length begin on different banks (bounded: 32 of them fit an int)
         int end = room;
         for (int o = 1; o < 32; o <<= 1) {
             const int below = __shfl_up_sync(0xffffffffu, end, o);
